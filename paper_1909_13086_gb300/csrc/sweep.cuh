@@ -322,6 +322,42 @@ __device__ __forceinline__ void emit(real p[9], real a, real B0, real B1x, real 
     p[8] = a * p[8] + (e68 - t6);
 }
 
+// ---- f and g as one pair ----
+// The two collisions are the same block operator on different coefficients, so
+// with flow on (FP32 arithmetic) they run as pairs (x: f, y: g) on sm_100's
+// packed FP32 instructions: one issue slot for both halves, each half rounded
+// as its scalar instruction would be.  The sweeps are bound by instruction
+// issue (16-bit storage) or by latency (FP32), not by the FP32 pipe.
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, both(-1.0f), a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// emit on a pair (FP32: the rest weight's share as the remainder).
+__device__ __forceinline__ void emit2(float2 p[9], float2 a, float2 B0, float2 B1x, float2 B1y, float2 B2xx,
+                                      float2 B2xy, float2 B2yy) {
+    const float2 third = both(1.0f / 3.0f), nthird = both(-(1.0f / 3.0f)), nsixth = both(-(1.0f / 6.0f));
+    const float2 twelfth = both(1.0f / 12.0f), ntwelfth = both(-(1.0f / 12.0f));
+    const float2 w1 = both(1.0f / 9.0f), w5 = both(1.0f / 36.0f);
+    const float2 S = add2(B2xx, B2yy);
+    const float2 W0 = fma2(both(-4.0f), fma2(w1, B0, mul2(w5, B0)), B0);
+    p[0] = fma2(a, p[0], fma2(both(-(2.0f / 3.0f)), S, W0));
+    const float2 e13 = fma2(nsixth, B2yy, fma2(w1, B0, mul2(third, B2xx)));
+    p[1] = fma2(a, p[1], fma2(third, B1x, e13));
+    p[3] = fma2(a, p[3], fma2(nthird, B1x, e13));
+    const float2 e24 = fma2(nsixth, B2xx, fma2(w1, B0, mul2(third, B2yy)));
+    p[2] = fma2(a, p[2], fma2(third, B1y, e24));
+    p[4] = fma2(a, p[4], fma2(nthird, B1y, e24));
+    const float2 e5 = fma2(w5, B0, mul2(twelfth, S));
+    const float2 e57 = fma2(both(0.25f), B2xy, e5), s5 = add2(B1x, B1y);
+    p[5] = fma2(a, p[5], fma2(twelfth, s5, e57));
+    p[7] = fma2(a, p[7], fma2(ntwelfth, s5, e57));
+    const float2 e68 = fma2(both(-0.25f), B2xy, e5), s6 = sub2(B1y, B1x);
+    p[6] = fma2(a, p[6], fma2(twelfth, s6, e68));
+    p[8] = fma2(a, p[8], fma2(ntwelfth, s6, e68));
+}
+
 // Raw first and second moments of nine populations (the diagonal pairs'
 // sums and differences shared).
 template <typename real>
@@ -347,6 +383,73 @@ struct Macro {
     real H, T, fl, rho, ux, uy;
 };
 
+// cell_update with flow in FP32 arithmetic, f and g as pairs: the same
+// operations in the same order as the scalar form (whose products are
+// contracted into the following add or subtract).
+template <typename S>
+__device__ __forceinline__ Macro<float> cell_update_pair(const SweepArgs<float> &a, float f[9], float g[9]) {
+    constexpr bool kDev = Store<S>::kDev;
+    constexpr float kF = Store<S>::kF, kG = Store<S>::kG;
+    float2 p[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) p[i] = make_float2(f[i], g[i]);
+    const float2 s = add2(add2(add2(add2(p[0], p[1]), add2(p[2], p[3])), add2(add2(p[4], p[5]), add2(p[6], p[7]))),
+                          p[8]);
+    const float2 s57 = add2(p[5], p[7]), s68 = add2(p[6], p[8]), d57 = sub2(p[5], p[7]), d68 = sub2(p[6], p[8]);
+    const float2 jx = add2(sub2(p[1], p[3]), sub2(d57, d68)), jy = add2(sub2(p[2], p[4]), add2(d57, d68));
+    const float2 d = add2(s57, s68);
+    const float2 xx = add2(add2(p[1], p[3]), d), yy = add2(add2(p[2], p[4]), d), xy = sub2(s57, s68);
+    Macro<float> m;
+    if constexpr (kF != 1.0f) m.rho = fmaf(s.x, 1.0f / kF, 1.0f);
+    else if constexpr (kDev) m.rho = 1.0f + s.x;
+    else m.rho = s.x;
+    if constexpr (kG != 1.0f) m.H = s.y * (1.0f / kG);
+    else m.H = s.y;
+    invert(m.H, a.Lh, a.inv_Lh, m.T, m.fl);
+    float Fk = a.gbeta * m.T;
+    float iu = recip(m.rho);
+    if constexpr (kF != 1.0f) {
+        iu = iu * (1.0f / kF);
+        Fk = Fk * kF;
+    }
+    const float ux = m.fl * jx.x * iu, uy = m.fl * fmaf(0.5f, Fk, jy.x) * iu;
+    m.ux = ux;
+    m.uy = uy;
+    const float third = 1.0f / 3.0f;
+    float T = m.T, rk = m.rho;
+    if constexpr (kG != 1.0f) T = m.T * kG;
+    const float R0 = s.x;  // rho, or rho - 1 for stored deviations, in stored units
+    if constexpr (kF != 1.0f) rk = m.rho * kF;
+    const float d1 = a.k1 - a.k0, d2 = a.k2 - a.k0, k0T = a.k0 * T;
+    const float e1 = a.k1f - a.k0f, e2 = a.k2f - a.k0f, k0 = a.k0f;
+    const float s1 = fmaf(-0.5f, a.k1f, 1.0f), s2 = fmaf(-0.5f, a.k2f, 1.0f);
+    const float rux = rk * ux, ruy = rk * uy;
+    // products with a second use are rounded, not contracted
+    const float rxx = __fmul_rn(rux, ux), rxy = __fmul_rn(rux, uy), ryy = __fmul_rn(ruy, uy);
+    const float A1x = e1 * __fsub_rn(jx.x, rux);
+    const float A1y = fmaf(e1, __fsub_rn(jy.x, ruy), -(s1 * Fk));
+    const float A2xx = e2 * __fsub_rn(fmaf(-R0, third, xx.x), rxx);
+    const float A2xy = fmaf(e2, __fsub_rn(xy.x, rxy), -(s2 * ux * Fk));
+    const float A2yy = fmaf(e2, __fsub_rn(fmaf(-R0, third, yy.x), ryy), -(s2 * 2.0f * uy * Fk));
+    const float2 B1x = make_float2(fmaf(k0, rux, -A1x), fmaf(k0T, ux, -(d1 * fmaf(-T, ux, jx.y))));
+    const float2 B1y = make_float2(fmaf(k0, ruy, -A1y), fmaf(k0T, uy, -(d1 * fmaf(-T, uy, jy.y))));
+    const float2 B2xx = make_float2(fmaf(k0, rxx, -A2xx), -d2 * fmaf(-T, third, xx.y));
+    const float2 B2xy = make_float2(fmaf(k0, rxy, -A2xy), -d2 * xy.y);
+    const float2 B2yy = make_float2(fmaf(k0, ryy, -A2yy), -d2 * fmaf(-T, third, yy.y));
+    emit2(p, make_float2(1.0f - k0, 1.0f - a.k0), make_float2(k0 * R0, k0T), B1x, B1y, B2xx, B2xy, B2yy);
+    p[0].y = fmaf(a.k0, s.y - T, p[0].y);
+    // FP32 storage: the rest population from the collision's mass invariant
+    // (cell_update)
+    if constexpr (!kDev)
+        p[0].x = s.x - (((p[1].x + p[2].x) + (p[3].x + p[4].x)) + ((p[5].x + p[6].x) + (p[7].x + p[8].x)));
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        f[i] = p[i].x;
+        g[i] = p[i].y;
+    }
+    return m;
+}
+
 // Steps 2-5 on one cell: macroscopic fields, then both collisions in place
 // (COLLIDE = false stops after the fields).  f and g are in stored units (see
 // ld_f); the returned fields are physical.  With the 16-bit codecs f holds
@@ -357,6 +460,7 @@ struct Macro {
 // T kG and H kG in place of T and H.
 template <typename real, typename S, bool FLOW, bool COLLIDE>
 __device__ __forceinline__ Macro<real> cell_update(const SweepArgs<real> &a, real f[9], real g[9]) {
+    if constexpr (FLOW && COLLIDE && sizeof(real) == 4) return cell_update_pair<S>(a, f, g);
     constexpr bool kDev = Store<S>::kDev;
     constexpr real kF = real(Store<S>::kF), kG = real(Store<S>::kG);
     Macro<real> m;
