@@ -60,6 +60,8 @@ struct ChunkGraph {
     bool diag = false;
     bool one_buffer = false;  // sweeps of one-buffer streaming, from phase `phase`
     int phase = 0;
+    int flip = 0, end_phase = 0;  // the handle's state after the piece: cur ^ flip, phase,
+    bool end_prev = false;        // has_prev (single lattices)
     cudaGraphExec_t exec = nullptr;
     unsigned long long stamp = 0;
 };
@@ -86,6 +88,9 @@ struct lbm_s {
     // layout (always between calls), 1 after a push sweep
     int streaming = LBM_STREAM_TWO_BUFFERS;  // set per precision by lbm_create
     int phase = 0;
+    bool streaming_chosen = false;  // by lbm_set_streaming: one sweep per step, as asked
+    int tile_w = 0, tile_h = 0, tile_t = 0;  // several steps per launch (tile_plan); tile_t = 0: off
+    double *qgroup = nullptr;
     long long step = 0;
     long long diag_every = 0;
     bool params_set = false;
@@ -198,6 +203,88 @@ void set_grid(lbm_s *h) {
     bands = std::max(1, std::min(bands, std::max(1, h->ny / 4)));
     h->sgrid = dim3(h->ntx, bands);
     h->snq = h->p.problem == LBM_CAVITY ? (int)h->sgrid.x : (int)h->sgrid.y;
+}
+
+// Region of the first of T steps of a core of w x h cells.
+int tile_cells(const lbm_s *h, int w, int hh, int T, int t) {
+    const int halo = 2 * (T - t);
+    const int rows = h->p.problem == LBM_STEFAN ? h->ny : std::min(h->ny, hh + halo);
+    return std::min(h->nx, w + halo) * rows;
+}
+
+size_t slot_bytes(const lbm_s *h) {
+    return h->p.flow_on ? 2 * h->esize : h->esize;  // f_i and g_i, or g_i
+}
+
+size_t tile_q_offset(const lbm_s *h, int w, int hh, int T) {
+    const size_t rows = h->p.problem == LBM_STEFAN ? (size_t)h->ny : (size_t)hh + 2 * T;
+    return (rows * (size_t)(w + 2 * T) * 9 * slot_bytes(h) + 15) / 16 * 16;
+}
+
+size_t tile_smem(const lbm_s *h, int w, int hh, int T) {
+    return tile_q_offset(h, w, hh, T) +
+           (size_t)T * 3 * (h->p.problem == LBM_STEFAN ? hh : w) * (h->precision == LBM_FP64 ? 8 : 4);
+}
+
+// Core and steps of the tile kernel for this lattice, or none.  A launch costs
+// `launch` whatever it does; a step the larger of `least` (its latency) and its
+// cells' issue time on the SM that holds the most of them.  The candidate with
+// the least time per step by this model, its constants fitted to GB300 (FP32,
+// measured / model in us per step: 64 x 32 1.4 / 1.3, 256 x 128 1.7 / 1.6,
+// 512 x 512 4.5 / 4.3).  A core's width is a multiple of 32 in the cavity, so
+// that the inflow's groups are a sweep's warps.
+// Which lattices: FP32 and 16-bit storage up to 2^19 cells (per step, sweep and
+// tiles: 256 x 128 FP32 5.4 and 1.7 us, 512 x 512 7.1 and 4.5, 1024 x 512 9.0 and
+// 8.3; 256 x 128 BF16-SR 7.8 and 1.9), above which the sweep's larger launches
+// have paid for themselves.  FP64 with flow is bound by its pipe and gains
+// nothing from fewer launches (128 x 64: 18.9 and 18.2 us); without flow up to
+// 2^14 cells (1024 x 4 Stefan: 8.6 and 3.6).
+void tile_plan(lbm_s *h) {
+    h->tile_t = 0;
+    const bool stefan = h->p.problem == LBM_STEFAN, fp64 = h->precision == LBM_FP64, flow = h->p.flow_on != 0;
+    const long long cells = (long long)h->nx * h->ny;
+    if (h->nx > kTileMaxNx || (stefan && h->ny > 32)) return;
+    if (cells > (fp64 ? (flow ? 0 : 1 << 14) : 1 << 19)) return;
+    const double per_cell = fp64 ? 18.6 : (h->esize == 2 ? 1.6 : 1.5) * (flow ? 1.0 : 0.6);
+    const double least = fp64 ? 2200.0 : 700.0, launch = 4500.0;
+    double best = 1e30;
+    for (int w = stefan ? 8 : 32; w <= 128; w *= 2)
+        for (int hh = stefan ? h->ny : 2; hh <= (stefan ? h->ny : 64); hh += hh < 16 ? 1 : 4)
+            for (int T = 2; T <= kTileMaxSteps; ++T) {
+                const size_t smem = tile_smem(h, w, hh, T);
+                const int most = tile_cells(h, w, hh, T, 1);
+                if (smem > kTileSmemMax || (long long)most * std::min(h->nx, w + 2 * T) >= (1 << 20)) break;
+                const long long tiles = (long long)((h->nx + w - 1) / w) * ((h->ny + hh - 1) / hh);
+                const double waves = (double)((tiles + h->num_sms - 1) / h->num_sms);
+                const double resident = std::max(1.0, std::floor(kTileSmemMax / (double)smem));
+                double ns = launch * std::ceil(waves / resident);
+                for (int t = 1; t <= T; ++t) ns += std::max(least, waves * per_cell * tile_cells(h, w, hh, T, t));
+                if (ns / T < best) {
+                    best = ns / T;
+                    h->tile_w = w;
+                    h->tile_h = hh;
+                    h->tile_t = T;
+                }
+            }
+}
+
+bool use_tiles(const lbm_s *h) { return h->tile_t >= 2 && !h->streaming_chosen && !use_staged(h); }
+
+TileArgs tile_args(const lbm_s *h, int T) {
+    TileArgs tl{};
+    tl.T = T;
+    tl.W = h->tile_w;
+    tl.H = h->tile_h;
+    tl.tiles_x = (h->nx + tl.W - 1) / tl.W;
+    tl.tiles_y = (h->ny + tl.H - 1) / tl.H;
+    tl.pitch = tl.W + 2 * T;
+    const int most = h->precision == LBM_FP64 ? kTileThreads64 : kTileThreads;
+    const int cells = tile_cells(h, tl.W, tl.H, T, 1), rounds = (cells + most - 1) / most;
+    tl.threads = std::min(most, ((cells + rounds - 1) / rounds + 31) / 32 * 32);
+    tl.q_offset = (unsigned)tile_q_offset(h, tl.W, tl.H, T);
+    tl.smem = (unsigned)tile_smem(h, tl.W, tl.H, T);
+    tl.qgroup = h->qgroup;
+    return tl;
 }
 
 double *staging(lbm_s *h) {
@@ -340,6 +427,43 @@ int launch_one_aa(lbm_s *h, bool diag) {
     return LBM_OK;
 }
 
+// T steps of a small lattice in one launch (tile.cuh), from buf[cur] into the
+// other buffer.  The parity word alternates from launch to launch with the
+// buffer; the rounding seed advances by T, so the populations are bitwise those
+// of T sweeps.
+template <typename real, typename S>
+int launch_tiles(lbm_s *h, int T) {
+    SweepArgs<real> a = make_args<real>(h, h->buf[h->cur], h->buf[h->cur ^ 1]);
+    cudaError_t e = launch_tile<real, S>(a, tile_args(h, T), h->p.problem, h->p.flow_on != 0, h->stream);
+    if (e != cudaSuccess) return set_err(h, LBM_ERR_CUDA, "tile launch failed: %s", cudaGetErrorString(e));
+    h->cur ^= 1;
+    h->has_prev = false;  // buf[cur ^ 1] is T steps old until the call's closing sweep
+    h->step += T;
+    return LBM_OK;
+}
+
+// len sweeps, the last one diagnostic if diag: one launch each, or, on small
+// lattices, several steps per launch -- evenly many, up to the plan's -- and the
+// diagnostic one by itself.
+template <typename real, typename S>
+int launch_sweeps(lbm_s *h, long long len, bool diag, bool one_buffer) {
+    int rc = LBM_OK;
+    if (use_tiles(h)) {
+        const long long plain = diag ? len - 1 : len, n = (plain + h->tile_t - 1) / h->tile_t;
+        for (long long k = 0; k < n && rc == LBM_OK; ++k) {
+            const int T = (int)(plain * (k + 1) / n - plain * k / n);
+            rc = T == 1 ? launch_one<real, S>(h, false) : launch_tiles<real, S>(h, T);
+        }
+        if (diag && rc == LBM_OK) rc = launch_one<real, S>(h, true);
+        return rc;
+    }
+    for (long long j = 0; j < len && rc == LBM_OK; ++j) {
+        const bool d = diag && j == len - 1;
+        rc = one_buffer ? launch_one_aa<real, S>(h, d) : launch_one<real, S>(h, d);
+    }
+    return rc;
+}
+
 void drop_graphs(lbm_s *h) {
     for (ChunkGraph &g : h->graphs) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
@@ -354,7 +478,6 @@ void drop_graphs(lbm_s *h) {
 // so a captured piece replays correctly at any later step.
 template <typename real, typename S>
 int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
-    auto launch = [&](bool d) { return one_buffer ? launch_one_aa<real, S>(h, d) : launch_one<real, S>(h, d); };
     bool graphs = h->graph_chunk >= 2 && len >= 2 && len <= h->graph_chunk;
     if (graphs) {
         cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -387,10 +510,12 @@ int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
             const long long step0 = h->step;
             const bool prev0 = h->has_prev;
             CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-            int rc = LBM_OK;
-            for (long long j = 0; j < len && rc == LBM_OK; ++j) rc = launch(diag && j == len - 1);
+            const int rc = launch_sweeps<real, S>(h, len, diag, one_buffer);
             cudaGraph_t graph = nullptr;
             cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
+            slot->flip = h->cur ^ cur0;
+            slot->end_phase = h->phase;
+            slot->end_prev = h->has_prev;
             h->cur = cur0;
             h->phase = phase0;
             h->step = step0;
@@ -413,23 +538,16 @@ int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
     if (graphs) {
         slot->stamp = ++h->graph_clock;
         CUDA_TRY(h, cudaGraphLaunch(slot->exec, h->stream));
-        if (one_buffer) {
-            h->phase ^= (int)(len & 1);
-            h->has_prev = false;
-        } else {
-            h->cur ^= (int)(len & 1);
-            h->has_prev = true;
-        }
+        h->cur ^= slot->flip;
+        h->phase = slot->end_phase;
+        h->has_prev = slot->end_prev;
         h->step += len;
         h->stats.sweeps_replayed += len;
         return LBM_OK;
     }
-    for (long long j = 0; j < len; ++j) {
-        const int rc = launch(diag && j == len - 1);
-        if (rc != LBM_OK) return rc;
-    }
-    h->stats.sweeps_direct += len;
-    return LBM_OK;
+    const int rc = launch_sweeps<real, S>(h, len, diag, one_buffer);
+    if (rc == LBM_OK) h->stats.sweeps_direct += len;
+    return rc;
 }
 
 // n sweeps, cut into pieces that end at the diagnostic sweeps (every
@@ -444,7 +562,8 @@ int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
 template <typename real, typename S>
 int enqueue_steps(lbm_s *h, long long n) {
     long long aa = 0;
-    if (h->streaming == LBM_STREAM_ONE_BUFFER && !use_staged(h) && n >= 3) aa = (n & 1) ? n - 1 : n - 2;
+    if (h->streaming == LBM_STREAM_ONE_BUFFER && !use_staged(h) && !use_tiles(h) && n >= 3)
+        aa = (n & 1) ? n - 1 : n - 2;
     for (long long done = 0; done < aa;) {
         long long len = aa - done;
         bool diag = false;
@@ -611,7 +730,8 @@ int lbm_create(int nx, int ny, int precision, void *cuda_stream, lbm_handle *out
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t nred = (nblk + 1023) / 1024;
     const size_t o_rec = 256, o_q = o_rec + up(sizeof(DevRecord)), o_d = o_q + up(nqmax * 8),
-                 o_d2 = o_d + up(nblk * 32), bytes = o_d2 + up(nred * 32);
+                 o_d2 = o_d + up(nblk * 32), o_g = o_d2 + up(nred * 32),
+                 bytes = o_g + (nx <= kTileMaxNx ? (size_t)kTileMaxSteps * ((nx + 127) / 128 * 4) * 8 : 0);
     h->scratch = dev_alloc(h, bytes);
     if (!h->scratch) {
         lbm_destroy(h);
@@ -623,6 +743,7 @@ int lbm_create(int nx, int ny, int precision, void *cuda_stream, lbm_handle *out
     h->qpart = reinterpret_cast<double *>(s + o_q);
     h->dpart = reinterpret_cast<double *>(s + o_d);
     h->dpart2 = reinterpret_cast<double *>(s + o_d2);
+    h->qgroup = reinterpret_cast<double *>(s + o_g);
     e = cudaMemsetAsync(h->scratch, 0, bytes, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
@@ -653,6 +774,7 @@ int lbm_set_params(lbm_handle h, const lbm_params *p) {
         h->strip_on = 0;
     }
     set_grid(h);
+    tile_plan(h);
     h->step = 0;
     h->cur = 0;
     h->phase = 0;  // a call cut short mid-way through its one-buffer sweeps may have left 1
@@ -758,6 +880,7 @@ int lbm_set_streaming(lbm_handle h, int mode) {
     if (!h || (mode != LBM_STREAM_TWO_BUFFERS && mode != LBM_STREAM_ONE_BUFFER))
         return set_err(h, LBM_ERR_ARG, "mode must be LBM_STREAM_TWO_BUFFERS or LBM_STREAM_ONE_BUFFER");
     drop_graphs(h);
+    h->streaming_chosen = true;
     h->streaming = mode;  // between calls buf[cur] always holds the pull layout (phase 0)
     return LBM_OK;
 }

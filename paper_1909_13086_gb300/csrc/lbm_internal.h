@@ -115,6 +115,24 @@ struct alignas(16) SweepArgs {
     double *oH, *oT, *oFL, *oUX, *oUY, *oRHO;
 };
 
+// Several steps of a small lattice in one launch (tile.cuh): T steps by blocks
+// that own cores of W x H cells each.
+constexpr int kTileThreads = 768;     // block size limit, FP32 arithmetic (80 registers)
+constexpr int kTileThreads64 = 256;   // FP64 (its pipe is busy with four warps; no spills)
+constexpr int kTileMaxSteps = 16;
+constexpr int kTileMaxNx = 4096;      // the inflow's fold: 32 lanes x 128 columns
+constexpr size_t kTileSmemMax = 230400;
+struct TileArgs {
+    int T;                 // steps of this launch, 1 .. kTileMaxSteps
+    int W, H;              // core of a block; W a multiple of 32 in the cavity
+    int tiles_x, tiles_y;  // cores in the lattice (Stefan: tiles_y = 1, H = ny <= 32)
+    int pitch;             // shared-memory cells per row: W + 2 T
+    int threads;           // block size
+    unsigned smem;         // dynamic shared memory: the slots, then at q_offset T x 3 x (W, or
+    unsigned q_offset;     // H in the Stefan problem) inflow terms in the working precision
+    double *qgroup;        // device scratch: T x (heated groups of 32 wall cells)
+};
+
 // Launchers, instantiated in sweep_fp32.cu / sweep_fp64.cu / sweep_f16.cu /
 // sweep_bf16.cu for (compute real, storage codec S) = (float, float),
 // (double, double), (float, F16<SR>), (float, BF16<SR>), SR = round to
@@ -129,6 +147,8 @@ struct BF16;
 template <typename real, typename S>
 cudaError_t launch_lattice(const SweepArgs<real> &a, int problem, bool flow, int mode,
                            dim3 grid, dim3 block, cudaStream_t s, bool pdl, int streaming = kPull);
+template <typename real, typename S>
+cudaError_t launch_tile(const SweepArgs<real> &a, const TileArgs &tl, int problem, bool flow, cudaStream_t s);
 template <typename real, typename S>
 cudaError_t launch_init(const SweepArgs<real> &a, double amp, uint64_t seed, dim3 grid,
                         dim3 block, cudaStream_t s);

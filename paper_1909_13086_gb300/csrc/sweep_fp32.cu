@@ -1,6 +1,7 @@
 // FP32 storage and arithmetic instantiation of the fused sweep.
-#include "sweep.cuh"
+#include "tile.cuh"
 
 namespace btrirt {
 BTRIRT_INSTANTIATE(float, float)
+BTRIRT_INSTANTIATE_TILE(float, float)
 }  // namespace btrirt
