@@ -147,9 +147,9 @@ int lbm_step(lbm_handle h, long long n);
 int lbm_set_diag_every(lbm_handle h, long long k);
 
 /* Launch shape of the sweep (the tuner's knobs): rows of the lattice walked by
- * each thread of a block (1 to 1024, default 1, or 3 with 16-bit storage);
+ * each thread of a block (1 to 1024, default 1, or 2 with 16-bit storage);
  * the distance, in rows, at which each block asks L2 to prefetch a later
- * block's tile rows (0 = off, default 16, or 32 with 16-bit storage); and
+ * block's tile rows (0 = off, default 16, or 0 with 16-bit storage); and
  * graph_chunk, the longest piece
  * of sweeps lbm_step replays from a CUDA graph (0 = launch every sweep
  * directly; default 128).  Successive sweeps visit the lattice's row bands in
@@ -347,8 +347,8 @@ int lbm_batch_count(lbm_batch b, int *count);
 int lbm_batch_step(lbm_batch b, long long n);
 
 /* Launch shape of the batch's step kernel: rows of a member walked by each
- * block (0 = the default: 2, or 4 with 16-bit storage; up to 1024), the L2
- * prefetch distance in rows (-1 = the default: 4),
+ * block (0 = the default: 2, or 3 with 16-bit storage; up to 1024), the L2
+ * prefetch distance in rows (-1 = the default: 0),
  * and interleave = 1 (the default) to number the blocks of a one-size batch
  * member after member (block b belongs to member b mod n) instead of member
  * by member (0; a batch whose members' block counts differ is always member

@@ -18,6 +18,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lbm.h"
@@ -35,16 +36,13 @@ void *g_alloc_ctx = nullptr;
 
 constexpr int kDefaultRows = 1;       // rows walked by each thread of a block (tuned on GB300)
 constexpr int kDefaultPrefetch = 16;  // L2 prefetch distance in rows (tuned on GB300)
-// 16-bit storage is bound by instruction issue, and a thread's set-up (indices,
-// the rounding seed, the block's tail) costs ~115 instructions against ~316
-// per cell: 3 rows per thread spread it, with every row of a block prefetched
-// (2048 x 1024 BF16-SR cavity on GB300, prefetch 8: 1 row 31.2 us, 2 rows
-// 28.6, 3 rows 27.9, 4 rows 29.9, 6 rows 30.0 us per step; with the
-// alternating sweep direction, 3 rows: prefetch 8 / 16 / 32 / 48 26.5 / 26.5 /
-// 26.3 / 26.2 us).  FP32 is memory bound and fastest at 1 row (2 rows: +0.6
-// us; prefetch 4 / 16 / 32: 41.8 / 41.5 / 41.4 us).
-constexpr int kDefaultRows16 = 3;
-constexpr int kDefaultPrefetch16 = 32;
+// 16-bit storage: 2 rows per thread spread a thread's set-up (indices, the rounding
+// seed, the block's tail), and with two cells per thread the loads in flight need no
+// prefetch (2048 x 1024 FP16-SR on GB300, us per step: 1 / 2 / 3 rows 22.6 / 21.1 /
+// 21.2; 2 rows, prefetch 0 / 16 / 48: 21.1 / 21.4 / 21.4).  FP32 is memory bound and
+// fastest at 1 row (35.9; 2 rows 36.7).
+constexpr int kDefaultRows16 = 2;
+constexpr int kDefaultPrefetch16 = 0;
 constexpr int kDefaultGraphChunk = 128;  // longest graph-replayed piece (0 = direct launches)
 constexpr int kGraphCache = 16;          // cached piece graphs per handle
 
@@ -313,6 +311,14 @@ SweepArgs<real> make_args(const lbm_s *h, const void *src, void *dst) {
     a.Lh = (real)h->d.Lh;
     a.inv_Lh = (real)(1.0 / h->d.Lh);
     a.gbeta = (real)h->d.gbeta;
+    a.d1 = a.k1 - a.k0;
+    a.d2 = a.k2 - a.k0;
+    a.e1 = a.k1f - a.k0f;
+    a.e2 = a.k2f - a.k0f;
+    a.a0 = real(1) - a.k0;
+    a.a0f = real(1) - a.k0f;
+    a.s1 = std::fma(real(-0.5), a.k1f, real(1));
+    a.s2 = std::fma(real(-0.5), a.k2f, real(1));
     a.strip_on = h->strip_on;
     a.lo2 = h->lo2;
     a.hi2 = h->hi2;
@@ -1139,8 +1145,8 @@ struct lbm_batch_s {
     std::vector<int> host_parity;
     int nblocks = 0;
     int uniform = 0;          // blocks per member when all members have the same count
-    int rows = 0;             // launch shape: rows per block (0: 2, or 4 with 16-bit storage),
-    int prefetch = -1;        // L2 prefetch distance (-1: 4 rows),
+    int rows = 0;             // launch shape: rows per block (0: 2, or 3 with 16-bit storage),
+    int prefetch = -1;        // L2 prefetch distance (-1: off),
     int interleave = 1;       // interleaved block order (uniform batches only; see batch_kernel)
     int streaming = -1;       // lbm_batch_set_streaming; -1: one buffer, two for FP64
     bool dirty = true;        // table must be rebuilt and uploaded
@@ -1188,14 +1194,12 @@ template <typename real>
 size_t entry_bytes() { return sizeof(BatchEntry<real>); }
 
 // Default launch shape of a batch, whatever the members' own lbm_set_launch
-// settings: 2 rows per block (4 with 16-bit storage), L2 prefetch 4 rows
-// ahead, blocks of a one-size batch interleaved over the members -- the
-// fastest shapes for 64 cavities of 256 x 128 on GB300 (FP32 46.1 us per
-// step, 55.9 with 2 rows member by member and no alternating direction;
-// BF16-SR 32.1 us, 43.3).  Longer prefetch distances run ahead of a small
-// member's sweep (FP32, 2 rows: prefetch 4 / 8 / 16 / 32 46.1 / 47.4 / 51.5 /
-// 57.5 us).  Results do not depend on it.
-constexpr int kBatchRows32 = 2, kBatchRows16 = 4, kBatchPrefetch32 = 4, kBatchPrefetch16 = 4;
+// settings: 2 rows per block (3 with 16-bit storage), no L2 prefetch, blocks of a
+// one-size batch interleaved over the members -- the fastest shapes for 32 cavities
+// of 256 x 128 on GB300 (us per step at 1 / 2 / 3 / 4 rows: FP32 18.9 / 17.7 / 18.0 /
+// 19.2, BF16-SR 15.6 / 15.1 / 14.7 / 14.9; prefetch 4: 18.0 and 14.9).  Results do
+// not depend on it.
+constexpr int kBatchRows32 = 2, kBatchRows16 = 3, kBatchPrefetch32 = 0, kBatchPrefetch16 = 0;
 
 template <typename real>
 void batch_build(lbm_batch_s *b) {

@@ -272,16 +272,9 @@ __device__ __forceinline__ uint32_t lcg_next32(uint32_t &s) {
 // ---- H -> (T, f_l): H_s = C_p T_m = 0, H_l = H_s + L.
 template <typename real>
 __device__ __forceinline__ void invert(real H, real Lh, real inv_Lh, real &T, real &fl) {
-    if (H <= real(0)) {
-        T = H;
-        fl = real(0);
-    } else if (H >= Lh) {
-        T = H - Lh;
-        fl = real(1);
-    } else {
-        T = real(0);
-        fl = H * inv_Lh;
-    }
+    // selects, no branches; a NaN H gives T = 0, f_l = NaN
+    T = H <= real(0) ? H : max(H - Lh, real(0));
+    fl = H <= real(0) ? real(0) : (H >= Lh ? real(1) : H * inv_Lh);
 }
 
 // 1 / x: the fast reciprocal in FP32 (about 2 ulp; the FP32 path's tolerance
@@ -332,6 +325,7 @@ __device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, both(-1.0f), a); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 // emit on a pair (FP32: the rest weight's share as the remainder).
@@ -420,9 +414,8 @@ __device__ __forceinline__ Macro<float> cell_update_pair(const SweepArgs<float> 
     if constexpr (kG != 1.0f) T = m.T * kG;
     const float R0 = s.x;  // rho, or rho - 1 for stored deviations, in stored units
     if constexpr (kF != 1.0f) rk = m.rho * kF;
-    const float d1 = a.k1 - a.k0, d2 = a.k2 - a.k0, k0T = a.k0 * T;
-    const float e1 = a.k1f - a.k0f, e2 = a.k2f - a.k0f, k0 = a.k0f;
-    const float s1 = fmaf(-0.5f, a.k1f, 1.0f), s2 = fmaf(-0.5f, a.k2f, 1.0f);
+    const float d1 = a.d1, d2 = a.d2, e1 = a.e1, e2 = a.e2, s1 = a.s1, s2 = a.s2;
+    const float k0 = a.k0f, k0T = a.k0 * T;
     const float rux = rk * ux, ruy = rk * uy;
     // products with a second use are rounded, not contracted
     const float rxx = __fmul_rn(rux, ux), rxy = __fmul_rn(rux, uy), ryy = __fmul_rn(ruy, uy);
@@ -436,7 +429,7 @@ __device__ __forceinline__ Macro<float> cell_update_pair(const SweepArgs<float> 
     const float2 B2xx = make_float2(fmaf(k0, rxx, -A2xx), -d2 * fmaf(-T, third, xx.y));
     const float2 B2xy = make_float2(fmaf(k0, rxy, -A2xy), -d2 * xy.y);
     const float2 B2yy = make_float2(fmaf(k0, ryy, -A2yy), -d2 * fmaf(-T, third, yy.y));
-    emit2(p, make_float2(1.0f - k0, 1.0f - a.k0), make_float2(k0 * R0, k0T), B1x, B1y, B2xx, B2xy, B2yy);
+    emit2(p, make_float2(a.a0f, a.a0), make_float2(k0 * R0, k0T), B1x, B1y, B2xx, B2xy, B2yy);
     p[0].y = fmaf(a.k0, s.y - T, p[0].y);
     // FP32 storage: the rest population from the collision's mass invariant
     // (cell_update)
@@ -448,6 +441,69 @@ __device__ __forceinline__ Macro<float> cell_update_pair(const SweepArgs<float> 
         g[i] = p[i].y;
     }
     return m;
+}
+
+// cell_update with flow in FP32 arithmetic on two cells at once (x and y of each
+// pair): the operations of cell_update_pair, every one of them packed.
+struct MacroTwo {
+    float2 H, fl, rho, ux, uy;
+};
+template <typename S>
+__device__ __forceinline__ MacroTwo cell_update_two(const SweepArgs<float> &a, float2 f[9], float2 g[9]) {
+    constexpr bool kDev = Store<S>::kDev;
+    constexpr float kF = Store<S>::kF, kG = Store<S>::kG;
+    float2 s[2], jx[2], jy[2], xx[2], xy[2], yy[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float2 *p = h ? g : f;
+        s[h] = add2(add2(add2(add2(p[0], p[1]), add2(p[2], p[3])), add2(add2(p[4], p[5]), add2(p[6], p[7]))), p[8]);
+        const float2 s57 = add2(p[5], p[7]), s68 = add2(p[6], p[8]), d57 = sub2(p[5], p[7]), d68 = sub2(p[6], p[8]);
+        jx[h] = add2(sub2(p[1], p[3]), sub2(d57, d68));
+        jy[h] = add2(sub2(p[2], p[4]), add2(d57, d68));
+        const float2 d = add2(s57, s68);
+        xx[h] = add2(add2(p[1], p[3]), d);
+        yy[h] = add2(add2(p[2], p[4]), d);
+        xy[h] = sub2(s57, s68);
+    }
+    float2 rho = s[0], H = s[1], T, fl;
+    if constexpr (kF != 1.0f) rho = fma2(s[0], both(1.0f / kF), both(1.0f));
+    else if constexpr (kDev) rho = add2(both(1.0f), s[0]);
+    if constexpr (kG != 1.0f) H = mul2(s[1], both(1.0f / kG));
+    invert(H.x, a.Lh, a.inv_Lh, T.x, fl.x);
+    invert(H.y, a.Lh, a.inv_Lh, T.y, fl.y);
+    float2 Fk = mul2(both(a.gbeta), T), iu = make_float2(recip(rho.x), recip(rho.y)), rk = rho;
+    if constexpr (kF != 1.0f) {
+        iu = mul2(iu, both(1.0f / kF));
+        Fk = mul2(Fk, both(kF));
+        rk = mul2(rho, both(kF));
+    }
+    const float2 ux = mul2(mul2(fl, jx[0]), iu), uy = mul2(mul2(fl, fma2(both(0.5f), Fk, jy[0])), iu);
+    const float2 nthird = both(-(1.0f / 3.0f)), R0 = s[0];
+    if constexpr (kG != 1.0f) T = mul2(T, both(kG));
+    // g
+    {
+        const float2 k0T = mul2(both(a.k0), T), nT = neg2(T), nd1 = both(-a.d1), nd2 = both(-a.d2);
+        const float2 B1x = fma2(k0T, ux, mul2(nd1, fma2(nT, ux, jx[1])));
+        const float2 B1y = fma2(k0T, uy, mul2(nd1, fma2(nT, uy, jy[1])));
+        emit2(g, both(a.a0), k0T, B1x, B1y, mul2(nd2, fma2(T, nthird, xx[1])), mul2(nd2, xy[1]),
+              mul2(nd2, fma2(T, nthird, yy[1])));
+        g[0] = fma2(both(a.k0), sub2(s[1], T), g[0]);
+    }
+    // f
+    const float2 rux = mul2(rk, ux), ruy = mul2(rk, uy), k0 = both(a.k0f), ne1 = both(-a.e1), ne2 = both(-a.e2);
+    const float2 sF = mul2(both(a.s1), Fk), s2 = both(a.s2), s22 = both(a.s2 * 2.0f);
+    // minus the relaxation terms A1, A2 of the scalar form
+    const float2 A1x = mul2(ne1, sub2(jx[0], rux));
+    const float2 A1y = fma2(ne1, sub2(jy[0], ruy), sF);
+    const float2 rxx = mul2(rux, ux), rxy = mul2(rux, uy), ryy = mul2(ruy, uy);
+    const float2 A2xx = mul2(ne2, sub2(fma2(R0, nthird, xx[0]), rxx));
+    const float2 A2xy = fma2(ne2, sub2(xy[0], rxy), mul2(mul2(s2, ux), Fk));
+    const float2 A2yy = fma2(ne2, sub2(fma2(R0, nthird, yy[0]), ryy), mul2(mul2(s22, uy), Fk));
+    emit2(f, both(a.a0f), mul2(k0, R0), fma2(k0, rux, A1x), fma2(k0, ruy, A1y), fma2(k0, rxx, A2xx),
+          fma2(k0, rxy, A2xy), fma2(k0, ryy, A2yy));
+    if constexpr (!kDev)
+        f[0] = sub2(s[0], add2(add2(add2(f[1], f[2]), add2(f[3], f[4])), add2(add2(f[5], f[6]), add2(f[7], f[8]))));
+    return {H, fl, rho, ux, uy};
 }
 
 // Steps 2-5 on one cell: macroscopic fields, then both collisions in place
@@ -1162,6 +1218,195 @@ __device__ __forceinline__ void finish_cell(const SweepArgs<real> &a, int x, int
     }
 }
 
+// ---- two neighbouring cells per thread (cavity, flow, FP32 arithmetic) ----
+// A thread with two columns runs all of the collision packed, and pays addresses,
+// uniform terms and loop overhead once for two cells.
+// Direction i of two neighbouring cells as stored: (f, f') and (g, g'), or the two
+// words of the paired layout.
+template <typename S>
+struct Two {
+    using T = uint2;
+    __device__ static void get(T v, float2 &f, float2 &g) {
+        f = make_float2(Store<S>::lo(v.x), Store<S>::lo(v.y));
+        g = make_float2(Store<S>::hi(v.x), Store<S>::hi(v.y));
+    }
+    __device__ static T load(const typename Store<S>::elem *p, int i) {
+        return __ldg(reinterpret_cast<const uint2 *>(p) + i * (kTW / 2));
+    }
+    // the cells' elements at two offsets (slot_ofs of a direction included)
+    __device__ static T load_at(const typename Store<S>::elem *p, int o0, int o1) {
+        return make_uint2(__ldg(reinterpret_cast<const uint32_t *>(p + o0)),
+                          __ldg(reinterpret_cast<const uint32_t *>(p + o1)));
+    }
+    __device__ static void store(typename Store<S>::elem *d, int i, T v) {
+        reinterpret_cast<uint2 *>(d)[i * (kTW / 2)] = v;
+    }
+    __device__ static void store_at(typename Store<S>::elem *d, int o, T v, bool second) {
+        *reinterpret_cast<uint32_t *>(d + o) = second ? v.y : v.x;
+    }
+};
+template <>
+struct Two<float> {
+    struct T {
+        float2 f, g;
+    };
+    __device__ static void get(const T &v, float2 &f, float2 &g) { f = v.f, g = v.g; }
+    __device__ static T load(const float *p, int i) {
+        return {__ldg(reinterpret_cast<const float2 *>(p + i * kTW)),
+                __ldg(reinterpret_cast<const float2 *>(p + (9 + i) * kTW))};
+    }
+    __device__ static T load_at(const float *p, int o0, int o1) {
+        return {make_float2(__ldg(p + o0), __ldg(p + o1)),
+                make_float2(__ldg(p + o0 + 9 * kTW), __ldg(p + o1 + 9 * kTW))};
+    }
+    __device__ static void store(float *d, int i, const T &v) {
+        *reinterpret_cast<float2 *>(d + i * kTW) = v.f;
+        *reinterpret_cast<float2 *>(d + (9 + i) * kTW) = v.g;
+    }
+    __device__ static void store_at(float *d, int o, const T &v, bool second) {
+        d[o] = second ? v.f.y : v.f.x;
+        d[o + 9 * kTW] = second ? v.g.y : v.g.x;
+    }
+};
+
+
+// Where a pair of cells (x, x + 1), x even, stands: its walls, and the elements
+// from its first cell to the columns beside the pair, one of which may lie in the
+// neighbouring tile.  has1: the second cell exists; an odd width's last pair has
+// one cell, and the other's column is padding of the tile: loaded, computed, never
+// stored, read by no cell.
+template <typename S>
+struct PairPlace {
+    bool left, right0, right1, has1, side;
+    int dL, dR;
+    static __device__ __forceinline__ constexpr int slot_ofs(int i) { return plane_ofs<S>(i, 0); }
+    // side: a lane of the warp touches a side wall (all lanes of the warp call)
+    __device__ __forceinline__ PairPlace(int x, int nx, int ny)
+        : left(x == 0), right0(x == nx - 1), right1(x + 1 >= nx - 1), has1(x + 1 < nx) {
+        constexpr int cs = col_step<S>();
+        const int lx = x % kTW;
+        const int tile = ny * kRS;  // elements from a column to the same one of the next tile
+        dL = lx == 0 && x > 0 ? cs * (kTW - 1) - tile : -cs;
+        dR = lx == kTW - 2 && x + 2 < nx ? tile - cs * (kTW - 2) : 2 * cs;
+        side = __any_sync(0xffffffffu, left || x + 1 >= nx - 1);
+    }
+    // the neighbour of the first / second cell against c_i lies beyond a wall
+    __device__ __forceinline__ bool wall0(int i, bool bottom, bool top) const {
+        return (cx_of(i) > 0 && left) || (cx_of(i) < 0 && right0) || (cy_of(i) > 0 && bottom) || (cy_of(i) < 0 && top);
+    }
+    __device__ __forceinline__ bool wall1(int i, bool bottom, bool top) const {
+        return !has1 || (cx_of(i) < 0 && right1) || (cy_of(i) > 0 && bottom) || (cy_of(i) < 0 && top);
+    }
+    // What streams into the pair, as stored (p: its first cell's element of plane
+    // 0); a direction from beyond a wall is the cell's own opposite population.
+    // Selects on 32-bit offsets; one path for all walls (a third one for the side
+    // walls alone, with fewer selects, outgrew the instruction cache: 2048 x 1024
+    // FP16-SR 22.2 us per step against 21.1).
+    __device__ __forceinline__ void pull(const typename Store<S>::elem *p, bool bottom, bool top,
+                                         typename Two<S>::T v[9]) const {
+        constexpr int cs = col_step<S>();
+        if (side || bottom || top) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const int cx = cx_of(i), in = slot_ofs(i) - cy_of(i) * kRS, own = slot_ofs(opp_of(i));
+                const int o0 = wall0(i, bottom, top) ? own : in + (cx > 0 ? dL : (cx < 0 ? cs : 0));
+                const int o1 = wall1(i, bottom, top) ? own + cs : in + (cx > 0 ? 0 : (cx < 0 ? dR : cs));
+                v[i] = Two<S>::load_at(p, o0, o1);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const int cx = cx_of(i), in = slot_ofs(i) - cy_of(i) * kRS;
+                if (cx == 0) v[i] = Two<S>::load(p - cy_of(i) * kRS, i);
+                else v[i] = Two<S>::load_at(p, in + (cx > 0 ? dL : cs), in + (cx > 0 ? 0 : dR));
+            }
+        }
+    }
+    // Direction i of the pair into the cells' own slots.
+    __device__ __forceinline__ void put_own(typename Store<S>::elem *p, int i, const typename Two<S>::T &v) const {
+        if (has1) Two<S>::store(p, i, v);
+        else Two<S>::store_at(p, slot_ofs(i), v, false);
+    }
+    // The push sweep of one-buffer streaming: into slot opp(i) of x + c_i, or the
+    // cell's own slot i where that lies beyond a wall.
+    __device__ __forceinline__ void push(typename Store<S>::elem *p, bool bottom, bool top, int i,
+                                         const typename Two<S>::T &v) const {
+        constexpr int cs = col_step<S>();
+        const int cx = cx_of(i), o = opp_of(i), out = slot_ofs(o) + cy_of(i) * kRS, own = slot_ofs(i);
+        if (side || bottom || top) {
+            const bool w0 = wall0(o, bottom, top), w1 = wall1(o, bottom, top);
+            Two<S>::store_at(p, w0 ? own : out + (cx > 0 ? cs : (cx < 0 ? dL : 0)), v, false);
+            if (has1) Two<S>::store_at(p, w1 ? own + cs : out + (cx > 0 ? dR : (cx < 0 ? 0 : cs)), v, true);
+        } else if (cx == 0) {
+            Two<S>::store(p + cy_of(i) * kRS, o, v);
+        } else {
+            Two<S>::store_at(p, out + (cx > 0 ? cs : dL), v, false);
+            Two<S>::store_at(p, out + (cx > 0 ? dR : 0), v, true);
+        }
+    }
+};
+
+// The pair's step result as stored, direction by direction, in the rounding order
+// of finish_cell for each cell.
+template <typename S, typename Put>
+__device__ __forceinline__ void emit_two(const SweepArgs<float> &a, int x, int y, const float2 f[9],
+                                         const float2 g[9], uint32_t step_seed, Put &&put) {
+    if constexpr (!Store<S>::kDev) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) put(i, typename Two<S>::T{f[i], g[i]});
+    } else if constexpr (!Store<S>::kSR) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            put(i, make_uint2(Store<S>::pack_rn(g[i].x, f[i].x), Store<S>::pack_rn(g[i].y, f[i].y)));
+    } else {
+        const uint32_t cell = (uint32_t)((long long)y * a.nx + x);
+        uint32_t r0 = hash32(step_seed ^ cell), r1 = hash32(step_seed ^ (cell + 1u));
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const uint32_t lo = Store<S>::pack_sr(g[i].x, f[i].x, lcg_next32(r0));
+            put(i, make_uint2(lo, Store<S>::pack_sr(g[i].y, f[i].y, lcg_next32(r1))));
+        }
+    }
+}
+
+// The three directions that enter a cell from the wall held at T_h.
+template <int PROB>
+__device__ __forceinline__ constexpr int hot_dir(int k) {
+    return PROB == kStefan ? (k == 0 ? 1 : (k == 1 ? 5 : 8)) : (k == 0 ? 2 : (k == 1 ? 5 : 6));
+}
+// wall_rule_g on a cell of that wall (g: the cell's own opposite populations
+// there), with each direction's inflow in the working precision (zero beside
+// the strip): its FP64 sum waits until the steps are done, off their path.
+template <typename real, typename S, int PROB>
+__device__ __forceinline__ void hot_wall(const SweepArgs<real> &a, int x, real g[9], real q[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        constexpr real kG = real(Store<S>::kG);
+        const int i = hot_dir<PROB>(k), xc2 = 2 * x + 1 - cx_of(i);
+        const real wt = real(2) * w_of<real>(i) * kG;
+        const bool hot = PROB == kStefan || (a.strip_on && xc2 >= a.lo2 && xc2 <= a.hi2);
+        q[k] = hot ? (wt - real(2) * g[i]) * (real(1) / kG) : real(0);
+        if (hot) g[i] = wt - g[i];
+    }
+}
+
+// hot_wall on the pair at y = 0; the inflow of the cells in the core.
+template <typename S>
+__device__ __forceinline__ double hot_wall_two(const SweepArgs<float> &a, int x, int xs, int xe,
+                                               float2 g[9]) {
+    float u[9], v[9], q[3];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) u[i] = g[i].x, v[i] = g[i].y;
+    double s = 0.0;
+    hot_wall<float, S, kCavity>(a, x, u, q);
+    if (x >= xs && x < xe) s += (double)q[0] + (double)q[1] + (double)q[2];
+    hot_wall<float, S, kCavity>(a, x + 1, v, q);
+    if (x + 1 >= xs && x + 1 < xe) s += (double)q[0] + (double)q[1] + (double)q[2];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = make_float2(u[i], v[i]);
+    return s;
+}
+
 // A block's end: the heated-wall inflow of this step (blocks touching the T_h
 // wall: the cavity's bottom row band, the Stefan problem's first tile column),
 // folded by the last such block to take a ticket, and the diagnostics
@@ -1306,18 +1551,97 @@ __device__ __forceinline__ void sweep_block(const SweepArgs<real> &a, const int 
     block_epilogue<real, PROB, MODE>(a, bx, by, gx, acc, sh);
 }
 
-// FP32 arithmetic: at least 8 blocks of 128 threads per SM (registers capped at
-// 64, the occupancy the memory pipeline needs); FP64 is ALU-bound and keeps its
-// registers.
+// sweep_block with two cells per thread: blocks of kTW / 2 threads.
+template <typename S, int MODE, int SM>
+__device__ __forceinline__ void sweep_block_two(const SweepArgs<float> &a, const int bx, const int by, const int gx,
+                                                double *sh) {
+    using E = typename Store<S>::elem;
+    using T = typename Two<S>::T;
+    const E *const src = static_cast<const E *>(a.src);
+    E *const dst = static_cast<E *>(a.dst);
+    const int x = bx * kTW + 2 * (int)threadIdx.x;
+    const int y0 = by * a.rows, y1 = min(y0 + a.rows, a.ny);
+    if (a.prefetch > 0 && (int)threadIdx.x < y1 - y0) {  // as in sweep_block
+        const int yp = (a.parity ? y0 - a.prefetch : y0 + a.prefetch) + (int)threadIdx.x;
+        if (yp >= 0 && yp < a.ny) prefetch_tile_row_l2(src + cell_index<S>(bx * kTW, yp, 0, a.ny));
+    }
+    const uint32_t step_seed = step_prologue<float, S, MODE>(a, bx, by);
+    const bool active = x < a.nx;
+    const PairPlace<S> at(x, a.nx, a.ny);
+    long long i0 = cell_index<S>(x, y0, 0, a.ny);
+    CellSums<float> acc;
+    for (int y = y0; y < y1; ++y, i0 += kRS) {
+        CellDiag<float> c0, c1;
+        if (active) {
+            const bool bottom = y == 0, top = y == a.ny - 1;
+            T v[9];
+            if (SM == kAALocal) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) v[i] = Two<S>::load(src + i0, opp_of(i));
+            } else {
+                at.pull(src + i0, bottom, top, v);
+            }
+            float2 f[9], g[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) Two<S>::get(v[i], f[i], g[i]);
+            if (bottom) acc.q += hot_wall_two<S>(a, x, 0, a.nx, g);
+            const MacroTwo m = cell_update_two<S>(a, f, g);
+            E *const d = dst + i0;
+            if (SM == kAAPush)
+                emit_two<S>(a, x, y, f, g, step_seed, [&](int i, const T &w) { at.push(d, bottom, top, i, w); });
+            else
+                emit_two<S>(a, x, y, f, g, step_seed, [&](int i, const T &w) { at.put_own(d, i, w); });
+            if (MODE == kSweepDiag) {
+                const float2 u2 = make_float2(m.ux.x * m.ux.x + m.uy.x * m.uy.x, m.ux.y * m.ux.y + m.uy.y * m.uy.y);
+                c0 = {m.fl.x, m.H.x, u2.x, !(isfinite(m.H.x) && isfinite(m.rho.x))};
+                if (at.has1) c1 = {m.fl.y, m.H.y, u2.y, !(isfinite(m.H.y) && isfinite(m.rho.y))};
+            }
+        }
+        if (MODE == kSweepDiag) {  // the whole warp, active or not
+            diag_row(acc, c0);
+            diag_row(acc, c1);
+        }
+    }
+    block_epilogue<float, kCavity, MODE>(a, bx, by, gx, acc, sh);
+}
+
+// Whether a sweep runs two cells per thread.
+template <typename real, int PROB, bool FLOW, int MODE>
+__host__ __device__ constexpr bool takes_two() {
+    return sizeof(real) == 4 && PROB == kCavity && FLOW && MODE != kFields;
+}
+template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM>
+__device__ __forceinline__ void sweep_any(const SweepArgs<real> &a, const int bx, const int by, const int gx,
+                                          double *sh) {
+    if constexpr (takes_two<real, PROB, FLOW, MODE>()) sweep_block_two<S, MODE, SM>(a, bx, by, gx, sh);
+    else sweep_block<real, S, PROB, FLOW, MODE, SM>(a, bx, by, gx, sh);
+}
+template <typename real, int PROB, bool FLOW, int MODE>
+__host__ __device__ constexpr int sweep_threads() {
+    return takes_two<real, PROB, FLOW, MODE>() ? kTW / 2 : kTW;
+}
+// Blocks per SM the register allocation aims at (BATCH: a batch kernel, whose
+// arguments sit in shared memory and take more registers).  Two cells per thread,
+// us per step at 8 / 10 / 12 blocks: 2048 x 1024 FP32 one buffer 36.4 / 35.9 / 36.2,
+// FP16-SR 21.7 / 21.6 / 21.1, 1001 x 701 BF16-SR 9.1 / 9.1 / 8.8; 32 x 256 x 128
+// batches FP32 18.2 / 17.7 / -, BF16-SR 15.0 / 14.7 / 15.7.
+template <typename real, typename S, int PROB, bool FLOW, int MODE, bool BATCH = false>
+__host__ __device__ constexpr int sweep_blocks() {
+    if (takes_two<real, PROB, FLOW, MODE>()) return Store<S>::kDev && !BATCH ? 12 : 10;
+    return sizeof(real) == 4 ? 1024 / kTW : 1;
+}
+
+// FP32 arithmetic, one cell per thread: at least 8 blocks of 128 threads per SM
+// (registers capped at 64, the occupancy the memory pipeline needs); FP64 is
+// ALU-bound and keeps its registers.
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM = kPull>
-__global__ void __launch_bounds__(kTW, sizeof(real) == 4 ? 1024 / kTW : 1)
+__global__ void __launch_bounds__(sweep_threads<real, PROB, FLOW, MODE>(), sweep_blocks<real, S, PROB, FLOW, MODE>())
     lattice_kernel(const SweepArgs<real> a) {
     __shared__ double sh[32 * 4];
     pdl_launch_dependents();
     pdl_wait();  // the previous sweep's populations, tickets and record
-    sweep_block<real, S, PROB, FLOW, MODE, SM>(a, blockIdx.x,
-                                               row_band((int)blockIdx.y, (int)gridDim.y, a.parity), gridDim.x,
-                                               sh);
+    sweep_any<real, S, PROB, FLOW, MODE, SM>(a, blockIdx.x, row_band((int)blockIdx.y, (int)gridDim.y, a.parity),
+                                             gridDim.x, sh);
 }
 
 // ---- the staged sweep (16-bit storage) ----
@@ -1613,7 +1937,8 @@ struct EntryLayout {
     static_assert(offsetof(BatchEntry<real>, a) == 0, "the argument sets open the entry");
 };
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM = kPull>
-__global__ void __launch_bounds__(kTW, sizeof(real) == 4 ? 1024 / kTW : 1)
+__global__ void __launch_bounds__(sweep_threads<real, PROB, FLOW, MODE>(),
+                                  sweep_blocks<real, S, PROB, FLOW, MODE, true>())
     batch_kernel(const BatchEntry<real> *entries, const int *starts, const int *parity, int n,
                  int uniform, int interleave, int j) {
     static_assert(sizeof(BatchEntry<real>) % 16 == 0, "entries are copied in 16-byte pieces");
@@ -1666,7 +1991,7 @@ __global__ void __launch_bounds__(kTW, sizeof(real) == 4 ? 1024 / kTW : 1)
     const BatchEntry<real> &e = *reinterpret_cast<const BatchEntry<real> *>(entry_sh);
     const SweepArgs<real> &a = e.a[meta[1]];
     const int l = (uniform > 0 && interleave) ? (int)(blockIdx.x / (unsigned)n) : (int)blockIdx.x - e.start;
-    sweep_block<real, S, PROB, FLOW, MODE, SM>(a, l % e.gx, row_band(l / e.gx, e.gy, a.parity), e.gx, sh);
+    sweep_any<real, S, PROB, FLOW, MODE, SM>(a, l % e.gx, row_band(l / e.gx, e.gy, a.parity), e.gx, sh);
 }
 
 // Per-entry diagnostics fold after a diagnostic batch step: block r folds the
@@ -1839,17 +2164,18 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
 template <typename real, typename S, int PROB, bool FLOW>
 static cudaError_t launch_mode(const SweepArgs<real> &a, int mode, dim3 grid, dim3 block,
                                cudaStream_t s, bool pdl, int streaming) {
+    const dim3 threads(sweep_threads<real, PROB, FLOW, kSweep>());  // of a sweep; `block`: of the other kernels
     if (streaming == kAAPush || streaming == kAALocal) {  // one-buffer streaming: sweeps only
         if (a.src != a.dst || a.staged) return cudaErrorInvalidValue;
         const bool push = streaming == kAAPush;
         switch (mode) {
             case kSweep:
-                return push ? launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep, kAAPush>, grid, block, s, pdl, a)
-                            : launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep, kAALocal>, grid, block, s, pdl, a);
+                return push ? launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep, kAAPush>, grid, threads, s, pdl, a)
+                            : launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep, kAALocal>, grid, threads, s, pdl, a);
             case kSweepDiag:
-                return push ? launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kAAPush>, grid, block, s, pdl,
+                return push ? launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kAAPush>, grid, threads, s, pdl,
                                        a)
-                            : launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kAALocal>, grid, block, s,
+                            : launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kAALocal>, grid, threads, s,
                                        pdl, a);
             default: return cudaErrorInvalidValue;
         }
@@ -1872,9 +2198,9 @@ static cudaError_t launch_mode(const SweepArgs<real> &a, int mode, dim3 grid, di
         }
     }
     switch (mode) {
-        case kSweep: return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep>, grid, block, s, pdl, a);
+        case kSweep: return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep>, grid, threads, s, pdl, a);
         case kSweepDiag:
-            return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag>, grid, block, s, pdl, a);
+            return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag>, grid, threads, s, pdl, a);
         case kFields: lattice_kernel<real, S, PROB, FLOW, kFields><<<grid, block, 0, s>>>(a); break;
         default: return cudaErrorInvalidValue;
     }
@@ -1912,10 +2238,11 @@ cudaError_t launch_batch(const void *entries, const int *starts, const int *pari
                          int uniform, int interleave, int nblocks, int problem, bool flow, bool diag,
                          int j, cudaStream_t s, bool pdl, int streaming) {
     const BatchEntry<real> *e = static_cast<const BatchEntry<real> *>(entries);
-    const dim3 grid(nblocks), block(kTW);
+    const dim3 grid(nblocks);
     cudaError_t err;
     if (streaming != kPull && streaming != kAAPush && streaming != kAALocal) return cudaErrorInvalidValue;
 #define BTRIRT_BATCH_SM(PROB, FLOW, SM)                                                                \
+    const dim3 block(sweep_threads<real, PROB, FLOW, kSweep>());                                           \
     err = diag ? launch_k(batch_kernel<real, S, PROB, FLOW, kSweepDiag, SM>, grid, block, s, pdl, e, starts, \
                           parity, n, uniform, interleave, j)                                           \
                : launch_k(batch_kernel<real, S, PROB, FLOW, kSweep, SM>, grid, block, s, pdl, e, starts,  \

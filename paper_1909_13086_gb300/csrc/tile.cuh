@@ -92,27 +92,6 @@ __device__ __forceinline__ void pull_first(const typename Store<S>::elem *b, con
     }
 }
 
-// The three directions that enter a cell from the wall held at T_h.
-template <int PROB>
-__device__ __forceinline__ constexpr int hot_dir(int k) {
-    return PROB == kStefan ? (k == 0 ? 1 : (k == 1 ? 5 : 8)) : (k == 0 ? 2 : (k == 1 ? 5 : 6));
-}
-// wall_rule_g on a cell of that wall (g: the cell's own opposite populations
-// there), with each direction's inflow in the working precision (zero beside
-// the strip): its FP64 sum waits until the steps are done, off their path.
-template <typename real, typename S, int PROB>
-__device__ __forceinline__ void hot_wall(const SweepArgs<real> &a, int x, real g[9], real q[3]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        constexpr real kG = real(Store<S>::kG);
-        const int i = hot_dir<PROB>(k), xc2 = 2 * x + 1 - cx_of(i);
-        const real wt = real(2) * w_of<real>(i) * kG;
-        const bool hot = PROB == kStefan || (a.strip_on && xc2 >= a.lo2 && xc2 <= a.hi2);
-        q[k] = hot ? (wt - real(2) * g[i]) * (real(1) / kG) : real(0);
-        if (hot) g[i] = wt - g[i];
-    }
-}
-
 // Rounds and packs the nine (f_i, g_i) of a cell to what is stored, in the order
 // of finish_cell (the rounding stream of the cell and step), and hands each to
 // put(i, value).

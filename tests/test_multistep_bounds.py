@@ -1,7 +1,8 @@
 """Index arithmetic of the kernels that take several steps per launch, replayed
 on the host: the tile kernel's shared-memory slots (every slot read was written
 by the step before, every access inside the block's allocation, every core cell
-left once), for ragged sizes and the smallest lattices."""
+left once), for ragged sizes and the smallest lattices; and the offsets of the
+sweeps that take two cells per thread."""
 import pytest
 
 C = [(0, 0), (1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1)]
@@ -72,3 +73,87 @@ def tile_replay(nx, ny, W, H, T, stefan):
     (100, 4, 8, 4, 7, True), (17, 2, 8, 2, 16, True), (40, 8, 16, 8, 4, True), (9, 5, 8, 5, 3, True)])
 def test_tile_slots(nx, ny, W, H, T, stefan):
     tile_replay(nx, ny, W, H, T, stefan)
+
+
+# ---- two cells per thread (PairPlace): the sweeps' offsets, element by element
+TW, RS = 128, 18 * 128
+
+
+def place(x, y, plane, ny, paired):
+    ofs = 2 * ((plane % 9) * TW + x % TW) + plane // 9 if paired else plane * TW + x % TW
+    return ((x // TW) * ny + y) * RS + ofs
+
+
+@pytest.mark.parametrize("paired", [False, True])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (3, 3), (5, 4), (64, 3), (126, 3), (127, 4), (128, 3), (129, 4),
+                                   (130, 3), (255, 3), (256, 4), (257, 3), (300, 3)])
+def test_pair_offsets(nx, ny, paired):
+    """Every load and store of a pair, as PairPlace computes it, is the element
+    that pull streaming and the push sweep's rule name; a cell's loads and stores
+    are the same elements; no element is stored by two cells; a missing second
+    cell loads padding of its own column and stores nothing."""
+    cs = 2 if paired else 1
+    stored = {}
+    for x in range(0, nx, 2):
+        lx, tile = x % TW, ny * RS
+        dL = cs * (TW - 1) - tile if lx == 0 and x > 0 else -cs
+        dR = tile - cs * (TW - 2) if lx == TW - 2 and x + 2 < nx else 2 * cs
+        left, right0, right1, has1 = x == 0, x == nx - 1, x + 1 >= nx - 1, x + 1 < nx
+        for y in range(ny):
+            p = place(x, y, 0, ny, paired)
+            bottom, top = y == 0, y == ny - 1
+            loads, stores = [set(), set()], [set(), set()]
+            for i, (cx, cy) in enumerate(C):
+                slot = 2 * i * TW if paired else i * TW
+                oslot = 2 * OPP[i] * TW if paired else OPP[i] * TW
+
+                def walls(j):
+                    wcx, wcy = C[j]
+                    w = (wcy > 0 and bottom) or (wcy < 0 and top)
+                    return ((wcx > 0 and left) or (wcx < 0 and right0) or w,
+                            not has1 or (wcx < 0 and right1) or w)
+
+                # pull
+                w0, w1 = walls(i)
+                src = slot - cy * RS
+                o0 = oslot if w0 else src + (dL if cx > 0 else cs if cx < 0 else 0)
+                o1 = oslot + cs if w1 else src + (0 if cx > 0 else dR if cx < 0 else cs)
+                if not (bottom or top):  # the side path's selects
+                    if cx == 0:
+                        s0, s1 = src, src + cs
+                    elif cx > 0:
+                        s0, s1 = oslot if left else src + dL, src if has1 else oslot + cs
+                    else:
+                        s0, s1 = oslot if right0 else src + cs, oslot + cs if right1 else src + dR
+                    assert s0 == o0 and (s1 == o1 or (not has1 and cx == 0))
+                    o1 = s1
+                for c, o in ((0, o0), (1, o1)):
+                    if c and not has1:
+                        # padding of the same column (cx = 0: of the row the direction comes from)
+                        assert any(p + o == place(x + 1, yy, q, ny, paired)
+                                   for yy in (y, y - cy) for q in (i, OPP[i]))
+                        continue
+                    sx, sy = x + c - cx, y - cy
+                    inside = 0 <= sx < nx and 0 <= sy < ny
+                    want = place(sx, sy, i, ny, paired) if inside else place(x + c, y, OPP[i], ny, paired)
+                    assert p + o == want, (nx, ny, x + c, y, i)
+                    loads[c].add(want)
+                # push
+                w0, w1 = walls(OPP[i])
+                out = oslot + cy * RS
+                t0 = slot if w0 else out + (cs if cx > 0 else dL if cx < 0 else 0)
+                t1 = slot + cs if w1 else out + (dR if cx > 0 else 0 if cx < 0 else cs)
+                if not (bottom or top) and cx != 0:
+                    t0 = (slot if right0 else out + cs) if cx > 0 else (slot if left else out + dL)
+                    t1 = slot + cs if cx > 0 and right1 else out + (dR if cx > 0 else 0)
+                for c, o in ((0, t0), (1, t1)):
+                    if c and not has1:
+                        continue
+                    tx, ty = x + c + cx, y + cy
+                    inside = 0 <= tx < nx and 0 <= ty < ny
+                    want = place(tx, ty, OPP[i], ny, paired) if inside else place(x + c, y, i, ny, paired)
+                    assert p + o == want, (nx, ny, x + c, y, i)
+                    stores[c].add(want)
+                    assert want not in stored
+                    stored[want] = 1
+            assert loads[0] == stores[0] and loads[1] == stores[1]
