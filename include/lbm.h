@@ -201,9 +201,10 @@ int lbm_set_launch(lbm_handle h, int rows_per_block, int prefetch_rows, int grap
  * storage up to 2^19 cells, FP64 without flow up to 2^14; a Stefan lattice up to
  * 32 rows high) advance several steps per launch, each block keeping its part of
  * the lattice in shared memory for up to 16 steps and computing its neighbours'
- * edge cells itself (256 x 128 FP32: 5.4 -> 1.7 us per step); a call's last
- * step and the diagnostic steps are sweeps.  Calling this, with either mode, asks
- * for one sweep per step.
+ * edge cells itself (256 x 128 FP32: 5.4 -> 1.7 us per step); larger FP32
+ * cavities with flow take two steps per pass over memory (2048 x 1024: 35.9 ->
+ * 26.4).  A call's last step and the diagnostic steps are sweeps.  Calling this,
+ * with either mode, asks for one sweep per step.
  * Otherwise the default is one buffer (2048 x 1024 cavity on GB300: FP32
  * 41.4 -> 36.6 us per step, BF16-SR 26.1 -> 24.4 us), except for LBM_FP64,
  * which is bound by its arithmetic and keeps two buffers.  Takes effect at the

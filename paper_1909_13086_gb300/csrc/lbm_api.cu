@@ -88,6 +88,7 @@ struct lbm_s {
     int phase = 0;
     bool streaming_chosen = false;  // by lbm_set_streaming: one sweep per step, as asked
     int tile_w = 0, tile_h = 0, tile_t = 0;  // several steps per launch (tile_plan); tile_t = 0: off
+    int band_strips = 0, band_bands = 0, band_threads = 0, band_prefetch = 0;  // two steps per launch (band_plan); 0: off
     double *qgroup = nullptr;
     long long step = 0;
     long long diag_every = 0;
@@ -285,6 +286,45 @@ TileArgs tile_args(const lbm_s *h, int T) {
     return tl;
 }
 
+// Strips and bands of the band kernel for this lattice, or none: FP32 cavities with
+// flow above the tile kernel's sizes.  16-bit storage halves the bytes and stays in
+// L2, and the sweep is faster (2048 x 1024 FP16-SR, sweep and bands: 21.2 and 24.8
+// us per step; FP32 36.4 and 26.4; 1500 x 700 FP32 16.3 and 14.3).  The narrowest
+// waste of columns decides the strip, one wave of resident blocks the bands.
+void band_plan(lbm_s *h) {
+    h->band_strips = 0;
+    if (h->tile_t > 0 || h->precision != LBM_FP32 || h->p.problem != LBM_CAVITY || !h->p.flow_on) return;
+    double best = 0.0;
+    const int pairs = (h->nx + 1) / 2;
+    for (int threads = 32; threads <= kBandThreads; threads += 32) {
+        int s = 1;  // strips whose column pairs and halo pairs fit
+        while ((pairs + s - 1) / s + std::min(s - 1, 2) > threads) ++s;
+        const double used = (double)pairs / ((double)s * threads);
+        if (s <= kBandMaxStrips && used > best) {
+            best = used;
+            h->band_strips = s;
+            h->band_threads = threads;
+        }
+    }
+    if (!h->band_strips) return;
+    const int resident = kBandBlocks * (kBandThreads / h->band_threads);
+    h->band_bands = std::max(1, std::min(h->num_sms * resident / h->band_strips, h->ny / 4));
+    h->band_prefetch = 0;
+}
+
+bool use_bands(const lbm_s *h) { return h->band_strips > 0 && !h->streaming_chosen && !use_staged(h); }
+
+BandArgs band_args(const lbm_s *h) {
+    BandArgs b{};
+    b.strips = h->band_strips;
+    b.bands = h->band_bands;
+    b.threads = h->band_threads;
+    b.prefetch = h->band_prefetch;
+    b.smem = (unsigned)(4 * 6 * 2 * h->band_threads * 2 * h->esize);  // rows, directions, columns, f and g
+    b.qgroup = h->qgroup;
+    return b;
+}
+
 double *staging(lbm_s *h) {
     if (!h->stage)
         h->stage = static_cast<double *>(dev_alloc(h, (size_t)kPlanes * h->nx * h->ny * sizeof(double)));
@@ -448,6 +488,23 @@ int launch_tiles(lbm_s *h, int T) {
     return LBM_OK;
 }
 
+// Two steps of a large cavity in one launch (band.cuh); buffers and parity as in
+// launch_tiles.
+template <typename real, typename S>
+int launch_bands(lbm_s *h) {
+    if constexpr (!std::is_same<S, float>::value) {
+        return set_err(h, LBM_ERR_STATE, "the band kernel takes FP32 storage");
+    } else {
+        SweepArgs<real> a = make_args<real>(h, h->buf[h->cur], h->buf[h->cur ^ 1]);
+        cudaError_t e = launch_band<S>(a, band_args(h), h->stream);
+        if (e != cudaSuccess) return set_err(h, LBM_ERR_CUDA, "band launch failed: %s", cudaGetErrorString(e));
+        h->cur ^= 1;
+        h->has_prev = false;
+        h->step += 2;
+        return LBM_OK;
+    }
+}
+
 // len sweeps, the last one diagnostic if diag: one launch each, or, on small
 // lattices, several steps per launch -- evenly many, up to the plan's -- and the
 // diagnostic one by itself.
@@ -460,6 +517,13 @@ int launch_sweeps(lbm_s *h, long long len, bool diag, bool one_buffer) {
             const int T = (int)(plain * (k + 1) / n - plain * k / n);
             rc = T == 1 ? launch_one<real, S>(h, false) : launch_tiles<real, S>(h, T);
         }
+        if (diag && rc == LBM_OK) rc = launch_one<real, S>(h, true);
+        return rc;
+    }
+    if (use_bands(h)) {
+        const long long plain = diag ? len - 1 : len;
+        for (long long k = 0; k < plain / 2 && rc == LBM_OK; ++k) rc = launch_bands<real, S>(h);
+        if ((plain & 1) && rc == LBM_OK) rc = launch_one<real, S>(h, false);
         if (diag && rc == LBM_OK) rc = launch_one<real, S>(h, true);
         return rc;
     }
@@ -568,7 +632,7 @@ int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
 template <typename real, typename S>
 int enqueue_steps(lbm_s *h, long long n) {
     long long aa = 0;
-    if (h->streaming == LBM_STREAM_ONE_BUFFER && !use_staged(h) && !use_tiles(h) && n >= 3)
+    if (h->streaming == LBM_STREAM_ONE_BUFFER && !use_staged(h) && !use_tiles(h) && !use_bands(h) && n >= 3)
         aa = (n & 1) ? n - 1 : n - 2;
     for (long long done = 0; done < aa;) {
         long long len = aa - done;
@@ -737,7 +801,8 @@ int lbm_create(int nx, int ny, int precision, void *cuda_stream, lbm_handle *out
     const size_t nred = (nblk + 1023) / 1024;
     const size_t o_rec = 256, o_q = o_rec + up(sizeof(DevRecord)), o_d = o_q + up(nqmax * 8),
                  o_d2 = o_d + up(nblk * 32), o_g = o_d2 + up(nred * 32),
-                 bytes = o_g + (nx <= kTileMaxNx ? (size_t)kTileMaxSteps * ((nx + 127) / 128 * 4) * 8 : 0);
+                 bytes = o_g + (nx <= kTileMaxNx ? (size_t)kTileMaxSteps * ((nx + 127) / 128 * 4)
+                                                 : (size_t)2 * kBandMaxStrips) * 8;
     h->scratch = dev_alloc(h, bytes);
     if (!h->scratch) {
         lbm_destroy(h);
@@ -781,6 +846,7 @@ int lbm_set_params(lbm_handle h, const lbm_params *p) {
     }
     set_grid(h);
     tile_plan(h);
+    band_plan(h);
     h->step = 0;
     h->cur = 0;
     h->phase = 0;  // a call cut short mid-way through its one-buffer sweeps may have left 1

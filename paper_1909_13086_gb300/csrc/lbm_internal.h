@@ -136,6 +136,19 @@ struct TileArgs {
     double *qgroup;        // device scratch: T x (heated groups of 32 wall cells)
 };
 
+// Two steps of a large cavity per pass over memory (band.cuh): one block per
+// strip of columns and band of rows.
+constexpr int kBandThreads = 64;  // block size limit; two columns a thread
+constexpr int kBandBlocks = 6;     // blocks per SM: 160 registers a thread, no spills
+constexpr int kBandMaxStrips = 1024;
+struct BandArgs {
+    int strips, bands;
+    int threads;     // one per two columns of the widest strip and its halo pairs
+    int prefetch;    // L2 prefetch distance in rows
+    unsigned smem;
+    double *qgroup;  // device scratch: 2 x strips
+};
+
 // Launchers, instantiated in sweep_fp32.cu / sweep_fp64.cu / sweep_f16.cu /
 // sweep_bf16.cu for (compute real, storage codec S) = (float, float),
 // (double, double), (float, F16<SR>), (float, BF16<SR>), SR = round to
@@ -150,6 +163,8 @@ struct BF16;
 template <typename real, typename S>
 cudaError_t launch_lattice(const SweepArgs<real> &a, int problem, bool flow, int mode,
                            dim3 grid, dim3 block, cudaStream_t s, bool pdl, int streaming = kPull);
+template <typename S>
+cudaError_t launch_band(const SweepArgs<float> &a, const BandArgs &b, cudaStream_t s);
 template <typename real, typename S>
 cudaError_t launch_tile(const SweepArgs<real> &a, const TileArgs &tl, int problem, bool flow, cudaStream_t s);
 template <typename real, typename S>

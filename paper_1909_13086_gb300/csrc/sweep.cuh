@@ -1244,6 +1244,13 @@ struct Two {
     __device__ static void store_at(typename Store<S>::elem *d, int o, T v, bool second) {
         *reinterpret_cast<uint32_t *>(d + o) = second ? v.y : v.x;
     }
+    // the band kernel's ring (band.cuh): p at the direction's plane of a row, c a
+    // column; planes `plane` words long
+    static constexpr int kPlanes = 1;
+    __device__ static void put(uint32_t *p, int c, int, T v) { *reinterpret_cast<uint2 *>(p + c) = v; }
+    __device__ static T take(const uint32_t *p, int c, const uint32_t *q, int d, int) {
+        return make_uint2(p[c], q[d]);
+    }
 };
 template <>
 struct Two<float> {
@@ -1266,6 +1273,15 @@ struct Two<float> {
     __device__ static void store_at(float *d, int o, const T &v, bool second) {
         d[o] = second ? v.f.y : v.f.x;
         d[o + 9 * kTW] = second ? v.g.y : v.g.x;
+    }
+    static constexpr int kPlanes = 2;
+    __device__ static void put(uint32_t *p, int c, int plane, const T &v) {
+        *reinterpret_cast<float2 *>(p + c) = v.f;
+        *reinterpret_cast<float2 *>(p + plane + c) = v.g;
+    }
+    __device__ static T take(const uint32_t *p, int c, const uint32_t *q, int d, int plane) {
+        return {make_float2(__uint_as_float(p[c]), __uint_as_float(q[d])),
+                make_float2(__uint_as_float(p[plane + c]), __uint_as_float(q[plane + d]))};
     }
 };
 

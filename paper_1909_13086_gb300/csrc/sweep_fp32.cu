@@ -1,7 +1,8 @@
 // FP32 storage and arithmetic instantiation of the fused sweep.
-#include "tile.cuh"
+#include "band.cuh"
 
 namespace btrirt {
 BTRIRT_INSTANTIATE(float, float)
 BTRIRT_INSTANTIATE_TILE(float, float)
+BTRIRT_INSTANTIATE_BAND(float)
 }  // namespace btrirt

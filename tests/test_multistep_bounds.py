@@ -1,8 +1,9 @@
 """Index arithmetic of the kernels that take several steps per launch, replayed
 on the host: the tile kernel's shared-memory slots (every slot read was written
 by the step before, every access inside the block's allocation, every core cell
-left once), for ragged sizes and the smallest lattices; and the offsets of the
-sweeps that take two cells per thread."""
+left once) and the band kernel's ring of rows (the three rows a step-2 row needs
+are still in the ring, neighbours inside the block, every cell left once), for
+ragged sizes, the smallest lattices and both marching directions."""
 import pytest
 
 C = [(0, 0), (1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1)]
@@ -73,6 +74,60 @@ def tile_replay(nx, ny, W, H, T, stefan):
     (100, 4, 8, 4, 7, True), (17, 2, 8, 2, 16, True), (40, 8, 16, 8, 4, True), (9, 5, 8, 5, 3, True)])
 def test_tile_slots(nx, ny, W, H, T, stefan):
     tile_replay(nx, ny, W, H, T, stefan)
+
+
+def band_replay(nx, ny, strips, bands, threads, up):
+    left = set()
+    pairs = (nx + 1) // 2
+    for s in range(strips):
+        xs, xe = 2 * (s * pairs // strips), min(nx, 2 * ((s + 1) * pairs // strips))
+        x_first, x_end = max(0, xs - 2), min(nx, xe + 2)
+        assert (x_end - x_first + 1) // 2 <= threads
+        for b in range(bands):
+            ya, yb = b * ny // bands, (b + 1) * ny // bands
+            r0, r1 = max(0, ya - 1), min(ny, yb + 1)
+            rows = r1 - r0
+            last = rows if (yb == ny if up else ya == 0) else rows - 1
+            ring = {}
+            for k in range(last + 1):
+                y = r0 + k if up else r1 - 1 - k
+                if k < rows:
+                    assert 0 <= y < ny
+                    ring[k & 3] = y
+                    # global loads of the row: within the tiles' rows, a pair in one tile
+                    for x in range(x_first, x_end, 2):
+                        assert x // 128 == (x + 1) // 128
+                        for j in (0, 1):
+                            for cx, cy in C:
+                                sx, sy = x + j - cx, y - cy
+                                wall = (cx > 0 and x + j == 0) or (cx < 0 and x + j >= nx - 1)
+                                wall |= (cy > 0 and y == 0) or (cy < 0 and y == ny - 1)
+                                if not wall:
+                                    assert 0 <= sx < -(-nx // 128) * 128 and 0 <= sy < ny
+                r = y - 1 if up else y + 1
+                if not ya <= r < yb:
+                    continue
+                assert ring[(k - 1) & 3] == r
+                for x in range(xs, xe):
+                    for cx, cy in C:
+                        sx, sy = x - cx, r - cy
+                        if not (0 <= sx < nx and 0 <= sy < ny):
+                            continue  # a wall: the cell's own slots
+                        assert x_first <= sx < x_end
+                        newer = (cy < 0) == up
+                        want = (k - 1) if cy == 0 else (k if newer else k - 2)
+                        assert ring[want & 3] == sy
+                    assert (x, r) not in left
+                    left.add((x, r))
+    assert len(left) == nx * ny
+
+
+@pytest.mark.parametrize("up", [True, False])
+@pytest.mark.parametrize("nx,ny,strips,bands,threads", [
+    (2, 2, 1, 1, 32), (2, 9, 1, 2, 32), (300, 37, 2, 9, 96), (257, 12, 3, 3, 64), (63, 31, 1, 7, 32),
+    (129, 8, 2, 1, 64), (250, 5, 4, 1, 64), (125, 6, 2, 2, 64)])
+def test_band_ring(nx, ny, strips, bands, threads, up):
+    band_replay(nx, ny, strips, bands, threads, up)
 
 
 # ---- two cells per thread (PairPlace): the sweeps' offsets, element by element
