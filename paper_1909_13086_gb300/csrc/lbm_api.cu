@@ -359,6 +359,7 @@ SweepArgs<real> make_args(const lbm_s *h, const void *src, void *dst) {
     a.a0f = real(1) - a.k0f;
     a.s1 = std::fma(real(-0.5), a.k1f, real(1));
     a.s2 = std::fma(real(-0.5), a.k2f, real(1));
+    a.unit = a.a0 == real(0) && (!h->p.flow_on || a.a0f == real(0));
     a.strip_on = h->strip_on;
     a.lo2 = h->lo2;
     a.hi2 = h->hi2;

@@ -86,9 +86,10 @@ struct alignas(16) SweepArgs {
     real k0f, k1f, k2f;    // f rates
     real Lh, gbeta;        // latent heat, g*beta
     real inv_Lh;           // 1 / Lh
-    // combinations of the rates in the working precision, for the FP32 collision:
+    // combinations of the rates in the working precision, for the collisions:
     // k1 - k0, k2 - k0, k1f - k0f, k2f - k0f, 1 - k0, 1 - k0f, 1 - k1f/2, 1 - k2f/2
     real d1, d2, e1, e2, a0, a0f, s1, s2;
+    int unit;              // k0 = 1, and k0f = 1 with flow: a0 = a0f = 0
     int strip_on;          // cavity: 1 if the heated segment is non-empty
     int lo2, hi2;          // cavity: crossing heated iff lo2 <= 2x + 1 - c_ix <= hi2
     // heated-wall inflow reduction (every sweep)

@@ -270,17 +270,42 @@ __device__ __forceinline__ uint32_t lcg_next32(uint32_t &s) {
 }
 
 // ---- H -> (T, f_l): H_s = C_p T_m = 0, H_l = H_s + L.
-template <typename real>
-__device__ __forceinline__ void invert(real H, real Lh, real inv_Lh, real &T, real &fl) {
+__device__ __forceinline__ void invert(float H, float Lh, float inv_Lh, float &T, float &fl) {
     // selects, no branches; a NaN H gives T = 0, f_l = NaN
-    T = H <= real(0) ? H : max(H - Lh, real(0));
-    fl = H <= real(0) ? real(0) : (H >= Lh ? real(1) : H * inv_Lh);
+    T = H <= 0.0f ? H : fmaxf(H - Lh, 0.0f);
+    fl = H <= 0.0f ? 0.0f : (H >= Lh ? 1.0f : H * inv_Lh);
+}
+// FP64: H is compared as an integer (for non-negative doubles the same order), so
+// that the narrow FP64 pipe gets one operation, not four.
+__device__ __forceinline__ void invert(double H, double Lh, double inv_Lh, double &T, double &fl) {
+    const long long h = __double_as_longlong(H), inf = 0x7ff0000000000000ll;
+    const bool nan = (h & 0x7fffffffffffffffll) > inf;
+    if (h <= 0 && !nan) {  // negative or zero
+        T = H;
+        fl = 0.0;
+    } else if (h >= __double_as_longlong(Lh) && !nan) {
+        T = H - Lh;
+        fl = 1.0;
+    } else {
+        T = 0.0;
+        fl = H * inv_Lh;
+    }
 }
 
 // 1 / x: the fast reciprocal in FP32 (about 2 ulp; the FP32 path's tolerance
-// is 1e-5), the exact quotient in FP64 (the parity path).
+// is 1e-5); in FP64 two Newton steps y <- y + y (1 - x y) from the hardware's
+// approximation (2^-20 or better, so the second leaves rounding error only), four
+// operations of the FP64 pipe against the exact quotient's eight or more, which
+// zeros, subnormals, infinities and NaN still take.
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__device__ __forceinline__ double recip(double x) {
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    if (e - 2u > 0x7fbu) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
 
 // p_i <- a p_i + w_i [B0 + 3 c_i.B1 + 9/2 Q_i:B2]  for all nine directions.
 // With X = B2xx, Y = B2yy, Z = B2xy, S = X + Y and Q_i = c_i c_i - I/3, the
@@ -290,15 +315,15 @@ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 // rounded weights sum to 1 + 7.45e-9, which would add k0 B0 7.45e-9 to every
 // cell's sum each step (a steady growth of the FP32 density); the rest weight's
 // share is therefore taken as B0 - 4 (w1 B0 + w5 B0), so that the shares sum
-// to B0 up to rounding.  FP64's weights sum to 1 within 1e-16 and keep w0 B0.
+// to B0 up to rounding.  (FP64: emit_wide; its weights sum to 1 within 1e-16.)
 template <typename real>
 __device__ __forceinline__ void emit(real p[9], real a, real B0, real B1x, real B1y, real B2xx,
                                      real B2xy, real B2yy) {
     const real third = real(1) / real(3), sixth = real(1) / real(6), twelfth = real(1) / real(12);
-    const real w0 = real(4) / real(9), w1 = real(1) / real(9), w5 = real(1) / real(36);
+    const real w1 = real(1) / real(9), w5 = real(1) / real(36);
     const real S = B2xx + B2yy;
     const real W1 = w1 * B0, W5 = w5 * B0;
-    const real W0 = sizeof(real) == 4 ? B0 - real(4) * (W1 + W5) : w0 * B0;
+    const real W0 = B0 - real(4) * (W1 + W5);
     p[0] = a * p[0] + (W0 - (real(2) / real(3)) * S);
     const real e13 = W1 + third * B2xx - sixth * B2yy, t1 = third * B1x;
     p[1] = a * p[1] + (e13 + t1);
@@ -506,6 +531,100 @@ __device__ __forceinline__ MacroTwo cell_update_two(const SweepArgs<float> &a, f
     return {H, fl, rho, ux, uy};
 }
 
+// ---- FP64: the collision in as few operations as it takes ----
+// GB300 does two FP64 operations per clock and SM, and nothing else bounds this
+// path, so the block operator is written for their number: sums shared between the
+// moments, products of rates formed on the host, u's division folded into
+// rho u = f_l (j + F/2), and with k0 = k0f = 1 (the default rates: a = 1 - k0 = 0)
+// no term in the old populations: about 150 FP64 instructions a cell with flow, 130
+// with unit rates, against 174.  On GB300, unit rates: 2048 x 1024 713 -> 500 us per
+// step, 1024 x 4 Stefan 3.6 -> 2.9.
+__device__ __forceinline__ void moments_wide(const double p[9], double &s, double &jx, double &jy, double &xx,
+                                             double &xy, double &yy) {
+    const double s57 = p[5] + p[7], s68 = p[6] + p[8], d57 = p[5] - p[7], d68 = p[6] - p[8], d = s57 + s68;
+    xx = (p[1] + p[3]) + d;
+    const double s24 = p[2] + p[4];
+    yy = s24 + d;
+    xy = s57 - s68;
+    s = p[0] + (xx + s24);
+    jx = (p[1] - p[3]) + (d57 - d68);
+    jy = (p[2] - p[4]) + (d57 + d68);
+}
+template <bool UNIT>
+__device__ __forceinline__ void emit_wide(double p[9], double a, double B0, double B1x, double B1y, double B2xx,
+                                          double B2xy, double B2yy) {
+    const double third = 1.0 / 3.0, sixth = 1.0 / 6.0, twelfth = 1.0 / 12.0;
+    const double S = B2xx + B2yy, W1 = B0 * (1.0 / 9.0);
+    auto put = [&](int i, double v) { p[i] = UNIT ? v : fma(a, p[i], v); };
+    put(0, fma(-2.0 / 3.0, S, B0 * (4.0 / 9.0)));
+    const double e13 = fma(-sixth, B2yy, fma(third, B2xx, W1));
+    put(1, fma(third, B1x, e13));
+    put(3, fma(-third, B1x, e13));
+    const double e24 = fma(-sixth, B2xx, fma(third, B2yy, W1));
+    put(2, fma(third, B1y, e24));
+    put(4, fma(-third, B1y, e24));
+    const double e5 = fma(twelfth, S, B0 * (1.0 / 36.0));
+    const double e57 = fma(0.25, B2xy, e5), s5 = B1x + B1y;
+    put(5, fma(twelfth, s5, e57));
+    put(7, fma(-twelfth, s5, e57));
+    const double e68 = fma(-0.25, B2xy, e5), s6 = B1y - B1x;
+    put(6, fma(twelfth, s6, e68));
+    put(8, fma(-twelfth, s6, e68));
+}
+template <bool FLOW, bool UNIT, bool COLLIDE>
+__device__ __forceinline__ Macro<double> collide_wide(const SweepArgs<double> &a, double f[9], double g[9]) {
+    const double third = 1.0 / 3.0;
+    Macro<double> m;
+    double gjx, gjy, gxx, gxy, gyy;
+    moments_wide(g, m.H, gjx, gjy, gxx, gxy, gyy);
+    invert(m.H, a.Lh, a.inv_Lh, m.T, m.fl);
+    m.rho = 1.0;
+    m.ux = m.uy = 0.0;
+    double jx = 0.0, jy = 0.0, xx = 0.0, xy = 0.0, yy = 0.0, Fy = 0.0, rux = 0.0, ruy = 0.0;
+    if constexpr (FLOW) {
+        moments_wide(f, m.rho, jx, jy, xx, xy, yy);
+        const double iu = recip(m.rho);
+        Fy = a.gbeta * m.T;
+        rux = m.fl * jx;  // rho u
+        ruy = m.fl * fma(0.5, Fy, jy);
+        m.ux = rux * iu;
+        m.uy = ruy * iu;
+    }
+    if (!COLLIDE) return m;
+    // g: B1 = k1 T u - (k1 - k0) j, B2 = (k2 - k0) (T/3 I - Pi)
+    const double T = m.T, k0T = UNIT ? T : a.k0 * T;
+    double B1x, B1y;
+    if constexpr (FLOW) {
+        const double k1T = a.k1 * T;
+        B1x = fma(k1T, m.ux, -(a.d1 * gjx));
+        B1y = fma(k1T, m.uy, -(a.d1 * gjy));
+    } else {
+        B1x = -a.d1 * gjx;
+        B1y = -a.d1 * gjy;
+    }
+    emit_wide<UNIT>(g, a.a0, k0T, B1x, B1y, -a.d2 * fma(-third, T, gxx), -a.d2 * gxy, -a.d2 * fma(-third, T, gyy));
+    g[0] = UNIT ? g[0] + (m.H - T) : fma(a.k0, m.H - T, g[0]);
+    if constexpr (FLOW) {
+        // f: B1 = k1 rho u - (k1 - k0) j + (1 - k1/2) F,
+        // B2 = k2 rho u u - (k2 - k0) (Pi - rho/3 I) + (1 - k2/2) (u F + F u)
+        const double sF = a.s2 * Fy, cy = fma(a.k2f, ruy, sF);
+        const double Bxx = fma(a.k2f * rux, m.ux, -(a.e2 * fma(-third, m.rho, xx)));
+        const double Bxy = fma(m.ux, cy, -(a.e2 * xy));
+        const double Byy = fma(m.uy, cy + sF, -(a.e2 * fma(-third, m.rho, yy)));
+        emit_wide<UNIT>(f, a.a0f, UNIT ? m.rho : a.k0f * m.rho, fma(a.k1f, rux, -(a.e1 * jx)),
+                        fma(a.k1f, ruy, fma(-a.e1, jy, a.s1 * Fy)), Bxx, Bxy, Byy);
+    }
+    return m;
+}
+template <bool FLOW, bool COLLIDE>
+__device__ __forceinline__ Macro<double> cell_update_wide(const SweepArgs<double> &a, double f[9], double g[9]) {
+    return a.unit ? collide_wide<FLOW, true, COLLIDE>(a, f, g) : collide_wide<FLOW, false, COLLIDE>(a, f, g);
+}
+template <bool FLOW, bool COLLIDE>
+__device__ __forceinline__ Macro<float> cell_update_wide(const SweepArgs<float> &, float *, float *) {
+    return {};  // FP64 only
+}
+
 // Steps 2-5 on one cell: macroscopic fields, then both collisions in place
 // (COLLIDE = false stops after the fields).  f and g are in stored units (see
 // ld_f); the returned fields are physical.  With the 16-bit codecs f holds
@@ -516,6 +635,7 @@ __device__ __forceinline__ MacroTwo cell_update_two(const SweepArgs<float> &a, f
 // T kG and H kG in place of T and H.
 template <typename real, typename S, bool FLOW, bool COLLIDE>
 __device__ __forceinline__ Macro<real> cell_update(const SweepArgs<real> &a, real f[9], real g[9]) {
+    if constexpr (sizeof(real) == 8) return cell_update_wide<FLOW, COLLIDE>(a, f, g);
     if constexpr (FLOW && COLLIDE && sizeof(real) == 4) return cell_update_pair<S>(a, f, g);
     constexpr bool kDev = Store<S>::kDev;
     constexpr real kF = real(Store<S>::kF), kG = real(Store<S>::kG);
@@ -548,50 +668,14 @@ __device__ __forceinline__ Macro<real> cell_update(const SweepArgs<real> &a, rea
     }
     if (!COLLIDE) return m;
 
-    const real third = real(1) / real(3);
-    // ---- g (Eq. 2 with Eq. 4)
-    {
-        real gjx, gjy, gxx, gxy, gyy;
-        raw_moments(g, gjx, gjy, gxx, gxy, gyy);
-        real T = m.T;
-        if constexpr (kG != real(1)) T = m.T * kG;
-        const real T3 = T * third;
-        const real d1 = a.k1 - a.k0, d2 = a.k2 - a.k0;
-        const real k0T = a.k0 * T;
-        const real B1x = k0T * m.ux - d1 * (gjx - T * m.ux);
-        const real B1y = k0T * m.uy - d1 * (gjy - T * m.uy);
-        emit(g, real(1) - a.k0, k0T, B1x, B1y, -d2 * (gxx - T3), -d2 * gxy, -d2 * (gyy - T3));
-        g[0] += a.k0 * (Hs - T);
-    }
-    // ---- f (same block operator, forcing folded into A1 and A2)
-    if (FLOW) {
-        const real ux = m.ux, uy = m.uy;
-        real rk = m.rho, R0 = m.rho;  // rho in stored units; the density term of B0
-        if constexpr (kDev) {
-            R0 = fs;
-            if constexpr (kF != real(1)) rk = m.rho * kF;
-        }
-        const real rux = rk * ux, ruy = rk * uy;
-        const real rxx = rux * ux, rxy = rux * uy, ryy = ruy * uy, r3 = R0 * third;
-        const real d1 = a.k1f - a.k0f, d2 = a.k2f - a.k0f;
-        const real s1 = real(1) - real(0.5) * a.k1f, s2 = real(1) - real(0.5) * a.k2f;
-        const real A1x = d1 * (fjx - rux);
-        const real A1y = d1 * (fjy - ruy) - s1 * Fk;
-        const real A2xx = d2 * (fxx - r3 - rxx);
-        const real A2xy = d2 * (fxy - rxy) - s2 * ux * Fk;
-        const real A2yy = d2 * (fyy - r3 - ryy) - s2 * real(2) * uy * Fk;
-        const real k0 = a.k0f;
-        emit(f, real(1) - k0, k0 * R0, k0 * rux - A1x, k0 * ruy - A1y, k0 * rxx - A2xx,
-             k0 * rxy - A2xy, k0 * ryy - A2yy);
-        // FP32 storage: the collision conserves mass, sum f*_i = sum f_i, and
-        // the rest population is taken from that invariant, so that the
-        // rounding of the nine emitted values leaves no drift in the density
-        // (other rounding biases of the emitted values add ~4e-9 per step in
-        // a convecting cavity).  16-bit storage rounds f*_i stochastically on
-        // store, which is unbiased.
-        if constexpr (!kDev && sizeof(real) == 4)
-            f[0] = fs - (((f[1] + f[2]) + (f[3] + f[4])) + ((f[5] + f[6]) + (f[7] + f[8])));
-    }
+    // ---- g without flow (Eq. 2 with Eq. 4, u = 0)
+    real gjx, gjy, gxx, gxy, gyy;
+    raw_moments(g, gjx, gjy, gxx, gxy, gyy);
+    real T = m.T;
+    if constexpr (kG != real(1)) T = m.T * kG;
+    const real T3 = T * (real(1) / real(3));
+    emit(g, a.a0, a.k0 * T, -a.d1 * gjx, -a.d1 * gjy, -a.d2 * (gxx - T3), -a.d2 * gxy, -a.d2 * (gyy - T3));
+    g[0] += a.k0 * (Hs - T);
     return m;
 }
 
