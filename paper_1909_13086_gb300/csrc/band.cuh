@@ -74,12 +74,6 @@ __device__ __forceinline__ void band_block(const SweepArgs<float> &a, const Band
         uint32_t *const rn = ring + (k & 3) * ring_row;
         T v0{}, v2{}, v4{};
         if (k < rows) {
-            if (b.prefetch > 0 && (int)threadIdx.x < 4) {
-                // the tiles that begin in this core: the row `prefetch` rows on
-                const int yp = up ? y + b.prefetch : y - b.prefetch, tile = (xs + kTW - 1) / kTW + (int)threadIdx.x;
-                if (tile * kTW < xe && yp >= max(0, r0 - 1) && yp < min(a.ny, r1 + 1))
-                    prefetch_tile_row_l2(src + cell_index<S>(tile * kTW, yp, 0, a.ny));
-            }
             if (active) {
                 float2 f[9], g[9];
 #pragma unroll
@@ -172,7 +166,7 @@ __device__ __forceinline__ void band_block(const SweepArgs<float> &a, const Band
 }
 
 template <typename S>
-__global__ void __launch_bounds__(kBandThreads, kBandBlocks)
+__global__ void __launch_bounds__(kBandThreads, kBandWarps / (kBandThreads / 32))
     band_kernel(const SweepArgs<float> a, const BandArgs b) {
     extern __shared__ __align__(16) unsigned char band_sm[];
     pdl_launch_dependents();
@@ -184,19 +178,41 @@ template <typename S>
 cudaError_t launch_band(const SweepArgs<float> &a, const BandArgs &b, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(band_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b.smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(b.strips, b.bands);
-    cfg.blockDim = dim3(b.threads);
-    cfg.dynamicSmemBytes = b.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, band_kernel<S>, a, b);
+    return launch_shared(band_kernel<S>, dim3(b.strips, b.bands), dim3(b.threads), b.smem, s, a, b);
 }
 
+template <typename S>
+__global__ void __launch_bounds__(kBandThreads, kBandWarps / (kBandThreads / 32))
+    batch_band_kernel(const BatchEntry<float> *entries, const int *mstarts, const int *parity, int n, int j,
+                      const BandArgs common) {
+    extern __shared__ __align__(16) unsigned char band_sm[];
+    __shared__ __align__(16) unsigned char entry_sh[sizeof(BatchEntry<float>)];
+    pdl_launch_dependents();
+    int r;
+    const BatchEntry<float> &e = batch_entry(entries, mstarts, n, entry_sh, r);
+    const int l = (int)blockIdx.x - e.mstart;
+    BandArgs b = common;
+    b.strips = e.mx;
+    b.bands = e.my;
+    b.qgroup = e.qgroup;
+    const int p = __ldg(parity + r) ^ (j & 1);
+    pdl_wait();
+    band_block<S>(e.a[p], b, l % b.strips, l / b.strips, band_sm);
+}
+
+template <typename S>
+cudaError_t launch_batch_band(const void *entries, const int *mstarts, const int *parity, int n, int nblocks, int j,
+                              const BandArgs &b, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(batch_band_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)b.smem);
+    if (e != cudaSuccess) return e;
+    return launch_shared(batch_band_kernel<S>, dim3(nblocks), dim3(b.threads), b.smem, s,
+                         static_cast<const BatchEntry<float> *>(entries), mstarts, parity, n, j, b);
+}
+
+#define BTRIRT_INSTANTIATE_BATCH_BAND(S)                                                                         \
+    template cudaError_t launch_batch_band<S>(const void *, const int *, const int *, int, int, int,           \
+                                              const BandArgs &, cudaStream_t);
 #define BTRIRT_INSTANTIATE_BAND(S) \
     template cudaError_t launch_band<S>(const SweepArgs<float> &, const BandArgs &, cudaStream_t);
 

@@ -64,6 +64,14 @@ struct ChunkGraph {
     unsigned long long stamp = 0;
 };
 
+// Plans of the kernels that take several steps per launch (tile_plan, band_plan).
+struct TilePlan {
+    int w = 0, h = 0, t = 0;  // core and most steps; t = 0: none
+};
+struct BandPlan {
+    int threads = 0, rows = 0;  // block size and rows per band; threads = 0: none
+};
+
 }  // namespace
 
 struct lbm_s {
@@ -87,8 +95,8 @@ struct lbm_s {
     int streaming = LBM_STREAM_TWO_BUFFERS;  // set per precision by lbm_create
     int phase = 0;
     bool streaming_chosen = false;  // by lbm_set_streaming: one sweep per step, as asked
-    int tile_w = 0, tile_h = 0, tile_t = 0;  // several steps per launch (tile_plan); tile_t = 0: off
-    int band_strips = 0, band_bands = 0, band_threads = 0, band_prefetch = 0;  // two steps per launch (band_plan); 0: off
+    TilePlan tile;                  // several steps per launch (plan_steps)
+    BandPlan band;
     double *qgroup = nullptr;
     long long step = 0;
     long long diag_every = 0;
@@ -204,7 +212,10 @@ void set_grid(lbm_s *h) {
     h->snq = h->p.problem == LBM_CAVITY ? (int)h->sgrid.x : (int)h->sgrid.y;
 }
 
-// Region of the first of T steps of a core of w x h cells.
+// ---- several steps per launch: plans ----
+// A plan serves one lattice, or the members of a batch (all alike but for size).
+
+// Cells of step t of T of a core of w x hh cells.
 int tile_cells(const lbm_s *h, int w, int hh, int T, int t) {
     const int halo = 2 * (T - t);
     const int rows = h->p.problem == LBM_STEFAN ? h->ny : std::min(h->ny, hh + halo);
@@ -225,7 +236,7 @@ size_t tile_smem(const lbm_s *h, int w, int hh, int T) {
            (size_t)T * 3 * (h->p.problem == LBM_STEFAN ? hh : w) * (h->precision == LBM_FP64 ? 8 : 4);
 }
 
-// Core and steps of the tile kernel for this lattice, or none.  A launch costs
+// Core and steps of the tile kernel for these lattices, or none.  A launch costs
 // `launch` whatever it does; a step the larger of `least` (its latency) and its
 // cells' issue time on the SM that holds the most of them.  The candidate with
 // the least time per step by this model, its constants fitted to GB300 (FP32,
@@ -238,47 +249,58 @@ size_t tile_smem(const lbm_s *h, int w, int hh, int T) {
 // have paid for themselves.  FP64 with flow is bound by its pipe and gains
 // nothing from fewer launches (128 x 64: 18.9 and 18.2 us); without flow up to
 // 2^14 cells (1024 x 4 Stefan: 8.6 and 3.6).
-void tile_plan(lbm_s *h) {
-    h->tile_t = 0;
+TilePlan tile_plan(lbm_s *const *lats, size_t n) {
+    TilePlan plan;
+    const lbm_s *h = lats[0];
     const bool stefan = h->p.problem == LBM_STEFAN, fp64 = h->precision == LBM_FP64, flow = h->p.flow_on != 0;
-    const long long cells = (long long)h->nx * h->ny;
-    if (h->nx > kTileMaxNx || (stefan && h->ny > 32)) return;
-    if (cells > (fp64 ? (flow ? 0 : 1 << 14) : 1 << 19)) return;
+    long long cells = 0;
+    for (size_t r = 0; r < n; ++r) {
+        cells += (long long)lats[r]->nx * lats[r]->ny;
+        if (lats[r]->nx > kTileMaxNx || (stefan && lats[r]->ny > 32)) return plan;
+        if (n > 1 && (fp64 || stefan || !flow)) return plan;  // no batch kernel for these
+    }
+    if (cells > (fp64 ? (flow ? 0 : 1 << 14) : 1 << 19)) return plan;
     const double per_cell = fp64 ? 18.6 : (h->esize == 2 ? 1.6 : 1.5) * (flow ? 1.0 : 0.6);
     const double least = fp64 ? 2200.0 : 700.0, launch = 4500.0;
     double best = 1e30;
     for (int w = stefan ? 8 : 32; w <= 128; w *= 2)
-        for (int hh = stefan ? h->ny : 2; hh <= (stefan ? h->ny : 64); hh += hh < 16 ? 1 : 4)
+        for (int hh = stefan ? h->ny : 2; hh <= (stefan ? h->ny : 64); hh += hh < 16 ? 1 : 4) {
+            long long tiles = 0;
+            const lbm_s *big = h;  // the member whose cores are the least clipped
+            for (size_t r = 0; r < n; ++r) {
+                const lbm_s *m = lats[r];
+                tiles += (long long)((m->nx + w - 1) / w) * ((m->ny + hh - 1) / hh);
+                if ((long long)m->nx * m->ny > (long long)big->nx * big->ny) big = m;
+            }
+            const double waves = (double)((tiles + h->num_sms - 1) / h->num_sms);
             for (int T = 2; T <= kTileMaxSteps; ++T) {
                 const size_t smem = tile_smem(h, w, hh, T);
-                const int most = tile_cells(h, w, hh, T, 1);
-                if (smem > kTileSmemMax || (long long)most * std::min(h->nx, w + 2 * T) >= (1 << 20)) break;
-                const long long tiles = (long long)((h->nx + w - 1) / w) * ((h->ny + hh - 1) / hh);
-                const double waves = (double)((tiles + h->num_sms - 1) / h->num_sms);
+                if (smem > kTileSmemMax || (long long)(w + 2 * T) * (w + 2 * T) * (hh + 2 * T) >= (1 << 20)) break;
                 const double resident = std::max(1.0, std::floor(kTileSmemMax / (double)smem));
                 double ns = launch * std::ceil(waves / resident);
-                for (int t = 1; t <= T; ++t) ns += std::max(least, waves * per_cell * tile_cells(h, w, hh, T, t));
+                for (int t = 1; t <= T; ++t) ns += std::max(least, waves * per_cell * tile_cells(big, w, hh, T, t));
                 if (ns / T < best) {
                     best = ns / T;
-                    h->tile_w = w;
-                    h->tile_h = hh;
-                    h->tile_t = T;
+                    plan.w = w;
+                    plan.h = hh;
+                    plan.t = T;
                 }
             }
+        }
+    return plan;
 }
 
-bool use_tiles(const lbm_s *h) { return h->tile_t >= 2 && !h->streaming_chosen && !use_staged(h); }
-
-TileArgs tile_args(const lbm_s *h, int T) {
+// tile_plan's core for T steps of h; a batch takes what its members share from
+// one of them.
+TileArgs tile_args(const lbm_s *h, const TilePlan &plan, int T, int cells) {
     TileArgs tl{};
     tl.T = T;
-    tl.W = h->tile_w;
-    tl.H = h->tile_h;
+    tl.W = plan.w;
+    tl.H = plan.h;
     tl.tiles_x = (h->nx + tl.W - 1) / tl.W;
     tl.tiles_y = (h->ny + tl.H - 1) / tl.H;
     tl.pitch = tl.W + 2 * T;
-    const int most = h->precision == LBM_FP64 ? kTileThreads64 : kTileThreads;
-    const int cells = tile_cells(h, tl.W, tl.H, T, 1), rounds = (cells + most - 1) / most;
+    const int most = h->precision == LBM_FP64 ? kTileThreads64 : kTileThreads, rounds = (cells + most - 1) / most;
     tl.threads = std::min(most, ((cells + rounds - 1) / rounds + 31) / 32 * 32);
     tl.q_offset = (unsigned)tile_q_offset(h, tl.W, tl.H, T);
     tl.smem = (unsigned)tile_smem(h, tl.W, tl.H, T);
@@ -286,44 +308,77 @@ TileArgs tile_args(const lbm_s *h, int T) {
     return tl;
 }
 
-// Strips and bands of the band kernel for this lattice, or none: FP32 cavities with
-// flow above the tile kernel's sizes.  16-bit storage halves the bytes and stays in
-// L2, and the sweep is faster (2048 x 1024 FP16-SR, sweep and bands: 21.2 and 24.8
-// us per step; FP32 36.4 and 26.4; 1500 x 700 FP32 16.3 and 14.3).  The narrowest
-// waste of columns decides the strip, one wave of resident blocks the bands.
-void band_plan(lbm_s *h) {
-    h->band_strips = 0;
-    if (h->tile_t > 0 || h->precision != LBM_FP32 || h->p.problem != LBM_CAVITY || !h->p.flow_on) return;
-    double best = 0.0;
+// Block size and rows per band of the band kernel for these lattices: cavities
+// with flow, FP32 arithmetic.  The block that wastes the fewest lanes on ragged
+// strips and halos; the fewest rows with which one wave of blocks holds all bands
+// (a band computes two rows more than it has).
+int band_strips(const lbm_s *h, int threads) {
     const int pairs = (h->nx + 1) / 2;
+    int s = std::max(1, pairs / threads);
+    while ((pairs + s - 1) / s + std::min(s - 1, 2) > threads) ++s;
+    return s;
+}
+BandPlan band_plan(lbm_s *const *lats, size_t n) {
+    BandPlan plan;
+    if (lats[0]->precision == LBM_FP64 || lats[0]->p.problem != LBM_CAVITY || !lats[0]->p.flow_on) return plan;
+    double best = 1e300;
+    long long strips = 0;
+    int tallest = 0;
     for (int threads = 32; threads <= kBandThreads; threads += 32) {
-        int s = 1;  // strips whose column pairs and halo pairs fit
-        while ((pairs + s - 1) / s + std::min(s - 1, 2) > threads) ++s;
-        const double used = (double)pairs / ((double)s * threads);
-        if (s <= kBandMaxStrips && used > best) {
-            best = used;
-            h->band_strips = s;
-            h->band_threads = threads;
+        double lanes = 0.0;
+        long long total = 0;
+        int most = 0;
+        for (size_t r = 0; r < n; ++r) {
+            const int s = band_strips(lats[r], threads);
+            most = std::max(most, s);
+            total += s;
+            lanes += (double)s * threads * lats[r]->ny;
+            tallest = std::max(tallest, lats[r]->ny);
+        }
+        if (most <= kBandMaxStrips && lanes < best) {
+            best = lanes;
+            plan.threads = threads;
+            strips = total;
         }
     }
-    if (!h->band_strips) return;
-    const int resident = kBandBlocks * (kBandThreads / h->band_threads);
-    h->band_bands = std::max(1, std::min(h->num_sms * resident / h->band_strips, h->ny / 4));
-    h->band_prefetch = 0;
+    if (!plan.threads) return plan;
+    const long long room = (long long)lats[0]->num_sms * (kBandWarps / (plan.threads / 32));
+    if (strips > room) {  // several waves: bands of 32 rows
+        plan.rows = 32;
+        return plan;
+    }
+    for (plan.rows = 4; plan.rows < tallest; ++plan.rows) {
+        long long blocks = 0;
+        for (size_t r = 0; r < n; ++r)
+            blocks += (long long)band_strips(lats[r], plan.threads) * ((lats[r]->ny + plan.rows - 1) / plan.rows);
+        if (blocks <= room) break;
+    }
+    return plan;
 }
 
-bool use_bands(const lbm_s *h) { return h->band_strips > 0 && !h->streaming_chosen && !use_staged(h); }
-
-BandArgs band_args(const lbm_s *h) {
+BandArgs band_args(const lbm_s *h, const BandPlan &plan) {
     BandArgs b{};
-    b.strips = h->band_strips;
-    b.bands = h->band_bands;
-    b.threads = h->band_threads;
-    b.prefetch = h->band_prefetch;
-    b.smem = (unsigned)(4 * 6 * 2 * h->band_threads * 2 * h->esize);  // rows, directions, columns, f and g
+    b.strips = band_strips(h, plan.threads);
+    b.bands = (h->ny + plan.rows - 1) / plan.rows;
+    b.threads = plan.threads;
+    b.smem = (unsigned)(4 * 6 * 2 * plan.threads * 2 * h->esize);  // rows, directions, columns, f and g
     b.qgroup = h->qgroup;
     return b;
 }
+
+// Which kernel takes a lattice's plain steps: tiles for small ones, bands for FP32
+// cavities above those, else the sweeps.  16-bit storage halves the bytes and stays
+// in L2, and its sweep is faster than the bands (2048 x 1024 FP16-SR, sweep and
+// bands: 21.1 and 24.8 us per step; FP32 35.9 and 26.4; 1500 x 700 FP32 16.3 and
+// 14.3).
+void plan_steps(lbm_s *h) {
+    h->tile = tile_plan(&h, 1);
+    h->band = BandPlan();
+    if (h->tile.t == 0 && h->precision == LBM_FP32) h->band = band_plan(&h, 1);
+}
+
+bool use_tiles(const lbm_s *h) { return h->tile.t >= 2 && !h->streaming_chosen && !use_staged(h); }
+bool use_bands(const lbm_s *h) { return h->band.threads > 0 && !h->streaming_chosen && !use_staged(h); }
 
 double *staging(lbm_s *h) {
     if (!h->stage)
@@ -481,7 +536,7 @@ int launch_one_aa(lbm_s *h, bool diag) {
 template <typename real, typename S>
 int launch_tiles(lbm_s *h, int T) {
     SweepArgs<real> a = make_args<real>(h, h->buf[h->cur], h->buf[h->cur ^ 1]);
-    cudaError_t e = launch_tile<real, S>(a, tile_args(h, T), h->p.problem, h->p.flow_on != 0, h->stream);
+    cudaError_t e = launch_tile<real, S>(a, tile_args(h, h->tile, T, tile_cells(h, h->tile.w, h->tile.h, T, 1)), h->p.problem, h->p.flow_on != 0, h->stream);
     if (e != cudaSuccess) return set_err(h, LBM_ERR_CUDA, "tile launch failed: %s", cudaGetErrorString(e));
     h->cur ^= 1;
     h->has_prev = false;  // buf[cur ^ 1] is T steps old until the call's closing sweep
@@ -497,7 +552,7 @@ int launch_bands(lbm_s *h) {
         return set_err(h, LBM_ERR_STATE, "the band kernel takes FP32 storage");
     } else {
         SweepArgs<real> a = make_args<real>(h, h->buf[h->cur], h->buf[h->cur ^ 1]);
-        cudaError_t e = launch_band<S>(a, band_args(h), h->stream);
+        cudaError_t e = launch_band<S>(a, band_args(h, h->band), h->stream);
         if (e != cudaSuccess) return set_err(h, LBM_ERR_CUDA, "band launch failed: %s", cudaGetErrorString(e));
         h->cur ^= 1;
         h->has_prev = false;
@@ -513,7 +568,7 @@ template <typename real, typename S>
 int launch_sweeps(lbm_s *h, long long len, bool diag, bool one_buffer) {
     int rc = LBM_OK;
     if (use_tiles(h)) {
-        const long long plain = diag ? len - 1 : len, n = (plain + h->tile_t - 1) / h->tile_t;
+        const long long plain = diag ? len - 1 : len, n = (plain + h->tile.t - 1) / h->tile.t;
         for (long long k = 0; k < n && rc == LBM_OK; ++k) {
             const int T = (int)(plain * (k + 1) / n - plain * k / n);
             rc = T == 1 ? launch_one<real, S>(h, false) : launch_tiles<real, S>(h, T);
@@ -846,8 +901,7 @@ int lbm_set_params(lbm_handle h, const lbm_params *p) {
         h->strip_on = 0;
     }
     set_grid(h);
-    tile_plan(h);
-    band_plan(h);
+    plan_steps(h);
     h->step = 0;
     h->cur = 0;
     h->phase = 0;  // a call cut short mid-way through its one-buffer sweeps may have left 1
@@ -905,10 +959,17 @@ int lbm_read_fields(lbm_handle h, unsigned mask, double *H, double *T, double *f
     for (int k = 0; k < 6; ++k) dev[k] = ((mask >> k) & 1u) && host[k] ? stage + k * P : nullptr;
     int rc = by_precision(h->precision, [&](auto t) { return BTRIRT_T(t, enqueue_fields)(h, dev); });
     if (rc != LBM_OK) return rc;
-    for (int k = 0; k < 6; ++k)
-        if (dev[k])
-            CUDA_TRY(h, cudaMemcpyAsync(host[k], dev[k], P * sizeof(double), cudaMemcpyDeviceToHost,
+    // one copy for fields that follow one another on the host as in the staging (each
+    // copy costs ~1.7 us whatever its size: 256 x 128, all six 46 us, 37 in one)
+    for (int k = 0; k < 6;) {
+        int e = k + 1;
+        if (dev[k]) {
+            while (e < 6 && dev[e] && host[e] == host[e - 1] + P) ++e;
+            CUDA_TRY(h, cudaMemcpyAsync(host[k], dev[k], (e - k) * P * sizeof(double), cudaMemcpyDeviceToHost,
                                         h->stream));
+        }
+        k = e;
+    }
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
@@ -1211,6 +1272,11 @@ struct lbm_batch_s {
     std::vector<int> host_starts;
     std::vector<int> host_parity;
     int nblocks = 0;
+    TilePlan tile;            // several steps per launch, unless lbm_batch_set_streaming
+    BandPlan band;            // asked for sweeps
+    int *mstarts = nullptr;   // device: first block of each member in such a launch
+    std::vector<int> host_mstarts;
+    int mblocks = 0;
     int uniform = 0;          // blocks per member when all members have the same count
     int rows = 0;             // launch shape: rows per block (0: 2, or 3 with 16-bit storage),
     int prefetch = -1;        // L2 prefetch distance (-1: off),
@@ -1220,8 +1286,9 @@ struct lbm_batch_s {
     int precision = -1, problem = -1, flow = -1;
     int graph_chunk = 128;    // longest graph-replayed piece; even, so that every
                               // piece starts at an even step of the call
-    ChunkGraph graphs[kGraphCache];  // pieces as for a single lattice (parity unused:
-                                     // the members' parities are a device table)
+    ChunkGraph graphs[kGraphCache];  // pieces as for a single lattice (parity: of the
+                                     // piece's first launch within its call; the
+                                     // members' own parities are a device table)
     unsigned long long graph_clock = 0;
     cudaEvent_t ev = nullptr;
     lbm_alloc_fn alloc = nullptr;
@@ -1260,6 +1327,8 @@ void batch_drop_graph(lbm_batch_s *b) {
 template <typename real>
 size_t entry_bytes() { return sizeof(BatchEntry<real>); }
 
+bool batch_sweeps_chosen(const lbm_batch_s *b) { return b->streaming >= 0; }
+
 // Default launch shape of a batch, whatever the members' own lbm_set_launch
 // settings: 2 rows per block (3 with 16-bit storage), no L2 prefetch, blocks of a
 // one-size batch interleaved over the members -- the fastest shapes for 32 cavities
@@ -1274,7 +1343,12 @@ void batch_build(lbm_batch_s *b) {
     b->host_entries.assign(eb * b->members.size(), 0);
     b->host_starts.assign(b->members.size(), 0);
     b->uniform = 0;
-    int start = 0;
+    int start = 0, mstart = 0;
+    // several steps per launch: tiles while the members are few and small, else bands
+    b->tile = tile_plan(b->members.data(), b->members.size());
+    b->band = BandPlan();
+    if (b->tile.t == 0) b->band = band_plan(b->members.data(), b->members.size());
+    b->host_mstarts.assign(b->members.size(), 0);
     for (size_t r = 0; r < b->members.size(); ++r) {
         lbm_s *h = b->members[r];
         const int rows = b->rows > 0 ? b->rows : (h->esize == 2 ? kBatchRows16 : kBatchRows32);
@@ -1294,9 +1368,57 @@ void batch_build(lbm_batch_s *b) {
         const int nb = e.gx * e.gy;
         b->uniform = r == 0 ? nb : (b->uniform == nb ? nb : 0);
         start += e.gx * e.gy;
+        if (b->tile.t > 0) {
+            const TileArgs tl = tile_args(h, b->tile, 2, 1);
+            e.mx = tl.tiles_x;
+            e.my = tl.tiles_y;
+        } else if (b->band.threads > 0) {
+            const BandArgs ba = band_args(h, b->band);
+            e.mx = ba.strips;
+            e.my = ba.bands;
+        }
+        e.qgroup = h->qgroup;
+        e.mstart = b->host_mstarts[r] = mstart;
+        mstart += e.mx * e.my;
         std::memcpy(b->host_entries.data() + r * eb, &e, eb);
     }
     b->nblocks = start;
+    b->mblocks = mstart;
+}
+
+// Launches of a batch's piece of len steps (the last one diagnostic if diag) that
+// takes several steps per launch, from launch j of the call; returns the number of
+// the next launch, or a negative status.
+template <typename S>
+int batch_multi(lbm_batch_s *b, long long len, bool diag, int j) {
+    const int nm = (int)b->members.size();
+    cudaError_t e = cudaSuccess;
+    auto sweep = [&](bool d) {
+        e = launch_batch<float, S>(b->entries, b->starts, b->parity, nm, b->uniform, b->uniform > 0 ? b->interleave : 0,
+                                   b->nblocks, b->problem, b->flow != 0, d, j & 1, b->stream, true, kPull);
+        ++j;
+    };
+    const long long plain = diag ? len - 1 : len;
+    const int most = b->tile.t > 0 ? b->tile.t : 2;
+    const long long n = (plain + most - 1) / most;
+    for (long long k = 0; k < n && e == cudaSuccess; ++k) {
+        const int T = b->tile.t > 0 ? (int)(plain * (k + 1) / n - plain * k / n) : (int)std::min(2ll, plain - 2 * k);
+        if (T == 1) {
+            sweep(false);
+        } else if (b->tile.t > 0) {
+            int cells = 1;  // of the largest member's first step
+            for (const lbm_s *h : b->members) cells = std::max(cells, tile_cells(h, b->tile.w, b->tile.h, T, 1));
+            e = launch_batch_tile<S>(b->entries, b->mstarts, b->parity, nm, b->mblocks, j & 1,
+                                     tile_args(b->members[0], b->tile, T, cells), b->stream);
+            ++j;
+        } else {
+            e = launch_batch_band<S>(b->entries, b->mstarts, b->parity, nm, b->mblocks, j & 1,
+                                     band_args(b->members[0], b->band), b->stream);
+            ++j;
+        }
+    }
+    if (diag && e == cudaSuccess) sweep(true);
+    return e == cudaSuccess ? j : batch_err(LBM_ERR_CUDA, "batch launch failed: %s", cudaGetErrorString(e));
 }
 
 template <typename real, typename S>
@@ -1307,6 +1429,8 @@ int batch_steps(lbm_batch_s *b, long long n) {
         BATCH_TRY(cudaMemcpyAsync(b->entries, b->host_entries.data(), b->host_entries.size(),
                                   cudaMemcpyHostToDevice, b->stream));
         BATCH_TRY(cudaMemcpyAsync(b->starts, b->host_starts.data(), b->host_starts.size() * sizeof(int),
+                                  cudaMemcpyHostToDevice, b->stream));
+        BATCH_TRY(cudaMemcpyAsync(b->mstarts, b->host_mstarts.data(), b->host_mstarts.size() * sizeof(int),
                                   cudaMemcpyHostToDevice, b->stream));
         batch_drop_graph(b);
         b->dirty = false;
@@ -1329,9 +1453,19 @@ int batch_steps(lbm_batch_s *b, long long n) {
     // call, an even number, alternate push (even j) and local (odd j) sweeps
     // in each member's buffer parity[r]; the last one or two run over the two
     // buffers, so that between calls every member's state is the two-buffer one.
-    const bool one = b->streaming < 0 ? b->precision != LBM_FP64 : b->streaming == LBM_STREAM_ONE_BUFFER;
+    const bool multi = !batch_sweeps_chosen(b) && (b->tile.t > 0 || b->band.threads > 0);
+    const bool one = !multi && (b->streaming < 0 ? b->precision != LBM_FP64 : b->streaming == LBM_STREAM_ONE_BUFFER);
+    int launches = 0;  // of several-step pieces: the buffers they have changed
     const long long aa = (one && n >= 3) ? ((n & 1) ? n - 1 : n - 2) : 0;
     auto direct = [&](long long from, long long len, bool diag, bool ob) -> int {
+        if constexpr (sizeof(real) == 4) {
+            if (multi) {
+                const int rc = batch_multi<S>(b, len, diag, launches);
+                if (rc < 0) return rc;
+                launches = rc;
+                return LBM_OK;
+            }
+        }
         for (long long j = 0; j < len; ++j) {
             const long long jj = from + j;
             const int sm = ob ? ((jj & 1) ? kAALocal : kAAPush) : kPull;
@@ -1352,7 +1486,8 @@ int batch_steps(lbm_batch_s *b, long long n) {
         const bool graphs = K >= 2 && len >= 2 && len <= K && !capturing;
         if (graphs) {
             for (ChunkGraph &g : b->graphs)
-                if (g.used && g.len == len && g.diag == diag && g.one_buffer == ob) slot = &g;
+                if (g.used && g.len == len && g.diag == diag && g.one_buffer == ob && g.parity == (launches & 1))
+                    slot = &g;
             if (!slot) {
                 ChunkGraph *victim = &b->graphs[0];
                 for (ChunkGraph &g : b->graphs) {
@@ -1365,10 +1500,14 @@ int batch_steps(lbm_batch_s *b, long long n) {
                 victim->len = (int)len;
                 victim->diag = diag;
                 victim->one_buffer = ob;
+                victim->parity = launches & 1;
                 victim->stamp = ++b->graph_clock;
             } else if (!slot->exec) {
                 BATCH_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+                const int before = launches;
                 const int rc = direct(0, len, diag, ob);
+                slot->flip = (launches ^ before) & 1;
+                launches = before;
                 cudaGraph_t g = nullptr;
                 const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
                 if (rc != LBM_OK || e2 != cudaSuccess) {
@@ -1388,6 +1527,7 @@ int batch_steps(lbm_batch_s *b, long long n) {
         if (slot && slot->exec) {
             slot->stamp = ++b->graph_clock;
             BATCH_TRY(cudaGraphLaunch(slot->exec, b->stream));
+            launches += slot->flip;
             return LBM_OK;
         }
         return direct(from, len, diag, ob);
@@ -1407,7 +1547,7 @@ int batch_steps(lbm_batch_s *b, long long n) {
     }
     for (lbm_s *h : b->members) {
         h->step += n;
-        h->cur ^= (int)(n & 1);
+        h->cur ^= (int)((multi ? launches : n) & 1);
         h->has_prev = true;
     }
     return LBM_OK;
@@ -1440,7 +1580,7 @@ int lbm_batch_create(int max_lattices, void *cuda_stream, lbm_batch *out) {
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming);
     const size_t table = ((size_t)max_lattices * sizeof(BatchEntry<double>) + 255) / 256 * 256;
-    const size_t bytes = table + 2 * (size_t)max_lattices * sizeof(int);
+    const size_t bytes = table + 3 * (size_t)max_lattices * sizeof(int);
     void *mem = nullptr;
     if (e == cudaSuccess) {
         if (b->alloc) {
@@ -1457,6 +1597,7 @@ int lbm_batch_create(int max_lattices, void *cuda_stream, lbm_batch *out) {
     b->entries = mem;
     b->parity = reinterpret_cast<int *>(static_cast<char *>(mem) + table);
     b->starts = b->parity + max_lattices;
+    b->mstarts = b->starts + max_lattices;
     *out = b;
     return LBM_OK;
 }
@@ -1615,7 +1756,11 @@ extern "C" int lbm_batch_autotune(lbm_batch b, int steps_per_trial, int *rows_ou
         std::vector<lbm_handle> scratch;
         lbm_batch t = nullptr;
         int rc = lbm_batch_create((int)b->members.size(), b->stream, &t);
-        if (rc == LBM_OK) t->streaming = b->streaming;
+        // shapes of the sweeps are timed, whether or not they take the plain steps
+        if (rc == LBM_OK)
+            t->streaming = b->streaming >= 0            ? b->streaming
+                           : b->precision == LBM_FP64 ? LBM_STREAM_TWO_BUFFERS
+                                                      : LBM_STREAM_ONE_BUFFER;
         for (size_t r = 0; r < b->members.size() && rc == LBM_OK; ++r) {
             const lbm_s *h = b->members[r];
             lbm_handle s = nullptr;

@@ -139,13 +139,12 @@ struct TileArgs {
 
 // Two steps of a large cavity per pass over memory (band.cuh): one block per
 // strip of columns and band of rows.
-constexpr int kBandThreads = 64;  // block size limit; two columns a thread
-constexpr int kBandBlocks = 6;     // blocks per SM: 160 registers a thread, no spills
-constexpr int kBandMaxStrips = 1024;
+constexpr int kBandThreads = 128;  // block size limit; two columns a thread
+constexpr int kBandWarps = 12;     // per SM: up to 168 registers a thread, no spills
+constexpr int kBandMaxStrips = 2048;
 struct BandArgs {
     int strips, bands;
     int threads;     // one per two columns of the widest strip and its halo pairs
-    int prefetch;    // L2 prefetch distance in rows
     unsigned smem;
     double *qgroup;  // device scratch: 2 x strips
 };
@@ -166,6 +165,16 @@ cudaError_t launch_lattice(const SweepArgs<real> &a, int problem, bool flow, int
                            dim3 grid, dim3 block, cudaStream_t s, bool pdl, int streaming = kPull);
 template <typename S>
 cudaError_t launch_band(const SweepArgs<float> &a, const BandArgs &b, cudaStream_t s);
+// The same for every lattice of a batch (cavities with flow): tl / b hold what the
+// lattices share, the entries their tiles, or strips and bands; mstarts[r] is entry
+// r's first block of nblocks; j: the launch's number in its call, which selects the
+// buffers (parity[r] ^ (j & 1)) as for a batch's sweeps.
+template <typename S>
+cudaError_t launch_batch_tile(const void *entries, const int *mstarts, const int *parity, int n, int nblocks, int j,
+                              const TileArgs &tl, cudaStream_t s);
+template <typename S>
+cudaError_t launch_batch_band(const void *entries, const int *mstarts, const int *parity, int n, int nblocks, int j,
+                              const BandArgs &b, cudaStream_t s);
 template <typename real, typename S>
 cudaError_t launch_tile(const SweepArgs<real> &a, const TileArgs &tl, int problem, bool flow, cudaStream_t s);
 template <typename real, typename S>
@@ -181,7 +190,9 @@ struct BatchEntry {
     SweepArgs<real> a[2];  // [p]: source buffer p, destination buffer 1 - p
     int start;             // first block of this lattice in the launch
     int gx, gy;            // tile columns and row bands
-    int pad;
+    int mx, my;            // several steps per launch: tiles, or strips and bands,
+    int mstart;            // their first block,
+    double *qgroup;        // and the inflow's scratch
 };
 
 // One step of a batch: `entries` points at n device BatchEntry<real> records

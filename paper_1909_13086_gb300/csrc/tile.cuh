@@ -334,23 +334,75 @@ __global__ void __launch_bounds__(sizeof(real) == 8 ? kTileThreads64 : kTileThre
     tile_block<real, S, PROB, FLOW>(a, tl, blockIdx.x, blockIdx.y, tile_sm);
 }
 
-template <typename real, typename S, int PROB, bool FLOW>
-static cudaError_t launch_tile_k(const SweepArgs<real> &a, const TileArgs &tl, cudaStream_t s) {
-    auto *kernel = tile_kernel<real, S, PROB, FLOW>;
-    // per device and idempotent; no state is kept here
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemMax);
-    if (e != cudaSuccess) return e;
+// A launch with dynamic shared memory and programmatic serialization.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_shared(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned smem, cudaStream_t s,
+                                 Args &&...args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tl.tiles_x, tl.tiles_y);
-    cfg.blockDim = dim3(tl.threads);
-    cfg.dynamicSmemBytes = tl.smem;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a, tl);
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// The entry of a batch that this block belongs to (number r), copied into shared
+// memory (sh, of sizeof(BatchEntry<float>)); the table is written only by copies the host
+// orders before the batch's launches, so this may precede pdl_wait.
+__device__ __forceinline__ const BatchEntry<float> &batch_entry(const BatchEntry<float> *entries, const int *mstarts,
+                                                                int n, unsigned char *sh, int &r) {
+    __shared__ int found;
+    if (threadIdx.x == 0) found = batch_find(mstarts, n, blockIdx.x);
+    __syncthreads();
+    r = found;
+    const int4 *s4 = reinterpret_cast<const int4 *>(entries + r);
+    for (unsigned k = threadIdx.x; k < sizeof(BatchEntry<float>) / 16; k += blockDim.x)
+        reinterpret_cast<int4 *>(sh)[k] = __ldg(s4 + k);
+    __syncthreads();
+    return *reinterpret_cast<const BatchEntry<float> *>(sh);
+}
+
+template <typename S>
+__global__ void __launch_bounds__(kTileThreads)
+    batch_tile_kernel(const BatchEntry<float> *entries, const int *mstarts, const int *parity, int n, int j,
+                      const TileArgs common) {
+    extern __shared__ __align__(16) unsigned char tile_sm[];
+    __shared__ __align__(16) unsigned char entry_sh[sizeof(BatchEntry<float>)];
+    pdl_launch_dependents();
+    int r;
+    const BatchEntry<float> &e = batch_entry(entries, mstarts, n, entry_sh, r);
+    const int l = (int)blockIdx.x - e.mstart;
+    TileArgs tl = common;
+    tl.tiles_x = e.mx;
+    tl.tiles_y = e.my;
+    tl.qgroup = e.qgroup;
+    const int p = __ldg(parity + r) ^ (j & 1);
+    pdl_wait();
+    tile_block<float, S, kCavity, true>(e.a[p], tl, l % tl.tiles_x, l / tl.tiles_x, tile_sm);
+}
+
+template <typename S>
+cudaError_t launch_batch_tile(const void *entries, const int *mstarts, const int *parity, int n, int nblocks, int j,
+                              const TileArgs &tl, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(batch_tile_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kTileSmemMax);
+    if (e != cudaSuccess) return e;
+    return launch_shared(batch_tile_kernel<S>, dim3(nblocks), dim3(tl.threads), tl.smem, s,
+                         static_cast<const BatchEntry<float> *>(entries), mstarts, parity, n, j, tl);
+}
+
+template <typename real, typename S, int PROB, bool FLOW>
+static cudaError_t launch_tile_k(const SweepArgs<real> &a, const TileArgs &tl, cudaStream_t s) {
+    auto *kernel = tile_kernel<real, S, PROB, FLOW>;
+    // per device and idempotent; no state is kept here
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemMax);
+    if (e != cudaSuccess) return e;
+    return launch_shared(kernel, dim3(tl.tiles_x, tl.tiles_y), dim3(tl.threads), tl.smem, s, a, tl);
 }
 
 template <typename real, typename S>
@@ -360,6 +412,9 @@ cudaError_t launch_tile(const SweepArgs<real> &a, const TileArgs &tl, int proble
     return flow ? launch_tile_k<real, S, kStefan, true>(a, tl, s) : launch_tile_k<real, S, kStefan, false>(a, tl, s);
 }
 
+#define BTRIRT_INSTANTIATE_BATCH_TILE(S)                                                                         \
+    template cudaError_t launch_batch_tile<S>(const void *, const int *, const int *, int, int, int,           \
+                                              const TileArgs &, cudaStream_t);
 #define BTRIRT_INSTANTIATE_TILE(REAL, S) \
     template cudaError_t launch_tile<REAL, S>(const SweepArgs<REAL> &, const TileArgs &, int, bool, cudaStream_t);
 

@@ -377,12 +377,14 @@ class Lattice:
         return lbm_diagnostics(self.h, raise_on_diverged)
 
     def fields(self, names=FIELD_NAMES) -> dict:
-        out = {k: np.empty((self.ny, self.nx)) for k in names}
+        # side by side in the library's order: read back in one copy
+        order = [k for k in FIELD_NAMES if k in names]
+        out = dict(zip(order, np.empty((len(order), self.ny, self.nx))))
         mask = 0
         for k in names:
             mask |= FIELD_BITS[k]
         lbm_read_fields(self.h, mask, *[out.get(k) for k in FIELD_NAMES])
-        return out
+        return {k: out[k] for k in names}
 
     def populations(self):
         f = np.empty((9, self.ny, self.nx))

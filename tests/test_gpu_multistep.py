@@ -1,0 +1,102 @@
+"""Several steps per launch (tiles in shared memory, bands of two steps, their
+batch forms) against one two-buffer sweep per step, which lbm_set_streaming asks
+for: populations, diagnostics, fields and history bitwise, at sizes around the
+edges of cores, strips and bands, at step counts that leave remainders, in every
+storage type the kernels take, with rates other than 1."""
+import numpy as np
+import pytest
+
+from paper_1909_13086_gb300 import lbm, workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def stream():
+    import torch
+
+    torch.cuda.set_device(0)
+    return torch.cuda.Stream().cuda_stream
+
+
+def start(nx, ny, p, prec, stream, seed=3):
+    lat = lbm.Lattice(nx, ny, p, precision=prec, stream=stream)
+    f, g = workloads.random_populations(nx, ny, seed)
+    w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+    lat.set_populations(w * (1 + 5.0 * (f - 1 / 9)), g, 0)
+    lbm.lbm_set_history(lat.h, 256)
+    return lat
+
+
+def state(lat):
+    f, g, step = lat.populations()
+    h = lbm.lbm_read_history(lat.h, 256)
+    return [f, g, step, *[v for _, v in sorted(lat.diagnostics(raise_on_diverged=False).items())],
+            *[v for _, v in sorted(lat.fields().items())], *[h[k] for k in sorted(h)]]
+
+
+def assert_same(a, b, what):
+    for k, (x, y) in enumerate(zip(state(a), state(b))):
+        assert np.array_equal(np.asarray(x), np.asarray(y), equal_nan=True), (what, k)
+
+
+def compare(nx, ny, p, prec, stream, calls, diag_every=0):
+    lat, ref = (start(nx, ny, p, prec, stream) for _ in range(2))
+    lbm.lbm_set_streaming(ref.h, lbm.LBM_STREAM_TWO_BUFFERS)
+    for n in calls:
+        for L in (lat, ref):
+            lbm.lbm_set_diag_every(L.h, diag_every)
+            L.step(n)
+        assert_same(lat, ref, (nx, ny, prec, n))
+
+
+RATES = dict(k0=0.9, k0f=1.1, k1f=1.2)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16sr", "fp16"])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (2, 40), (31, 3), (33, 17), (64, 32), (65, 33), (257, 129), (700, 90)])
+def test_tiles(stream, prec, nx, ny):
+    compare(nx, ny, workloads.params(Ra=1e5, strip_center=0.4, **RATES), prec, stream, (2, 3, 18, 33, 33, 33), 9)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16sr", "bf16"])
+@pytest.mark.parametrize("problem,nx,ny", [("stefan", 2, 2), ("stefan", 17, 4), ("stefan", 300, 32), ("stefan", 40, 33),
+                                           ("cavity", 33, 17), ("cavity", 130, 70)])
+def test_tiles_without_flow(stream, prec, problem, nx, ny):
+    if problem == "stefan":
+        p = workloads.stefan_1024x4(Ste=0.5, nx=nx)[2]
+    else:
+        p = workloads.params(Ra=1e5, flow_on=0, strip_width=0.6)
+    compare(nx, ny, p, prec, stream, (2, 3, 18, 33))
+
+
+@pytest.mark.parametrize("nx,ny", [(1023, 520), (1025, 513), (8, 65535), (4500, 130), (2048, 1024)])
+def test_bands(stream, nx, ny):
+    compare(nx, ny, workloads.params(Ra=1e6, strip_center=0.6, **RATES), "fp32", stream, (2, 3, 10, 10, 11), 4)
+
+
+MEMBERS = [(256, 128, dict(Ra=1e6, strip_center=0.2)), (300, 77, dict(Ra=1e5, strip_center=0.65)), (64, 32, dict()),
+           (3, 5, dict(Ra=1e4)), (131, 9, dict(Ra=1e6, strip_width=0.4))]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16sr"])
+@pytest.mark.parametrize("copies", [1, 14])
+def test_batches(stream, prec, copies):
+    """Few small members (tiles) and many (bands), one of them a step ahead;
+    odd and even calls, pieces direct and replayed."""
+    groups = []
+    for mode in (None, lbm.LBM_STREAM_TWO_BUFFERS):
+        lats = [start(nx, ny, workloads.params(**RATES, **kw), prec, stream, seed=k)
+                for k, (nx, ny, kw) in enumerate(MEMBERS * copies)]
+        lats[1].step(1)
+        b = lbm.Batch(len(lats), stream)
+        for lat in lats:
+            b.add(lat)
+        if mode is not None:
+            lbm.lbm_batch_set_streaming(b.b, mode)
+        for n in (1, 2, 3, 20, 135, 20, 135, 20):
+            b.step(n)
+        b.close()
+        groups.append(lats)
+    for k, (x, y) in enumerate(zip(*groups)):
+        assert_same(x, y, (prec, copies, k))
