@@ -146,7 +146,8 @@ int lbm_step(lbm_handle h, long long n);
  * each lbm_step call only, the default). */
 int lbm_set_diag_every(lbm_handle h, long long k);
 
-/* Launch shape of the sweep (the tuner's knobs): rows of the lattice walked by
+/* Launch shape of the sweep (the tuner's knobs; steps taken several per launch,
+ * see lbm_set_streaming, depend on graph_chunk only): rows of the lattice walked by
  * each thread of a block (1 to 1024, default 1, or 2 with 16-bit storage);
  * the distance, in rows, at which each block asks L2 to prefetch a later
  * block's tile rows (0 = off, default 16, or 0 with 16-bit storage); and
@@ -198,10 +199,10 @@ int lbm_set_launch(lbm_handle h, int rows_per_block, int prefetch_rows, int grap
  * staged 16-bit sweep and lbm_step_static always use two buffers; a batch has
  * its own setting (lbm_batch_set_streaming).
  * Until this is called the library chooses: small lattices (FP32 and 16-bit
- * storage up to 2^19 cells, FP64 without flow up to 2^14; a Stefan lattice up to
- * 32 rows high) advance several steps per launch, each block keeping its part of
+ * storage up to 2^19 cells, FP64 up to 2^15 with flow and 2^14 without; a Stefan
+ * lattice up to 32 rows high) advance several steps per launch, each block keeping its part of
  * the lattice in shared memory for up to 16 steps and computing its neighbours'
- * edge cells itself (256 x 128 FP32: 5.4 -> 1.7 us per step); larger FP32
+ * edge cells itself (256 x 128 FP32: 5.4 -> 1.6 us per step); larger FP32
  * cavities with flow take two steps per pass over memory (2048 x 1024: 35.9 ->
  * 26.4).  A call's last step and the diagnostic steps are sweeps.  Calling this,
  * with either mode, asks for one sweep per step.
@@ -363,8 +364,9 @@ int lbm_batch_set_launch(lbm_batch b, int rows_per_block, int prefetch_rows, int
  * buffer, and the closing steps run over two buffers, so that between calls
  * every member's state is the two-buffer one (results do not depend on the
  * mode, bit for bit; members may be stepped alone or in other batches between
- * calls).  Until this is called the batch follows its precision: one buffer,
- * two for LBM_FP64.  Synchronises the batch's stream.  Errors: LBM_ERR_ARG. */
+ * calls).  Until this is called a batch of cavities with flow takes several steps
+ * per launch, as a single lattice does (lbm_set_streaming), and any other follows
+ * its precision: one buffer, two for LBM_FP64.  Synchronises the batch's stream.  Errors: LBM_ERR_ARG. */
 int lbm_batch_set_streaming(lbm_batch b, int mode);
 
 /* Autotuner for a batch: times rows per block (1, 2, 3, 4) x prefetch distance
@@ -397,7 +399,8 @@ int lbm_batch_destroy(lbm_batch b);
  * legacy default stream).  Both buffers use the library's tile-major layout:
  * element ((x / 128) * ny + y) * 2304 + p * 128 + x % 128 for plane p (0..8 =
  * f_0..f_8, 9..17 = g_0..g_8), ceil(nx / 128) * ny * 2304 elements of FP32
- * (LBM_FP32) or FP64 (LBM_FP64).  With flow_on = 0 the f planes are neither
+ * (LBM_FP32) or FP64 (LBM_FP64), on any element boundary (16-byte ones are
+ * fastest).  With flow_on = 0 the f planes are neither
  * read nor written.  `step` is the step number of src.  If `out` is non-NULL
  * the call synchronises the stream and fills it with the diagnostics of step
  * + 1, where Q_cum covers this call only; with out = NULL it returns without

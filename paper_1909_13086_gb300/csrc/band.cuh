@@ -176,7 +176,8 @@ __global__ void __launch_bounds__(kBandThreads, kBandWarps / (kBandThreads / 32)
 
 template <typename S>
 cudaError_t launch_band(const SweepArgs<float> &a, const BandArgs &b, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(band_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b.smem);
+    cudaError_t e = cudaFuncSetAttribute(band_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kBandSmemMax);
     if (e != cudaSuccess) return e;
     return launch_shared(band_kernel<S>, dim3(b.strips, b.bands), dim3(b.threads), b.smem, s, a, b);
 }
@@ -204,7 +205,7 @@ template <typename S>
 cudaError_t launch_batch_band(const void *entries, const int *mstarts, const int *parity, int n, int nblocks, int j,
                               const BandArgs &b, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(batch_band_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)b.smem);
+                                         (int)kBandSmemMax);
     if (e != cudaSuccess) return e;
     return launch_shared(batch_band_kernel<S>, dim3(nblocks), dim3(b.threads), b.smem, s,
                          static_cast<const BatchEntry<float> *>(entries), mstarts, parity, n, j, b);

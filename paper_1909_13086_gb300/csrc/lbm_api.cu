@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -246,9 +247,9 @@ size_t tile_smem(const lbm_s *h, int w, int hh, int T) {
 // Which lattices: FP32 and 16-bit storage up to 2^19 cells (per step, sweep and
 // tiles: 256 x 128 FP32 5.4 and 1.7 us, 512 x 512 7.1 and 4.5, 1024 x 512 9.0 and
 // 8.3; 256 x 128 BF16-SR 7.8 and 1.9), above which the sweep's larger launches
-// have paid for themselves.  FP64 with flow is bound by its pipe and gains
-// nothing from fewer launches (128 x 64: 18.9 and 18.2 us); without flow up to
-// 2^14 cells (1024 x 4 Stefan: 8.6 and 3.6).
+// have paid for themselves.  FP64: its pipe binds all but the launches, so up to 2^15
+// cells with flow (sweep and tiles: 64 x 32 9.9 and 7.1, 256 x 128 20.1 and 13.9) and
+// 2^14 without (1024 x 4 Stefan: 8.6 and 2.9).
 TilePlan tile_plan(lbm_s *const *lats, size_t n) {
     TilePlan plan;
     const lbm_s *h = lats[0];
@@ -259,9 +260,9 @@ TilePlan tile_plan(lbm_s *const *lats, size_t n) {
         if (lats[r]->nx > kTileMaxNx || (stefan && lats[r]->ny > 32)) return plan;
         if (n > 1 && (fp64 || stefan || !flow)) return plan;  // no batch kernel for these
     }
-    if (cells > (fp64 ? (flow ? 0 : 1 << 14) : 1 << 19)) return plan;
-    const double per_cell = fp64 ? 18.6 : (h->esize == 2 ? 1.6 : 1.5) * (flow ? 1.0 : 0.6);
-    const double least = fp64 ? 2200.0 : 700.0, launch = 4500.0;
+    if (cells > (fp64 ? (flow ? 1 << 15 : 1 << 14) : 1 << 19)) return plan;
+    const double per_cell = fp64 ? (flow ? 43.0 : 18.6) : (h->esize == 2 ? 1.6 : 1.5) * (flow ? 1.0 : 0.6);
+    const double least = fp64 ? (flow ? 6000.0 : 2200.0) : 700.0, launch = 4500.0;
     double best = 1e30;
     for (int w = stefan ? 8 : 32; w <= 128; w *= 2)
         for (int hh = stefan ? h->ny : 2; hh <= (stefan ? h->ny : 64); hh += hh < 16 ? 1 : 4) {
@@ -1344,10 +1345,17 @@ void batch_build(lbm_batch_s *b) {
     b->host_starts.assign(b->members.size(), 0);
     b->uniform = 0;
     int start = 0, mstart = 0;
-    // several steps per launch: tiles while the members are few and small, else bands
+    // several steps per launch: tiles while the members are few and small, else bands;
+    // with 16-bit storage bands for narrow members only, where half of a sweep's warps
+    // touch a side wall (us per step, bands and sweeps: BF16-SR 64 x 256 x 128 25.1 and
+    // 27.3, 12 mixed up to 512 x 256 12.7 and 14.3, 8 x 512 x 256 15.2 and 14.3; FP32
+    // 27.4 and 39.5, 12.9 and 14.9, 16.9 and 16.8)
+    int narrow = 0;
+    for (const lbm_s *h : b->members) narrow += h->nx <= 384;
     b->tile = tile_plan(b->members.data(), b->members.size());
     b->band = BandPlan();
-    if (b->tile.t == 0) b->band = band_plan(b->members.data(), b->members.size());
+    if (b->tile.t == 0 && (b->precision == LBM_FP32 || 2 * narrow > (int)b->members.size()))
+        b->band = band_plan(b->members.data(), b->members.size());
     b->host_mstarts.assign(b->members.size(), 0);
     for (size_t r = 0; r < b->members.size(); ++r) {
         lbm_s *h = b->members[r];
@@ -1842,6 +1850,13 @@ constexpr size_t kStaticBytes = kStaticOffD2 + ((kStaticFold * 32 + 255) / 256) 
 // Held by every GPU that loads this library, until the process exits.
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
 
+// One block, one word a thread: clears the tickets and the record, and sets the
+// record's step counter -- one launch where a memset and a copy were two.
+__global__ void static_begin_kernel(unsigned long long *scratch, unsigned long long step) {
+    constexpr size_t kCounter = (kStaticOffRec + offsetof(DevRecord, counter)) / 8;
+    scratch[threadIdx.x] = threadIdx.x == kCounter ? step : 0ull;
+}
+
 std::mutex g_static_mutex;
 void *g_static_addr[256] = {};  // device address of g_static_scratch, per device ordinal
 
@@ -1861,7 +1876,8 @@ extern "C" int lbm_step_static(const void *src, void *dst, int nx, int ny, int p
     t.precision = precision;
     t.ntx = (nx + kTW - 1) / kTW;
     t.rows = 1;
-    t.prefetch = kDefaultPrefetch;
+    // the caller's buffers: bulk prefetches start on 16-byte boundaries
+    t.prefetch = (reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) % 16 ? 0 : kDefaultPrefetch;
     set_grid(&t);
     const unsigned long long nblk = (unsigned long long)t.grid.x * t.grid.y;
     const int nq = p->problem == LBM_CAVITY ? (int)t.grid.x : (int)t.grid.y;
@@ -1914,24 +1930,27 @@ extern "C" int lbm_step_static(const void *src, void *dst, int nx, int ny, int p
 
     // The array keeps the previous call's contents: the tickets and the record
     // must start from zero, and the record's step counter from `step`.
-    const unsigned long long counter = (unsigned long long)step;
-    e = cudaMemsetAsync(base, 0, kStaticOffQ, t.stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&t.rec->counter, &counter, sizeof(counter), cudaMemcpyHostToDevice, t.stream);
+    static_begin_kernel<<<1, kStaticOffQ / 8, 0, t.stream>>>(reinterpret_cast<unsigned long long *>(base),
+                                                             (unsigned long long)step);
+    e = cudaGetLastError();
     if (e != cudaSuccess)
         return set_err(nullptr, LBM_ERR_CUDA, "lbm_step_static: clearing the scratch failed: %s",
                        cudaGetErrorString(e));
     t.step = step;
+    // the sweep and the fold are scheduled while the launch before them drains (not on
+    // the legacy default stream, whose other streams wait for it launch by launch);
+    // the clearing kernel itself waits for all the caller has queued
+    const bool pdl = t.stream != nullptr;
     if (precision == LBM_FP64) {
         SweepArgs<double> a = make_args<double>(&t, src, dst);
         a.step = step + 1;
         e = launch_lattice<double, double>(a, p->problem, p->flow_on != 0, kSweepDiag, t.grid, t.block,
-                                           t.stream, false);
+                                           t.stream, pdl);
     } else {
         SweepArgs<float> a = make_args<float>(&t, src, dst);
         a.step = step + 1;
         e = launch_lattice<float, float>(a, p->problem, p->flow_on != 0, kSweepDiag, t.grid, t.block,
-                                         t.stream, false);
+                                         t.stream, pdl);
     }
     if (e != cudaSuccess)
         return set_err(nullptr, LBM_ERR_CUDA, "lbm_step_static: launch failed: %s", cudaGetErrorString(e));

@@ -28,7 +28,9 @@ enum Mode {
 //            goes to its own slot i: the pull layout again.
 // Each cell reads and writes the same 18 locations in either sweep, so no two
 // cells touch one location, and the populations are those of the pull sweeps.
-enum Streaming { kPull = 0, kAAPush = 1, kAALocal = 2 };
+// kPullNarrow is kPull with accesses of one value each, for a caller's buffers that are
+// not on 8-byte boundaries (launch_mode).
+enum Streaming { kPull = 0, kAAPush = 1, kAALocal = 2, kPullNarrow = 3 };
 
 // Population layout in device memory ("tile-major structure of arrays").
 // The lattice is cut into column tiles of kTW cells.  Within a tile, each row
@@ -142,6 +144,7 @@ struct TileArgs {
 constexpr int kBandThreads = 128;  // block size limit; two columns a thread
 constexpr int kBandWarps = 12;     // per SM: up to 168 registers a thread, no spills
 constexpr int kBandMaxStrips = 2048;
+constexpr size_t kBandSmemMax = 4 * 6 * 2 * kBandThreads * 2 * sizeof(float);  // band_args
 struct BandArgs {
     int strips, bands;
     int threads;     // one per two columns of the widest strip and its halo pairs

@@ -1705,29 +1705,30 @@ __device__ __forceinline__ void sweep_block_two(const SweepArgs<float> &a, const
     block_epilogue<float, kCavity, MODE>(a, bx, by, gx, acc, sh);
 }
 
-// Whether a sweep runs two cells per thread.
-template <typename real, int PROB, bool FLOW, int MODE>
+// Whether a sweep runs two cells per thread (its 8-byte accesses need buffers on
+// 8-byte boundaries).
+template <typename real, int PROB, bool FLOW, int MODE, int SM = kPull>
 __host__ __device__ constexpr bool takes_two() {
-    return sizeof(real) == 4 && PROB == kCavity && FLOW && MODE != kFields;
+    return sizeof(real) == 4 && PROB == kCavity && FLOW && MODE != kFields && SM != kPullNarrow;
 }
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM>
 __device__ __forceinline__ void sweep_any(const SweepArgs<real> &a, const int bx, const int by, const int gx,
                                           double *sh) {
-    if constexpr (takes_two<real, PROB, FLOW, MODE>()) sweep_block_two<S, MODE, SM>(a, bx, by, gx, sh);
-    else sweep_block<real, S, PROB, FLOW, MODE, SM>(a, bx, by, gx, sh);
+    if constexpr (takes_two<real, PROB, FLOW, MODE, SM>()) sweep_block_two<S, MODE, SM>(a, bx, by, gx, sh);
+    else sweep_block<real, S, PROB, FLOW, MODE, SM == kPullNarrow ? kPull : SM>(a, bx, by, gx, sh);
 }
-template <typename real, int PROB, bool FLOW, int MODE>
+template <typename real, int PROB, bool FLOW, int MODE, int SM = kPull>
 __host__ __device__ constexpr int sweep_threads() {
-    return takes_two<real, PROB, FLOW, MODE>() ? kTW / 2 : kTW;
+    return takes_two<real, PROB, FLOW, MODE, SM>() ? kTW / 2 : kTW;
 }
 // Blocks per SM the register allocation aims at (BATCH: a batch kernel, whose
 // arguments sit in shared memory and take more registers).  Two cells per thread,
 // us per step at 8 / 10 / 12 blocks: 2048 x 1024 FP32 one buffer 36.4 / 35.9 / 36.2,
 // FP16-SR 21.7 / 21.6 / 21.1, 1001 x 701 BF16-SR 9.1 / 9.1 / 8.8; 32 x 256 x 128
 // batches FP32 18.2 / 17.7 / -, BF16-SR 15.0 / 14.7 / 15.7.
-template <typename real, typename S, int PROB, bool FLOW, int MODE, bool BATCH = false>
+template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM, bool BATCH>
 __host__ __device__ constexpr int sweep_blocks() {
-    if (takes_two<real, PROB, FLOW, MODE>()) return Store<S>::kDev && !BATCH ? 12 : 10;
+    if (takes_two<real, PROB, FLOW, MODE, SM>()) return Store<S>::kDev && !BATCH ? 12 : 10;
     return sizeof(real) == 4 ? 1024 / kTW : 1;
 }
 
@@ -1735,7 +1736,8 @@ __host__ __device__ constexpr int sweep_blocks() {
 // (registers capped at 64, the occupancy the memory pipeline needs); FP64 is
 // ALU-bound and keeps its registers.
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM = kPull>
-__global__ void __launch_bounds__(sweep_threads<real, PROB, FLOW, MODE>(), sweep_blocks<real, S, PROB, FLOW, MODE>())
+__global__ void __launch_bounds__(sweep_threads<real, PROB, FLOW, MODE, SM>(),
+                                  sweep_blocks<real, S, PROB, FLOW, MODE, SM, false>())
     lattice_kernel(const SweepArgs<real> a) {
     __shared__ double sh[32 * 4];
     pdl_launch_dependents();
@@ -2038,7 +2040,7 @@ struct EntryLayout {
 };
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM = kPull>
 __global__ void __launch_bounds__(sweep_threads<real, PROB, FLOW, MODE>(),
-                                  sweep_blocks<real, S, PROB, FLOW, MODE, true>())
+                                  sweep_blocks<real, S, PROB, FLOW, MODE, SM, true>())
     batch_kernel(const BatchEntry<real> *entries, const int *starts, const int *parity, int n,
                  int uniform, int interleave, int j) {
     static_assert(sizeof(BatchEntry<real>) % 16 == 0, "entries are copied in 16-byte pieces");
@@ -2300,6 +2302,12 @@ static cudaError_t launch_mode(const SweepArgs<real> &a, int mode, dim3 grid, di
     switch (mode) {
         case kSweep: return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep>, grid, threads, s, pdl, a);
         case kSweepDiag:
+            if constexpr (takes_two<real, PROB, FLOW, kSweepDiag>() && !Store<S>::kDev) {
+                // lbm_step_static's buffers are the caller's
+                if ((reinterpret_cast<uintptr_t>(a.src) | reinterpret_cast<uintptr_t>(a.dst)) % 8)
+                    return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kPullNarrow>, grid, dim3(kTW), s,
+                                    pdl, a);
+            }
             return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag>, grid, threads, s, pdl, a);
         case kFields: lattice_kernel<real, S, PROB, FLOW, kFields><<<grid, block, 0, s>>>(a); break;
         default: return cudaErrorInvalidValue;
