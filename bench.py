@@ -3,7 +3,7 @@
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-One step = one fused collide-and-stream sweep (pull streaming with the wall
+One step = one fused collide-and-stream update (pull streaming with the wall
 rules, H -> (T, f_l) inversion, g and f block collisions, buoyancy, the
 per-step heated-wall inflow reduction) over the whole 2048 x 1024 lattice in
 FP32; the FP64 diagnostics reductions (melt fraction, sum H, max |u|, NaN
@@ -29,9 +29,9 @@ the aggregate MLUPS and the 16-bit results' largest melt-fraction and Nusselt
 differences from an FP64 run of the same requests.
 
 --batch N times the batched path instead: N cavities of 256 x 128 (the
-serving size; Ra and strip centre varied, seeded) advanced together, one fused
-launch per step over all of them (graph-replayed); the last step carries the
-diagnostics.  Same JSON line, device-resident timing only.
+serving size; Ra and strip centre varied, seeded) advanced together, two steps
+per launch over all of them (one in FP64; graph-replayed); the last step carries
+the diagnostics.  Same JSON line, device-resident timing only.
 """
 from __future__ import annotations
 
@@ -61,7 +61,7 @@ FP64_FLOPS_PER_LUP = 227
 # GB300 FP64 pipe: 2 FMA per clock per SM, 2 flops each, 152 SMs, 2070 MHz.
 FP64_PEAK_TFLOPS = 2 * 2 * 152 * 2.070e9 / 1e12
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1909_13086_gb300", "csrc", f)
-                  for f in ("sweep.cuh", "lbm_internal.h")]
+                  for f in ("sweep.cuh", "tile.cuh", "band.cuh", "lbm_internal.h")]
 
 
 def sweep_launches(warmup: int, steps: int) -> int:
@@ -73,6 +73,24 @@ def sweep_launches(warmup: int, steps: int) -> int:
     return steps + len(diag)
 
 
+def kernel_launches(precision: str, warmup: int, steps: int) -> int:
+    """Kernels launched by lbm_step(steps) after `warmup` steps.  FP32 takes two
+    steps per launch: the library cuts the call into pieces that end at the
+    diagnostic steps and are at most 128 long; a piece's last step, if diagnostic,
+    is a sweep and a fold, an odd step before it a sweep."""
+    if precision != "fp32":
+        return sweep_launches(warmup, steps)
+    total, at, end = 0, warmup, warmup + steps
+    while at < end:
+        stop = min(end, (at // DIAG_EVERY + 1) * DIAG_EVERY)
+        diag = stop - at <= 128
+        n = min(stop - at, 128)
+        plain = n - 1 if diag else n
+        total += plain // 2 + plain % 2 + (2 if diag else 0)
+        at += n
+    return total
+
+
 def workload_config(precision: str) -> dict:
     one = precision != "fp64"   # the library's default streaming (lbm_set_streaming)
     mb = BYTES_PER_LUP[precision] * NX * NY / 2 / 1e6      # one buffer of populations
@@ -80,10 +98,12 @@ def workload_config(precision: str) -> dict:
                         f"{precision.upper()} populations",
             "nx": NX, "ny": NY, "precision": precision,
             "diagnostics": f"fused every {DIAG_EVERY} steps; heated-wall flux every step",
-            "streaming": ("one buffer (push / local sweeps), the call's last 1-2 sweeps over two buffers"
+            "streaming": ("one buffer read and the other written per two steps (bands); diagnostic steps are sweeps"
+                          if precision == "fp32" else
+                          "one buffer (push / local sweeps), the call's last 1-2 sweeps over two buffers"
                           if one else "two buffers"),
-            "l2": (f"inputs larger than L2 ({mb:.0f} MB of populations in the buffer a step reads and "
-                   "writes), no flush" if one and mb > L2_MB else
+            "l2": (f"inputs larger than L2 ({mb:.0f} MB of populations read and as many written per two "
+                   "steps), no flush" if one and mb > L2_MB else
                    f"the populations ({mb:.0f} MB in the one buffer a step reads and writes) fit in the "
                    f"{L2_MB:.0f} MB L2: a step reads what the previous one wrote, no flush" if one else
                    f"inputs larger than L2 (2 x {mb:.0f} MB populations), no flush")}
@@ -148,9 +168,9 @@ def profile_path(precision: str, batch: int = 0) -> str:
 
 
 def profiled_traffic(precision: str = "fp32", batch: int = 0) -> float | None:
-    """DRAM bytes per launch of the sweep in `precision` (of the batch kernel
-    over `batch` lattices) from the committed ncu summary, if it was taken on
-    the current kernel source."""
+    """DRAM bytes per step in `precision` (of the batch kernels over `batch`
+    lattices) from the committed ncu summary, if it was taken on the current
+    kernel source."""
     try:
         text = open(profile_path(precision, batch)).read()
     except OSError:
@@ -415,8 +435,9 @@ def run_ours(args) -> None:
                 "peak_source": f"{peak_kind} HBM copy bandwidth",
                 "algorithmic_bytes_per_launch": alg_bytes}
     if traffic:
-        # The DRAM side: the profiled bytes per launch (warm L2, as in this
-        # loop) over the measured time.  A step that starts on rows the
+        # The DRAM side: the profiled bytes per step (warm L2, as in this
+        # loop) over the measured time.  FP32 moves populations once per two
+        # steps.  A step that starts on rows the
         # previous one left in L2 moves fewer bytes than it reads and writes,
         # so `frac` (algorithmic bytes) can exceed 1 while this stays below.
         roofline["dram_achieved"] = round(traffic / kernel_s / 1e9, 1)
@@ -441,7 +462,7 @@ def run_ours(args) -> None:
         "config": workload_config(prec),
         "roofline": roofline,
         "e2e": e2e,
-        "gpu_launches": sweep_launches(args.warmup, args.steps),
+        "gpu_launches": kernel_launches(prec, args.warmup, args.steps),
         "clocks": clocks.summary(),
         "melt_fraction": d["melt_fraction"],
     }
@@ -560,19 +581,17 @@ def run_batch(args) -> None:
         "ms_per_step": round(kernel_s * 1e3, 4), "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": prec, "data": "synthetic",
         "config": {"workload": f"batch of {n} cavities {BATCH_NX}x{BATCH_NY} (Ra 1e6-1e8, strip "
-                               f"W/4 at 0.2-0.8 W, seeded), {prec.upper()} populations, one fused "
-                               "launch per step", "lattices": n, "precision": prec,
-                   "streaming": ("one buffer (push / local sweeps), the call's last 1-2 steps over two buffers"
-                                 if prec != "fp64" else "two buffers"),
-                   # a step reads and writes every population once: half the algorithmic bytes
-                   # is the state; with two buffers the step touches twice that
+                               f"W/4 at 0.2-0.8 W, seeded), {prec.upper()} populations, "
+                               + ("one fused launch per step" if prec == "fp64" else "several steps per launch"
+                                  if cells <= 1 << 19 else "two steps per launch"),
+                   "lattices": n, "precision": prec,
+                   "streaming": ("two buffers" if prec == "fp64" else
+                                 "one buffer read and the other written per launch, the last step a sweep"),
+                   # the populations in both buffers
                    "l2": (f"inputs larger than L2 ({alg_bytes / 1e6:.0f} MB of populations in the two "
-                          "buffers), no flush" if prec == "fp64" else
-                          f"inputs larger than L2 ({alg_bytes / 2e6:.0f} MB of populations in the buffer "
-                          "a step reads and writes), no flush" if alg_bytes / 2 > L2_MB * 1e6 else
-                          f"the populations ({alg_bytes / 2e6:.0f} MB in the one buffer a step reads and "
-                          f"writes) fit in the {L2_MB:.0f} MB L2: a step reads what the previous one "
-                          "wrote, no flush"),
+                          "buffers), no flush" if alg_bytes > L2_MB * 1e6 else
+                          f"the populations ({alg_bytes / 1e6:.0f} MB in the two buffers) fit in the "
+                          f"{L2_MB:.0f} MB L2: a step reads what the previous one wrote, no flush"),
                    "launch": ({"rows": tuned["rows"], "prefetch": tuned["prefetch"],
                                "interleave": tuned["interleave"], "by": "lbm_batch_autotune"}
                               if tuned else "default")},
@@ -581,7 +600,11 @@ def run_batch(args) -> None:
                      "peak_source": f"{peak_kind} HBM copy bandwidth",
                      "algorithmic_bytes_per_launch": alg_bytes},
         "e2e": None,
-        "gpu_launches": args.steps + 1,
+        # two steps per launch and an odd one alone (up to 2^19 cells at most 16 per
+        # launch), the diagnostic step and its fold
+        "gpu_launches": (args.steps + 1 if prec == "fp64" else
+                         -(-(args.steps - 1) // 16) + 2 if cells <= 1 << 19 else
+                         (args.steps - 1) // 2 + (args.steps - 1) % 2 + 2),
         "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)

@@ -288,6 +288,12 @@ TilePlan tile_plan(lbm_s *const *lats, size_t n) {
                 }
             }
         }
+    // FP32 cavities with flow have the bands to go to.  Where a launch can hold two
+    // steps only, or a step takes over 9 us, those are faster (us per step, tiles and
+    // bands: 700 x 500 7.5 and 6.6, 600 x 600 7.5 and 6.6, 16 x 256 x 128 10.5 and 8.6;
+    // but 1024 x 512 7.9 and 8.3, 2 x 512 x 512 8.5 and 9.1, 12 x 256 x 128 7.2 and 7.8).
+    if (h->precision == LBM_FP32 && flow && !stefan && cells > 1 << 18 && (plan.t <= 2 || best > 9000.0))
+        plan = TilePlan();
     return plan;
 }
 
@@ -961,13 +967,20 @@ int lbm_read_fields(lbm_handle h, unsigned mask, double *H, double *T, double *f
     int rc = by_precision(h->precision, [&](auto t) { return BTRIRT_T(t, enqueue_fields)(h, dev); });
     if (rc != LBM_OK) return rc;
     // one copy for fields that follow one another on the host as in the staging (each
-    // copy costs ~1.7 us whatever its size: 256 x 128, all six 46 us, 37 in one)
+    // copy costs ~1.7 us whatever its size: 256 x 128, all six 46 us, 37 in one).
+    // Neighbours may still be separate pinned allocations, which a copy may not span:
+    // it is refused then, and they are copied one by one.
     for (int k = 0; k < 6;) {
         int e = k + 1;
         if (dev[k]) {
             while (e < 6 && dev[e] && host[e] == host[e - 1] + P) ++e;
-            CUDA_TRY(h, cudaMemcpyAsync(host[k], dev[k], (e - k) * P * sizeof(double), cudaMemcpyDeviceToHost,
-                                        h->stream));
+            if (e - k > 1 && cudaMemcpyAsync(host[k], dev[k], (e - k) * P * sizeof(double), cudaMemcpyDeviceToHost,
+                                             h->stream) != cudaSuccess) {
+                cudaGetLastError();
+                e = k + 1;
+            }
+            if (e - k == 1)
+                CUDA_TRY(h, cudaMemcpyAsync(host[k], dev[k], P * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         }
         k = e;
     }

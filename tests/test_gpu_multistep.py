@@ -125,3 +125,18 @@ def test_static_step_takes_buffers_on_any_element(offset):
                                 s.cuda_stream)
         out.append((bufs[1][k:k + n].cpu().numpy(), d))
     assert np.array_equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 256), (256, 128)])
+def test_fields_into_separate_pinned_arrays(stream, nx, ny):
+    """Six pinned arrays of a power-of-two size usually follow one another in
+    memory without being one allocation; a copy may not span two of them."""
+    import torch
+
+    lat = lbm.Lattice(nx, ny, workloads.params(Ra=1e6), precision="fp32", stream=stream)
+    lat.step(5)
+    want = lat.fields()
+    pinned = [torch.empty(ny, nx, dtype=torch.float64, pin_memory=True).numpy() for _ in range(6)]
+    lbm.lbm_read_fields(lat.h, 63, *sorted(pinned, key=lambda a: a.ctypes.data))
+    for name, got in zip(lbm.FIELD_NAMES, sorted(pinned, key=lambda a: a.ctypes.data)):
+        assert np.array_equal(got, want[name]), name
