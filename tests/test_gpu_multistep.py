@@ -70,6 +70,13 @@ def test_tiles_without_flow(stream, prec, problem, nx, ny):
     compare(nx, ny, p, prec, stream, (2, 3, 18, 33))
 
 
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16sr"])
+@pytest.mark.parametrize("nx,ny", [(3, 2), (40, 5), (130, 32)])
+def test_tiles_of_a_periodic_lattice_with_flow(stream, prec, nx, ny):
+    p = workloads.params(problem=workloads.STEFAN, Ra=1e4, alpha_override=0.05, **RATES)
+    compare(nx, ny, p, prec, stream, (2, 3, 18, 33))
+
+
 @pytest.mark.parametrize("nx,ny", [(1023, 520), (1025, 513), (8, 65535), (4500, 130), (2048, 1024)])
 def test_bands(stream, nx, ny):
     compare(nx, ny, workloads.params(Ra=1e6, strip_center=0.6, **RATES), "fp32", stream, (2, 3, 10, 10, 11), 4)
