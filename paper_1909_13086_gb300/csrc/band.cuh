@@ -20,6 +20,13 @@
 // those of two sweeps.  The bands of one launch run at the same time, one wave of
 // blocks; successive launches march them in opposite directions, so that each
 // starts on the rows the previous one wrote last.
+//
+// 2048 x 1024 FP32 on GB300: 36.7 us per step with one-buffer sweeps, 26.3 here: 137
+// MB of DRAM traffic per step (161 before) at 5.2 TB/s, 0.77 of the copy bandwidth.
+// What is left is latency: the loads of the next row wait in registers through step 2
+// of the row before, which leaves 12 warps per SM.  Without them 16 warps fit, and it
+// takes 36.6 us: the larger rings leave too little L1 for the lines that a pair's two
+// halves share.
 #pragma once
 
 #include "tile.cuh"

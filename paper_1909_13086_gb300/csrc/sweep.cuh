@@ -1,8 +1,9 @@
 // sweep.cuh -- the fused B-TriRT collide-and-stream kernel (device code).
 //
 // Layout: tile-major structure of arrays (lbm_internal.h).  One thread per
-// lattice column of a kTW-wide tile, walking `rows` rows; a warp covers 32
-// consecutive cells of one row, so every load and store is a coalesced 128 B
+// lattice column of a kTW-wide tile (two neighbouring columns in the cavity
+// sweeps with flow in FP32 arithmetic, sweep_block_two), walking `rows` rows; a
+// warp covers 32 (64) consecutive cells of one row, so every load and store is a coalesced 128 B
 // line (FP32).  In the interior the 18 pull loads of a cell are one base
 // register plus compile-time offsets; boundary rows and the two warps of a
 // row that touch a side wall take a generic path with the wall rules.
@@ -340,12 +341,12 @@ __device__ __forceinline__ void emit(real p[9], real a, real B0, real B1x, real 
     p[8] = a * p[8] + (e68 - t6);
 }
 
-// ---- f and g as one pair ----
-// The two collisions are the same block operator on different coefficients, so
-// with flow on (FP32 arithmetic) they run as pairs (x: f, y: g) on sm_100's
-// packed FP32 instructions: one issue slot for both halves, each half rounded
-// as its scalar instruction would be.  The sweeps are bound by instruction
-// issue (16-bit storage) or by latency (FP32), not by the FP32 pipe.
+// ---- packed FP32 pairs ----
+// sm_100's packed FP32 instructions: one issue slot for both halves, each half
+// rounded as its scalar instruction would be (the FP32 pipe's rate is the same).
+// Where a thread has one cell the pair is (f, g): the two collisions are the same
+// block operator on different coefficients (2048 x 1024 FP16-SR 24.7 -> 23.6 us per
+// step).  Where it has two, every operation is packed over the cells (-> 21.1).
 __device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, both(-1.0f), a); }

@@ -17,6 +17,12 @@
 // A cell's nine slots lie next to each other (f_i and g_i together in one): the
 // strides of 9 x 4, 8 or 16 bytes from lane to lane meet no bank twice, and all
 // nine are one base plus immediate offsets.
+//
+// On GB300, us per step, sweeps and tiles: 64 x 32 FP32 4.9 and 1.4, 256 x 128 FP32 5.4
+// and 1.6, BF16-SR 7.8 and 1.8, 512 x 512 FP32 7.1 and 4.6, 1024 x 4 Stefan FP64 8.6 and
+// 2.9.  Bound by latency: 4.2 us a launch, then per step one cell's chain and the
+// barrier (256 x 128: 43 % issue active).  Two cells per thread, as in the sweeps, has
+// half the warps and is slower (512 x 512 5.4).
 #pragma once
 
 #include "sweep.cuh"
