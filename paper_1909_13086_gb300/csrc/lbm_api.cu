@@ -1271,7 +1271,7 @@ extern "C" int lbm_autotune(lbm_handle h, int steps_per_trial, int *rows_out, in
 }
 
 // ---------------------------------------------------------------------------
-// Batches: many lattices advanced by one launch per step.
+// Batches: many lattices advanced by shared launches, one per step or per several.
 // ---------------------------------------------------------------------------
 struct lbm_batch_s {
     int device = 0;

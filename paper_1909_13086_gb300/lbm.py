@@ -400,7 +400,7 @@ class Lattice:
 
 
 class Batch:
-    """Lattices advanced together by one fused launch per step."""
+    """Lattices advanced together by shared launches, one per step or per several."""
 
     def __init__(self, max_lattices: int = 64, stream: int | None = None):
         self.b = lbm_batch_create(max_lattices, stream)

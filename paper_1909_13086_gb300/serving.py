@@ -3,7 +3,7 @@
 Requests (grid size, Rayleigh number, heated-strip position, storage precision,
 step budget) arrive as a Poisson stream.  The server keeps every admitted
 request's populations resident on the GPU.  Requests of one storage precision
-and size class form a group: one ``Batch`` (one fused launch per step for all
+and size class form a group: one ``Batch`` (shared launches for all
 members, graph-replayed) on the group's own CUDA stream, advanced in quanta of
 ``quantum`` steps.  Groups run concurrently, so small lattices never wait for
 a large one's step, and the host polls each group's quantum by event: when it
