@@ -306,9 +306,9 @@ int lbm_write_populations(lbm_handle h, const double *f, const double *g, long l
 /* ---- Batches: many lattices advanced together ------------------------------
  * A batch advances all its lattices by shared launches, one per step or per
  * several (lbm_batch_set_streaming): the blocks of every member form one grid
- * (each block looks up its lattice and tile in a device table), so lattices too small to fill the GPU alone -- the
- * 256 x 128 requests of a serving stream -- share it, and the per-step launch
- * cost is paid once.  lbm_batch_step cuts its steps into pieces (128 plain
+ * (each block looks up its lattice and tile in a device table), so lattices
+ * too small to fill the GPU alone -- the 256 x 128 requests of a serving
+ * stream -- share it, and the launch cost is paid once.  lbm_batch_step cuts its steps into pieces (128 plain
  * steps while more than 128 remain, then the rest, ending with the diagnostic
  * step) and, as lbm_step does, replays a piece from a CUDA graph from the
  * second time it is asked for (graphs are kept per batch composition); every
