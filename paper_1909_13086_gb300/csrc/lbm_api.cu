@@ -250,7 +250,9 @@ size_t tile_smem(const lbm_s *h, int w, int hh, int T) {
 // have paid for themselves.  FP64: its pipe binds all but the launches, so up to 2^15
 // cells with flow (sweep and tiles: 64 x 32 9.9 and 7.1, 256 x 128 20.1 and 13.9) and
 // 2^14 without (1024 x 4 Stefan: 8.6 and 2.9).
-TilePlan tile_plan(lbm_s *const *lats, size_t n) {
+// A batch, of one member too, has the kernel for cavities with flow in FP32
+// arithmetic only (launch_batch_tile).
+TilePlan tile_plan(lbm_s *const *lats, size_t n, bool batch) {
     TilePlan plan;
     const lbm_s *h = lats[0];
     const bool stefan = h->p.problem == LBM_STEFAN, fp64 = h->precision == LBM_FP64, flow = h->p.flow_on != 0;
@@ -258,8 +260,8 @@ TilePlan tile_plan(lbm_s *const *lats, size_t n) {
     for (size_t r = 0; r < n; ++r) {
         cells += (long long)lats[r]->nx * lats[r]->ny;
         if (lats[r]->nx > kTileMaxNx || (stefan && lats[r]->ny > 32)) return plan;
-        if (n > 1 && (fp64 || stefan || !flow)) return plan;  // no batch kernel for these
     }
+    if (batch && (fp64 || stefan || !flow)) return plan;
     if (cells > (fp64 ? (flow ? 1 << 15 : 1 << 14) : 1 << 19)) return plan;
     const double per_cell = fp64 ? (flow ? 43.0 : 18.6) : (h->esize == 2 ? 1.6 : 1.5) * (flow ? 1.0 : 0.6);
     const double least = fp64 ? (flow ? 6000.0 : 2200.0) : 700.0, launch = 4500.0;
@@ -379,7 +381,7 @@ BandArgs band_args(const lbm_s *h, const BandPlan &plan) {
 // bands: 21.1 and 24.8 us per step; FP32 35.9 and 26.4; 1500 x 700 FP32 16.3 and
 // 14.3).
 void plan_steps(lbm_s *h) {
-    h->tile = tile_plan(&h, 1);
+    h->tile = tile_plan(&h, 1, false);
     h->band = BandPlan();
     if (h->tile.t == 0 && h->precision == LBM_FP32) h->band = band_plan(&h, 1);
 }
@@ -1365,7 +1367,7 @@ void batch_build(lbm_batch_s *b) {
     // 27.4 and 39.5, 12.9 and 14.9, 16.9 and 16.8)
     int narrow = 0;
     for (const lbm_s *h : b->members) narrow += h->nx <= 384;
-    b->tile = tile_plan(b->members.data(), b->members.size());
+    b->tile = tile_plan(b->members.data(), b->members.size(), true);
     b->band = BandPlan();
     if (b->tile.t == 0 && (b->precision == LBM_FP32 || 2 * narrow > (int)b->members.size()))
         b->band = band_plan(b->members.data(), b->members.size());

@@ -1,0 +1,38 @@
+// Prints the plans the library makes, on the host: each input line
+//     precision problem flow streaming n  nx ny  nx ny ...
+// describes a batch of n lattices (streaming: -1 as lbm_batch_create leaves it);
+// the output line holds the batch's plan and the first lattice's own:
+//     batch tile w h t  band threads rows | solo tile w h t  band threads rows
+#include "lbm_api.cu"
+
+#include <iostream>
+
+int main() {
+    int precision, problem, flow, streaming, n;
+    while (std::cin >> precision >> problem >> flow >> streaming >> n) {
+        std::vector<lbm_s> lats(n);
+        lbm_batch_s b;
+        b.precision = precision;
+        b.problem = problem;
+        b.flow = flow;
+        b.streaming = streaming;
+        for (lbm_s &h : lats) {
+            std::cin >> h.nx >> h.ny;
+            h.precision = precision;
+            h.esize = precision == LBM_FP64 ? 8 : (precision == LBM_FP32 ? 4 : 2);
+            h.ntx = (h.nx + kTW - 1) / kTW;
+            h.num_sms = 152;
+            h.p.problem = problem;
+            h.p.flow_on = flow;
+            set_grid(&h);
+            plan_steps(&h);
+            b.members.push_back(&h);
+        }
+        if (precision == LBM_FP64) batch_build<double>(&b);
+        else batch_build<float>(&b);
+        const lbm_s &h = lats[0];
+        std::printf("%d %d %d %d %d %d %d %d %d %d\n", b.tile.w, b.tile.h, b.tile.t, b.band.threads, b.band.rows,
+                    h.tile.w, h.tile.h, h.tile.t, h.band.threads, h.band.rows);
+    }
+    return 0;
+}

@@ -147,3 +147,25 @@ def test_fields_into_separate_pinned_arrays(stream, nx, ny):
     lbm.lbm_read_fields(lat.h, 63, *sorted(pinned, key=lambda a: a.ctypes.data))
     for name, got in zip(lbm.FIELD_NAMES, sorted(pinned, key=lambda a: a.ctypes.data)):
         assert np.array_equal(got, want[name]), name
+
+
+@pytest.mark.parametrize("prec,problem,kw,nx,ny", [
+    ("fp64", "cavity", {}, 64, 32), ("fp64", "cavity", dict(flow_on=0), 33, 17), ("fp64", "stefan", {}, 300, 4),
+    ("fp32", "cavity", {}, 65, 33), ("fp32", "cavity", dict(flow_on=0), 130, 70), ("fp32", "stefan", {}, 300, 32),
+    ("bf16sr", "cavity", {}, 31, 3), ("bf16sr", "stefan", {}, 17, 4), ("fp16", "cavity", dict(flow_on=0), 64, 32)])
+def test_batch_of_one(stream, prec, problem, kw, nx, ny):
+    """One member, of every kind, whether or not the batch kernels take several
+    steps of it: the member alone, one sweep per step, over odd and even calls."""
+    p = workloads.stefan_1024x4(Ste=0.5, nx=nx)[2] if problem == "stefan" else workloads.params(Ra=1e5, **RATES, **kw)
+    lat, ref = (start(nx, ny, p, prec, stream) for _ in range(2))
+    lbm.lbm_set_streaming(ref.h, lbm.LBM_STREAM_TWO_BUFFERS)
+    b = lbm.Batch(1, stream)
+    b.add(lat)
+    for n in (1, 3, 20, 135, 3, 135):
+        b.step(n)
+        ref.step(n)
+        for x, y in zip(lat.populations(), ref.populations()):
+            assert np.array_equal(x, y), (prec, problem, n)
+        for k, v in ref.fields().items():
+            assert np.array_equal(lat.fields()[k], v), (prec, problem, n, k)
+    b.close()
