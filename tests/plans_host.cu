@@ -3,6 +3,7 @@
 // describes a batch of n lattices (streaming: -1 as lbm_batch_create leaves it);
 // the output line holds the batch's plan and the first lattice's own:
 //     batch tile w h t  band threads rows | solo tile w h t  band threads rows
+//     | solo tiles, dynamic shared memory of one
 #include "lbm_api.cu"
 
 #include <iostream>
@@ -31,8 +32,10 @@ int main() {
         if (precision == LBM_FP64) batch_build<double>(&b);
         else batch_build<float>(&b);
         const lbm_s &h = lats[0];
-        std::printf("%d %d %d %d %d %d %d %d %d %d\n", b.tile.w, b.tile.h, b.tile.t, b.band.threads, b.band.rows,
-                    h.tile.w, h.tile.h, h.tile.t, h.band.threads, h.band.rows);
+        TileArgs tl{};
+        if (h.tile.t) tl = tile_args(&h, h.tile, h.tile.t, tile_cells(&h, h.tile.w, h.tile.h, h.tile.t, 1));
+        std::printf("%d %d %d %d %d %d %d %d %d %d %d %u\n", b.tile.w, b.tile.h, b.tile.t, b.band.threads, b.band.rows,
+                    h.tile.w, h.tile.h, h.tile.t, h.band.threads, h.band.rows, tl.tiles_x * tl.tiles_y, tl.smem);
     }
     return 0;
 }
