@@ -169,3 +169,11 @@ def test_batch_of_one(stream, prec, problem, kw, nx, ny):
         for k, v in ref.fields().items():
             assert np.array_equal(lat.fields()[k], v), (prec, problem, n, k)
     b.close()
+
+
+@pytest.mark.parametrize("every", [1, 2, 3, 4, 5])
+def test_bands_between_frequent_diagnostics(stream, every):
+    """Pieces too short for bands, or with an odd plain step: swept in place except for
+    the call's last; the fields of the step before are there after every call."""
+    compare(1025, 513, workloads.params(Ra=1e6, strip_center=0.6, **RATES), "fp32", stream, (1, 2, 3, 4, 12, 12, 13, 12),
+            every)
