@@ -329,8 +329,10 @@ TileArgs tile_args(const lbm_s *h, const TilePlan &plan, int T, int cells) {
 
 // Block size and rows per band of the band kernel for these lattices: cavities
 // with flow, FP32 arithmetic.  The block that wastes the fewest lanes on ragged
-// strips and halos; the fewest rows with which one wave of blocks holds all bands
-// (a band computes two rows more than it has).
+// strips and halos; the rows with the least waves of blocks x (rows + the two more a
+// band computes).  That is one wave, unless whole members leave too much of it
+// empty (256 x 256 x 128, us per step: one wave of 256 blocks FP32 143.8, BF16-SR 145.6;
+// three waves 104.1, 92.5; sweeps 177.6, 114.5).
 int band_strips(const lbm_s *h, int threads) {
     const int pairs = (h->nx + 1) / 2;
     int s = std::max(1, pairs / threads);
@@ -362,14 +364,28 @@ BandPlan band_plan(lbm_s *const *lats, size_t n) {
     }
     if (!plan.threads) return plan;
     const long long room = (long long)lats[0]->num_sms * (kBandWarps / (plan.threads / 32));
-    if (strips > room) {  // several waves: bands of 32 rows
-        plan.rows = 32;
-        return plan;
-    }
-    for (plan.rows = 4; plan.rows < tallest; ++plan.rows) {
-        long long blocks = 0;
-        for (size_t r = 0; r < n; ++r)
-            blocks += (long long)band_strips(lats[r], plan.threads) * ((lats[r]->ny + plan.rows - 1) / plan.rows);
+    // a wide lattice of 5 to 16 rows in L2, whose strips leave no room for a second band
+    // each: sweeps (us per step, bands and sweeps: 65536 x 16 21.1 and 16.0, 65536 x 8
+    // 12.4 and 11.6, 131072 x 8 19.3 and 17.0; but 65536 x 4 8.0 and 9.9, 131072 x 16
+    // 35.3 and 40.5)
+    if (n == 1 && 2 * strips > room && tallest > 4 && tallest <= 16 && (long long)lats[0]->nx * tallest <= 1 << 20)
+        return BandPlan();
+    const int highest = strips > room ? std::min(tallest, 64) : tallest;  // one wave may not be had
+    std::vector<int> each(n);
+    for (size_t r = 0; r < n; ++r) each[r] = band_strips(lats[r], plan.threads);
+    long long least = 1ll << 62;
+    for (int rows = std::min(4, highest); rows <= highest; ++rows) {
+        long long blocks = 0, longest = 0;
+        for (size_t r = 0; r < n; ++r) {
+            const int bands = (lats[r]->ny + rows - 1) / rows;
+            blocks += (long long)each[r] * bands;
+            longest = std::max(longest, (long long)(lats[r]->ny + bands - 1) / bands);
+        }
+        const long long cost = (blocks + room - 1) / room * (longest + 2);
+        if (cost <= least) {
+            least = cost;
+            plan.rows = rows;
+        }
         if (blocks <= room) break;
     }
     return plan;

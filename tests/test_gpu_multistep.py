@@ -177,3 +177,23 @@ def test_bands_between_frequent_diagnostics(stream, every):
     the call's last; the fields of the step before are there after every call."""
     compare(1025, 513, workloads.params(Ra=1e6, strip_center=0.6, **RATES), "fp32", stream, (1, 2, 3, 4, 12, 12, 13, 12),
             every)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16sr"])
+def test_batch_bands_in_several_waves(stream, prec):
+    """1200 members of 40 x 30: more bands than blocks that run at once."""
+    groups = []
+    for mode in (None, lbm.LBM_STREAM_TWO_BUFFERS):
+        lats = [lbm.Lattice(40, 30, workloads.params(Ra=1e5, strip_center=0.2 + 0.0005 * k, seed=k, init_amp=0.1, **RATES),
+                            precision=prec, stream=stream) for k in range(1200)]
+        b = lbm.Batch(len(lats), stream)
+        for lat in lats:
+            b.add(lat)
+        if mode is not None:
+            lbm.lbm_batch_set_streaming(b.b, mode)
+        for n in (3, 20, 7):
+            b.step(n)
+        b.close()
+        groups.append([lat.populations() for lat in lats[::173]])
+    for x, y in zip(*groups):
+        assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1]) and x[2] == y[2] == 30

@@ -62,3 +62,37 @@ def test_an_sm_holds_its_share_of_fp64_tiles_and_no_more(plans, problem, flow, s
         share = -(-solo["tiles"] // 152)
         assert solo["t"] >= 2 and solo["smem"] <= 230400
         assert share * (solo["smem"] + 1024 + 256) <= 228 * 1024 < (share + 1) * (solo["smem"] + 1024), size
+
+
+def band_cost(plan, nx, ny, n):
+    """(waves, waves x the rows a band computes) of n lattices on 152 SMs."""
+    pairs, threads = (nx + 1) // 2, plan["threads"]
+    s = max(1, pairs // threads)
+    while -(-pairs // s) + min(s - 1, 2) > threads:
+        s += 1
+    bands = -(-ny // plan["rows"])
+    waves = -(-n * s * bands // (152 * (12 // (threads // 32))))
+    return waves, waves * (-(-ny // bands) + 2)
+
+
+@pytest.mark.parametrize("prec,size,n,most", [
+    ("fp32", (256, 128), 256, 90), ("bf16sr", (256, 128), 256, 90), ("bf16sr", (128, 64), 512, 50),
+    ("fp32", (128, 64), 512, 50), ("fp16", (256, 128), 230, 90)])
+def test_bands_of_many_members_fill_their_waves(plans, prec, size, n, most):
+    """One band per member left 44 % of a wave empty (a cost of 130 for 256 x 128, 66
+    for 128 x 64)."""
+    batch = plans(prec, workloads.CAVITY, 1, [size] * n)[0]
+    assert batch["threads"] > 0 and band_cost(batch, *size, n)[1] <= most
+
+
+@pytest.mark.parametrize("nx,ny", [(2048, 1024), (1024, 1024), (1500, 700), (700, 500), (3000, 3000), (16, 65535), (5000, 200),
+                                   (4500, 2), (8192, 64)])
+def test_bands_of_one_lattice_take_one_wave(plans, nx, ny):
+    solo = plans("fp32", workloads.CAVITY, 1, [(nx, ny)])[1]
+    assert solo["threads"] > 0 and 1 <= solo["rows"] and band_cost(solo, nx, ny, 1)[0] == 1
+
+
+@pytest.mark.parametrize("nx,ny,bands", [(65536, 8, False), (65536, 16, False), (131072, 8, False), (65536, 4, True),
+                                         (131072, 4, True), (131072, 16, True), (32768, 16, True), (262144, 2, True)])
+def test_wide_lattices_of_few_rows(plans, nx, ny, bands):
+    assert (plans("fp32", workloads.CAVITY, 1, [(nx, ny)])[1]["threads"] > 0) == bands
