@@ -150,8 +150,8 @@ int lbm_set_diag_every(lbm_handle h, long long k);
  * see lbm_set_streaming, depend on graph_chunk only): rows of the lattice walked by
  * each thread of a block (1 to 1024, default 1, or 2 with 16-bit storage);
  * the distance, in rows, at which each block asks L2 to prefetch a later
- * block's tile rows (0 = off, default 16, or 0 with 16-bit storage); and
- * graph_chunk, the longest piece
+ * block's tile rows (0 = off, default 16; with 16-bit storage 0, or 32 where a
+ * population buffer exceeds 96 MB); and graph_chunk, the longest piece
  * of sweeps lbm_step replays from a CUDA graph (0 = launch every sweep
  * directly; default 128).  Successive sweeps visit the lattice's row bands in
  * opposite directions (the two wall bands first), each starting on the rows
@@ -349,8 +349,10 @@ int lbm_batch_count(lbm_batch b, int *count);
 int lbm_batch_step(lbm_batch b, long long n);
 
 /* Launch shape of the batch's step kernel: rows of a member walked by each
- * block (0 = the default: 2, or 3 with 16-bit storage; up to 1024), the L2
- * prefetch distance in rows (-1 = the default: 0),
+ * block (0 = the default: 2; with 16-bit storage 3 for cavities with flow, else 4;
+ * up to 1024), the L2 prefetch distance in rows (-1 = the default: 4, but for
+ * cavities with flow other than LBM_FP64 0 unless the storage is 16-bit and the
+ * members' populations exceed 64 MB),
  * and interleave = 1 (the default) to number the blocks of a one-size batch
  * member after member (block b belongs to member b mod n) instead of member
  * by member (0; a batch whose members' block counts differ is always member

@@ -40,10 +40,13 @@ constexpr int kDefaultPrefetch = 16;  // L2 prefetch distance in rows (tuned on 
 // 16-bit storage: 2 rows per thread spread a thread's set-up (indices, the rounding
 // seed, the block's tail), and with two cells per thread the loads in flight need no
 // prefetch (2048 x 1024 FP16-SR on GB300, us per step: 1 / 2 / 3 rows 22.6 / 21.1 /
-// 21.2; 2 rows, prefetch 0 / 16 / 48: 21.1 / 21.4 / 21.4).  FP32 is memory bound and
+// 21.2; 2 rows, prefetch 0 / 16 / 48: 21.1 / 21.4 / 21.4), unless the buffer outgrows
+// L2's share of it (prefetch 0 / 32: 2048 x 1536, 113 MB, BF16-SR 31.5 / 30.9; 3000 x
+// 3000 FP16 103.0 / 94.8; 4096 x 4096 193.3 / 174.0).  FP32 is memory bound and
 // fastest at 1 row (35.9; 2 rows 36.7).
 constexpr int kDefaultRows16 = 2;
-constexpr int kDefaultPrefetch16 = 0;
+constexpr int kDefaultPrefetch16 = 32;
+constexpr size_t kPrefetchFrom16 = 96u << 20;  // bytes of one buffer; below: off
 constexpr int kDefaultGraphChunk = 128;  // longest graph-replayed piece (0 = direct launches)
 constexpr int kGraphCache = 16;          // cached piece graphs per handle
 
@@ -191,6 +194,8 @@ void dev_free(lbm_s *h, void *p) {
 size_t buffer_bytes(const lbm_s *h) {
     return (size_t)h->ntx * (size_t)h->ny * (size_t)kRS * h->esize;
 }
+
+int default_prefetch16(const lbm_s *h) { return buffer_bytes(h) > kPrefetchFrom16 ? kDefaultPrefetch16 : 0; }
 
 // Resident blocks per SM of the staged sweep (128 threads, 64 registers,
 // about 25 KB of shared memory each).
@@ -861,7 +866,7 @@ int lbm_create(int nx, int ny, int precision, void *cuda_stream, lbm_handle *out
     h->ntx = (nx + kTW - 1) / kTW;
     if (h->esize == 2) {
         h->rows = kDefaultRows16;
-        h->prefetch = kDefaultPrefetch16;
+        h->prefetch = default_prefetch16(h);
     }
     // One-buffer streaming where it pays: a step whose working set is one
     // buffer finds more of the previous step's rows in L2, and the local sweep
@@ -1330,8 +1335,8 @@ struct lbm_batch_s {
     std::vector<int> host_mstarts;
     int mblocks = 0;
     int uniform = 0;          // blocks per member when all members have the same count
-    int rows = 0;             // launch shape: rows per block (0: 2, or 3 with 16-bit storage),
-    int prefetch = -1;        // L2 prefetch distance (-1: off),
+    int rows = 0;             // launch shape: rows per block (0: batch_shape's),
+    int prefetch = -1;        // L2 prefetch distance (-1: batch_shape's),
     int interleave = 1;       // interleaved block order (uniform batches only; see batch_kernel)
     int streaming = -1;       // lbm_batch_set_streaming; -1: one buffer, two for FP64
     bool dirty = true;        // table must be rebuilt and uploaded
@@ -1382,12 +1387,27 @@ size_t entry_bytes() { return sizeof(BatchEntry<real>); }
 bool batch_sweeps_chosen(const lbm_batch_s *b) { return b->streaming >= 0; }
 
 // Default launch shape of a batch, whatever the members' own lbm_set_launch
-// settings: 2 rows per block (3 with 16-bit storage), no L2 prefetch, blocks of a
-// one-size batch interleaved over the members -- the fastest shapes for 32 cavities
-// of 256 x 128 on GB300 (us per step at 1 / 2 / 3 / 4 rows: FP32 18.9 / 17.7 / 18.0 /
-// 19.2, BF16-SR 15.6 / 15.1 / 14.7 / 14.9; prefetch 4: 18.0 and 14.9).  Results do
-// not depend on it.
-constexpr int kBatchRows32 = 2, kBatchRows16 = 3, kBatchPrefetch32 = 0, kBatchPrefetch16 = 0;
+// settings; blocks of a one-size batch are interleaved over the members.  The fastest
+// shapes on GB300; results do not depend on them.
+// - Two cells per thread (cavities with flow in FP32 arithmetic): 2 rows per block, 3
+//   with 16-bit storage, no L2 prefetch (32 x 256 x 128, us per step at 1 / 2 / 3 / 4 rows:
+//   FP32 18.9 / 17.7 / 18.0 / 19.2, BF16-SR 15.6 / 15.1 / 14.7 / 14.9; prefetch 4: 18.0
+//   and 14.9), but 4 rows ahead for 16-bit members of more than 64 MB together (one buffer
+//   each; BF16-SR, prefetch 0 / 4: 48 x 256 x 128, 57 MB, 20.8 / 20.9; 96 40.9 / 39.7; 32
+//   x 512 x 256 53.1 / 49.9; a call of one step, 64 x 256 x 128, 75 MB, 42.1 / 40.6).
+// - One cell per thread: 2 rows, 4 with 16-bit storage, 4 rows ahead (32 x 512 x 256
+//   periodic with flow, at prefetch 0 and 4: FP32 102.1 and 95.3; FP16, 3 rows and none
+//   ahead against 4 and 4: 70.6 and 67.2).
+struct BatchShape {
+    int rows, prefetch;
+};
+BatchShape batch_shape(const lbm_batch_s *b) {
+    const bool half = b->precision != LBM_FP32 && b->precision != LBM_FP64;
+    if (b->problem != LBM_CAVITY || !b->flow || b->precision == LBM_FP64) return {half ? 4 : 2, 4};
+    size_t total = 0;
+    for (const lbm_s *h : b->members) total += buffer_bytes(h);
+    return {half ? 3 : 2, half && total > (64u << 20) ? 4 : 0};
+}
 
 template <typename real>
 void batch_build(lbm_batch_s *b) {
@@ -1408,16 +1428,17 @@ void batch_build(lbm_batch_s *b) {
     if (b->tile.t == 0 && (b->precision == LBM_FP32 || 2 * narrow > (int)b->members.size()))
         b->band = band_plan(b->members.data(), b->members.size());
     b->host_mstarts.assign(b->members.size(), 0);
+    const BatchShape shape = batch_shape(b);
     for (size_t r = 0; r < b->members.size(); ++r) {
         lbm_s *h = b->members[r];
-        const int rows = b->rows > 0 ? b->rows : (h->esize == 2 ? kBatchRows16 : kBatchRows32);
+        const int rows = b->rows > 0 ? b->rows : shape.rows;
         const int gy = (h->ny + rows - 1) / rows;
         BatchEntry<real> e{};
         for (int p = 0; p < 2; ++p) {
             e.a[p] = make_args<real>(h, h->buf[p], h->buf[p ^ 1]);
             e.a[p].parity = p;
             e.a[p].rows = rows;
-            e.a[p].prefetch = b->prefetch >= 0 ? b->prefetch : (h->esize == 2 ? kBatchPrefetch16 : kBatchPrefetch32);
+            e.a[p].prefetch = b->prefetch >= 0 ? b->prefetch : shape.prefetch;
             e.a[p].nq = h->p.problem == LBM_CAVITY ? (int)h->grid.x : gy;
         }
         e.start = start;

@@ -191,7 +191,7 @@ def lbm_set_diag_every(h, k: int) -> None:
 
 def lbm_set_launch(h, rows: int = 1, prefetch: int = 16, graph_chunk: int = 128) -> None:
     """Launch shape (the defaults are the library's FP32 ones; with 16-bit
-    storage the library starts from 2 rows and no prefetch)."""
+    storage the library starts from 2 rows and no prefetch, or 32 on large lattices)."""
     _check(lib().lbm_set_launch(h, int(rows), int(prefetch), int(graph_chunk)), h)
 
 

@@ -3,7 +3,9 @@
 // describes a batch of n lattices (streaming: -1 as lbm_batch_create leaves it);
 // the output line holds the batch's plan and the first lattice's own:
 //     batch tile w h t  band threads rows | solo tile w h t  band threads rows
-//     | solo tiles, dynamic shared memory of one
+//     | solo tiles, dynamic shared memory of one | default prefetch of the first lattice
+//     with 16-bit storage, and of the batch
+//     | rows per block of the batch's sweeps
 #include "lbm_api.cu"
 
 #include <iostream>
@@ -29,13 +31,19 @@ int main() {
             plan_steps(&h);
             b.members.push_back(&h);
         }
-        if (precision == LBM_FP64) batch_build<double>(&b);
-        else batch_build<float>(&b);
+        int prefetch = 0;
+        if (precision == LBM_FP64) {
+            batch_build<double>(&b);
+        } else {
+            batch_build<float>(&b);
+            prefetch = reinterpret_cast<BatchEntry<float> *>(b.host_entries.data())->a[0].prefetch;
+        }
         const lbm_s &h = lats[0];
         TileArgs tl{};
         if (h.tile.t) tl = tile_args(&h, h.tile, h.tile.t, tile_cells(&h, h.tile.w, h.tile.h, h.tile.t, 1));
-        std::printf("%d %d %d %d %d %d %d %d %d %d %d %u\n", b.tile.w, b.tile.h, b.tile.t, b.band.threads, b.band.rows,
-                    h.tile.w, h.tile.h, h.tile.t, h.band.threads, h.band.rows, tl.tiles_x * tl.tiles_y, tl.smem);
+        std::printf("%d %d %d %d %d %d %d %d %d %d %d %u %d %d %d\n", b.tile.w, b.tile.h, b.tile.t, b.band.threads, b.band.rows,
+                    h.tile.w, h.tile.h, h.tile.t, h.band.threads, h.band.rows, tl.tiles_x * tl.tiles_y, tl.smem,
+                    default_prefetch16(&h), prefetch, batch_shape(&b).rows);
     }
     return 0;
 }

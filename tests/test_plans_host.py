@@ -23,7 +23,7 @@ def plans(tmp_path_factory):
         out = subprocess.run([exe], input=" ".join(map(str, line)), capture_output=True, text=True, check=True).stdout
         keys = ("w", "h", "t", "threads", "rows")
         v = [int(x) for x in out.split()]
-        return dict(zip(keys, v[:5])), dict(zip(keys + ("tiles", "smem"), v[5:]))
+        return dict(zip(keys, v[:5])), dict(zip(keys + ("tiles", "smem", "prefetch16", "batch_prefetch", "batch_rows"), v[5:]))
 
     return ask
 
@@ -96,3 +96,22 @@ def test_bands_of_one_lattice_take_one_wave(plans, nx, ny):
                                          (131072, 4, True), (131072, 16, True), (32768, 16, True), (262144, 2, True)])
 def test_wide_lattices_of_few_rows(plans, nx, ny, bands):
     assert (plans("fp32", workloads.CAVITY, 1, [(nx, ny)])[1]["threads"] > 0) == bands
+
+
+@pytest.mark.parametrize("prec,size,n,solo_pf,batch_pf", [
+    ("bf16sr", (2048, 1024), 1, 0, 4), ("fp16", (2048, 1536), 1, 32, 4), ("fp16", (4096, 4096), 1, 32, 4),
+    ("bf16", (256, 128), 48, 0, 0), ("fp16sr", (256, 128), 64, 0, 4), ("fp32", (2048, 1024), 2, 0, 0)])
+def test_16_bit_storage_beyond_l2_prefetches(plans, prec, size, n, solo_pf, batch_pf):
+    solo = plans(prec, workloads.CAVITY, 1, [size] * n)[1]
+    assert solo["batch_prefetch"] == batch_pf
+    if prec != "fp32":
+        assert solo["prefetch16"] == solo_pf
+
+
+@pytest.mark.parametrize("prec,problem,flow,rows,prefetch", [
+    ("fp32", workloads.CAVITY, 1, 2, 0), ("bf16sr", workloads.CAVITY, 1, 3, 0), ("fp32", workloads.STEFAN, 1, 2, 4),
+    ("fp16", workloads.STEFAN, 0, 4, 4), ("bf16", workloads.CAVITY, 0, 4, 4), ("fp32", workloads.CAVITY, 0, 2, 4)])
+def test_batch_shapes(plans, prec, problem, flow, rows, prefetch):
+    """Members stepped one cell per thread keep their own shape."""
+    solo = plans(prec, problem, flow, [(256, 128)] * 32)[1]
+    assert (solo["batch_rows"], solo["batch_prefetch"]) == (rows, prefetch)
