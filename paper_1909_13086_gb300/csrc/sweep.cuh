@@ -1726,10 +1726,13 @@ __host__ __device__ constexpr int sweep_threads() {
 // arguments sit in shared memory and take more registers).  Two cells per thread,
 // us per step at 8 / 10 / 12 blocks: 2048 x 1024 FP32 one buffer 36.4 / 35.9 / 36.2,
 // FP16-SR 21.7 / 21.6 / 21.1, 1001 x 701 BF16-SR 9.1 / 9.1 / 8.8; 32 x 256 x 128
-// batches FP32 18.2 / 17.7 / -, BF16-SR 15.0 / 14.7 / 15.7.
+// batches FP32 18.2 / 17.7 / -, BF16-SR 15.0 / 14.7 / 15.7.  The FP32 batch's diagnostic
+// sweep spills at 10 (calls of one step, 10 / 8: 32 x 256 x 128 32.5 / 30.9, 8 x 1024 x 512
+// 99.2 / 98.5).
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM, bool BATCH>
 __host__ __device__ constexpr int sweep_blocks() {
-    if (takes_two<real, PROB, FLOW, MODE, SM>()) return Store<S>::kDev && !BATCH ? 12 : 10;
+    if (takes_two<real, PROB, FLOW, MODE, SM>())
+        return Store<S>::kDev ? (BATCH ? 10 : 12) : (BATCH && MODE == kSweepDiag ? 8 : 10);
     return sizeof(real) == 4 ? 1024 / kTW : 1;
 }
 
