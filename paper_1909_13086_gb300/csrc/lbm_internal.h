@@ -28,9 +28,9 @@ enum Mode {
 //            goes to its own slot i: the pull layout again.
 // Each cell reads and writes the same 18 locations in either sweep, so no two
 // cells touch one location, and the populations are those of the pull sweeps.
-// kPullNarrow is kPull with accesses of one value each, for a caller's buffers that are
-// not on 8-byte boundaries (launch_mode).
-enum Streaming { kPull = 0, kAAPush = 1, kAALocal = 2, kPullNarrow = 3 };
+// The narrow forms are the same sweeps with one cell per thread and accesses of one value
+// each, where the others take two (launch_mode).
+enum Streaming { kPull = 0, kAAPush = 1, kAALocal = 2, kPullNarrow = 3, kAAPushNarrow = 4, kAALocalNarrow = 5 };
 
 // Population layout in device memory ("tile-major structure of arrays").
 // The lattice is cut into column tiles of kTW cells.  Within a tile, each row

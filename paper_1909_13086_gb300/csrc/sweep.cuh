@@ -1710,13 +1710,13 @@ __device__ __forceinline__ void sweep_block_two(const SweepArgs<float> &a, const
 // 8-byte boundaries).
 template <typename real, int PROB, bool FLOW, int MODE, int SM = kPull>
 __host__ __device__ constexpr bool takes_two() {
-    return sizeof(real) == 4 && PROB == kCavity && FLOW && MODE != kFields && SM != kPullNarrow;
+    return sizeof(real) == 4 && PROB == kCavity && FLOW && MODE != kFields && SM < kPullNarrow;
 }
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM>
 __device__ __forceinline__ void sweep_any(const SweepArgs<real> &a, const int bx, const int by, const int gx,
                                           double *sh) {
     if constexpr (takes_two<real, PROB, FLOW, MODE, SM>()) sweep_block_two<S, MODE, SM>(a, bx, by, gx, sh);
-    else sweep_block<real, S, PROB, FLOW, MODE, SM == kPullNarrow ? kPull : SM>(a, bx, by, gx, sh);
+    else sweep_block<real, S, PROB, FLOW, MODE, (SM >= kPullNarrow ? SM - kPullNarrow : SM)>(a, bx, by, gx, sh);
 }
 template <typename real, int PROB, bool FLOW, int MODE, int SM = kPull>
 __host__ __device__ constexpr int sweep_threads() {
@@ -2267,22 +2267,41 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// A sweep, by one cell per thread although two would do:
+// - where pairs leave half of the threads of all blocks idle, or three in four of every
+//   second block's (us per step, two cells and one: 16 x 65535 BF16-SR 84.8 and 51.2, 64 x
+//   16384 FP16 22.8 and 16.3, 160 x 6500 18.8 and 14.2, FP32 in one buffer 21.4 and 18.9).
+//   FP32 over two buffers and the diagnostic sweeps gain nothing by it;
+// - on a caller's FP32 buffers off 8-byte boundaries (lbm_step_static).
+template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM>
+static cudaError_t launch_sweep(const SweepArgs<real> &a, dim3 grid, cudaStream_t s, bool pdl) {
+    if constexpr (takes_two<real, PROB, FLOW, MODE, SM>()) {
+        bool one = false;
+        if constexpr (MODE == kSweep) one = a.nx <= kTW / 2 || (a.nx > kTW && a.nx <= kTW + kTW / 4);
+        else one = (reinterpret_cast<uintptr_t>(a.src) | reinterpret_cast<uintptr_t>(a.dst)) % 8 != 0;
+        // FP32: kPull of kSweepDiag, the others of kSweep; 16-bit: all of kSweep
+        if constexpr (Store<S>::kDev ? MODE == kSweep : (MODE == kSweep) == (SM != kPull)) {
+            if (one)
+                return launch_k(lattice_kernel<real, S, PROB, FLOW, MODE, SM + kPullNarrow>, grid, dim3(kTW), s, pdl, a);
+        }
+    }
+    return launch_k(lattice_kernel<real, S, PROB, FLOW, MODE, SM>, grid, dim3(sweep_threads<real, PROB, FLOW, MODE, SM>()),
+                    s, pdl, a);
+}
+
 template <typename real, typename S, int PROB, bool FLOW>
 static cudaError_t launch_mode(const SweepArgs<real> &a, int mode, dim3 grid, dim3 block,
                                cudaStream_t s, bool pdl, int streaming) {
-    const dim3 threads(sweep_threads<real, PROB, FLOW, kSweep>());  // of a sweep; `block`: of the other kernels
     if (streaming == kAAPush || streaming == kAALocal) {  // one-buffer streaming: sweeps only
         if (a.src != a.dst || a.staged) return cudaErrorInvalidValue;
         const bool push = streaming == kAAPush;
         switch (mode) {
             case kSweep:
-                return push ? launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep, kAAPush>, grid, threads, s, pdl, a)
-                            : launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep, kAALocal>, grid, threads, s, pdl, a);
+                return push ? launch_sweep<real, S, PROB, FLOW, kSweep, kAAPush>(a, grid, s, pdl)
+                            : launch_sweep<real, S, PROB, FLOW, kSweep, kAALocal>(a, grid, s, pdl);
             case kSweepDiag:
-                return push ? launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kAAPush>, grid, threads, s, pdl,
-                                       a)
-                            : launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kAALocal>, grid, threads, s,
-                                       pdl, a);
+                return push ? launch_sweep<real, S, PROB, FLOW, kSweepDiag, kAAPush>(a, grid, s, pdl)
+                            : launch_sweep<real, S, PROB, FLOW, kSweepDiag, kAALocal>(a, grid, s, pdl);
             default: return cudaErrorInvalidValue;
         }
     }
@@ -2304,15 +2323,8 @@ static cudaError_t launch_mode(const SweepArgs<real> &a, int mode, dim3 grid, di
         }
     }
     switch (mode) {
-        case kSweep: return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweep>, grid, threads, s, pdl, a);
-        case kSweepDiag:
-            if constexpr (takes_two<real, PROB, FLOW, kSweepDiag>() && !Store<S>::kDev) {
-                // lbm_step_static's buffers are the caller's
-                if ((reinterpret_cast<uintptr_t>(a.src) | reinterpret_cast<uintptr_t>(a.dst)) % 8)
-                    return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag, kPullNarrow>, grid, dim3(kTW), s,
-                                    pdl, a);
-            }
-            return launch_k(lattice_kernel<real, S, PROB, FLOW, kSweepDiag>, grid, threads, s, pdl, a);
+        case kSweep: return launch_sweep<real, S, PROB, FLOW, kSweep, kPull>(a, grid, s, pdl);
+        case kSweepDiag: return launch_sweep<real, S, PROB, FLOW, kSweepDiag, kPull>(a, grid, s, pdl);
         case kFields: lattice_kernel<real, S, PROB, FLOW, kFields><<<grid, block, 0, s>>>(a); break;
         default: return cudaErrorInvalidValue;
     }

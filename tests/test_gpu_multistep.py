@@ -197,3 +197,20 @@ def test_batch_bands_in_several_waves(stream, prec):
         groups.append([lat.populations() for lat in lats[::173]])
     for x, y in zip(*groups):
         assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1]) and x[2] == y[2] == 30
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16", "bf16", "fp16sr", "bf16sr"])
+@pytest.mark.parametrize("nx", [2, 3, 33, 64, 65, 129, 160, 161])
+def test_narrow_lattices_by_every_path(stream, prec, nx):
+    """Widths around those where sweeps take one cell per thread: several steps per
+    launch, one buffer and two buffers end in the same bits."""
+    p = workloads.params(Ra=1e5, strip_center=0.4, strip_width=0.5, **RATES)
+    lats = [start(nx, 37, p, prec, stream) for _ in range(3)]
+    lbm.lbm_set_streaming(lats[1].h, lbm.LBM_STREAM_ONE_BUFFER)
+    lbm.lbm_set_streaming(lats[2].h, lbm.LBM_STREAM_TWO_BUFFERS)
+    for n in (1, 2, 7, 20, 7, 20):
+        for lat in lats:
+            lbm.lbm_set_diag_every(lat.h, 5)
+            lat.step(n)
+        assert_same(lats[0], lats[2], (prec, nx, n))
+        assert_same(lats[1], lats[2], (prec, nx, n))
