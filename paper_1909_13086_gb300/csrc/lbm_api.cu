@@ -281,12 +281,15 @@ TilePlan tile_plan(lbm_s *const *lats, size_t n, bool batch) {
                 if ((long long)m->nx * m->ny > (long long)big->nx * big->ny) big = m;
             }
             const double waves = (double)((tiles + h->num_sms - 1) / h->num_sms);
+            // the steps of a launch: the core's, and each on one more ring of halo
+            double steps = std::max(least, waves * per_cell * tile_cells(big, w, hh, 1, 1));
+            if (steps >= best) continue;  // the least a step of this core can take
             for (int T = 2; T <= kTileMaxSteps; ++T) {
                 const size_t smem = tile_smem(h, w, hh, T);
                 if (smem > kTileSmemMax || (long long)(w + 2 * T) * (w + 2 * T) * (hh + 2 * T) >= (1 << 20)) break;
                 const double resident = std::max(1.0, std::floor(kTileSmemMax / (double)smem));
-                double ns = launch * std::ceil(waves / resident);
-                for (int t = 1; t <= T; ++t) ns += std::max(least, waves * per_cell * tile_cells(big, w, hh, T, t));
+                steps += std::max(least, waves * per_cell * tile_cells(big, w, hh, T, 1));
+                const double ns = launch * std::ceil(waves / resident) + steps;
                 if (ns / T < best) {
                     best = ns / T;
                     plan.w = w;
