@@ -297,11 +297,12 @@ __device__ __forceinline__ void invert(double H, double Lh, double inv_Lh, doubl
 // is 1e-5); in FP64 two Newton steps y <- y + y (1 - x y) from the hardware's
 // approximation (2^-20 or better, so the second leaves rounding error only), four
 // operations of the FP64 pipe against the exact quotient's eight or more, which
-// zeros, subnormals, infinities and NaN still take.
+// zeros, subnormals, infinities and NaN still take, and numbers whose reciprocal, or
+// the approximation to it, may be such (below 2^-1021, from 2^1021).
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double recip(double x) {
     const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-    if (e - 2u > 0x7fbu) return 1.0 / x;
+    if (e - 2u > 0x7f9u) return 1.0 / x;  // e: 2 .. 0x7fb go on
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     y = fma(y, fma(-x, y, 1.0), y);
