@@ -198,19 +198,19 @@ int lbm_set_launch(lbm_handle h, int rows_per_block, int prefetch_rows, int grap
  * still in L2 when the next one reads it.  Both buffers stay allocated.  The
  * staged 16-bit sweep and lbm_step_static always use two buffers; a batch has
  * its own setting (lbm_batch_set_streaming).
- * Until this is called the library chooses: small lattices (FP32 and 16-bit
- * storage up to 2^19 cells, FP64 up to 2^15 with flow and 2^14 without; a Stefan
+ * LBM_STREAM_AUTO (the default) leaves the choice to the library: small lattices (FP32
+ * and 16-bit storage up to 2^19 cells, FP64 up to 2^15 with flow and 2^14 without; a Stefan
  * lattice up to 32 rows high) advance several steps per launch, each block keeping its part of
  * the lattice in shared memory for up to 16 steps and computing its neighbours'
  * edge cells itself (256 x 128 FP32: 5.4 -> 1.6 us per step); larger FP32
  * cavities with flow take two steps per pass over memory (2048 x 1024: 35.9 ->
- * 26.4).  A call's last step and the diagnostic steps are sweeps.  Calling this,
- * with either mode, asks for one sweep per step.
- * Otherwise the default is one buffer (2048 x 1024 cavity on GB300: FP32
- * 41.4 -> 36.6 us per step, BF16-SR 26.1 -> 24.4 us), except for LBM_FP64,
- * which is bound by its arithmetic and keeps two buffers.  Takes effect at the
+ * 26.4).  A call's last step and the diagnostic steps are sweeps.  All others are
+ * swept in one buffer (2048 x 1024 cavity on GB300: BF16-SR 26.1 -> 24.4 us per
+ * step), except for LBM_FP64, which is bound by its arithmetic and keeps two buffers.
+ * The other two modes ask for one sweep per step.  Takes effect at the
  * next lbm_step.  Errors: LBM_ERR_ARG. */
 enum { LBM_STREAM_TWO_BUFFERS = 0, LBM_STREAM_ONE_BUFFER = 1 };
+enum { LBM_STREAM_AUTO = -1 };
 int lbm_set_streaming(lbm_handle h, int mode);
 
 /* Sweep kernel for 16-bit storage.  The staged sweep (an option for LBM_FP16,
@@ -366,9 +366,10 @@ int lbm_batch_set_launch(lbm_batch b, int rows_per_block, int prefetch_rows, int
  * buffer, and the closing steps run over two buffers, so that between calls
  * every member's state is the two-buffer one (results do not depend on the
  * mode, bit for bit; members may be stepped alone or in other batches between
- * calls).  Until this is called a batch of cavities with flow takes several steps
- * per launch, as a single lattice does (lbm_set_streaming), and any other follows
- * its precision: one buffer, two for LBM_FP64.  Synchronises the batch's stream.  Errors: LBM_ERR_ARG. */
+ * calls).  With LBM_STREAM_AUTO, the default, a batch of cavities with flow takes several
+ * steps per launch, as a single lattice does (lbm_set_streaming; not LBM_FP64, and with
+ * 16-bit storage larger batches only where most members are at most 384 columns wide), and
+ * any other follows its precision: one buffer, two for LBM_FP64.  Synchronises the batch's stream.  Errors: LBM_ERR_ARG. */
 int lbm_batch_set_streaming(lbm_batch b, int mode);
 
 /* Autotuner for a batch: times rows per block (1, 2, 3, 4) x prefetch distance

@@ -195,6 +195,10 @@ size_t buffer_bytes(const lbm_s *h) {
     return (size_t)h->ntx * (size_t)h->ny * (size_t)kRS * h->esize;
 }
 
+int default_streaming(int precision) {
+    return precision == LBM_FP64 ? LBM_STREAM_TWO_BUFFERS : LBM_STREAM_ONE_BUFFER;
+}
+
 int default_prefetch16(const lbm_s *h) { return buffer_bytes(h) > kPrefetchFrom16 ? kDefaultPrefetch16 : 0; }
 
 // Resident blocks per SM of the staged sweep (128 threads, 64 registers,
@@ -875,8 +879,8 @@ int lbm_create(int nx, int ny, int precision, void *cuda_stream, lbm_handle *out
     // buffer finds more of the previous step's rows in L2, and the local sweep
     // reads and writes aligned own slots (2048 x 1024 cavity on GB300: FP32
     // 41.4 -> 36.5 us per step, BF16-SR 26.1 -> 24.2, FP16-SR 26.5 -> 24.5).
-    // FP64 is bound by its arithmetic (698 us per step either way).
-    h->streaming = precision == LBM_FP64 ? LBM_STREAM_TWO_BUFFERS : LBM_STREAM_ONE_BUFFER;
+    // FP64 is bound by its arithmetic (about 490 us per step either way).
+    h->streaming = default_streaming(precision);
     set_grid(h);
     h->alloc = g_alloc;
     h->release = g_free;
@@ -1071,11 +1075,13 @@ int lbm_set_staging(lbm_handle h, int bands) {
 }
 
 int lbm_set_streaming(lbm_handle h, int mode) {
-    if (!h || (mode != LBM_STREAM_TWO_BUFFERS && mode != LBM_STREAM_ONE_BUFFER))
-        return set_err(h, LBM_ERR_ARG, "mode must be LBM_STREAM_TWO_BUFFERS or LBM_STREAM_ONE_BUFFER");
+    if (!h || (mode != LBM_STREAM_AUTO && mode != LBM_STREAM_TWO_BUFFERS && mode != LBM_STREAM_ONE_BUFFER))
+        return set_err(h, LBM_ERR_ARG,
+                       "mode must be LBM_STREAM_AUTO, LBM_STREAM_TWO_BUFFERS or LBM_STREAM_ONE_BUFFER");
     drop_graphs(h);
-    h->streaming_chosen = true;
-    h->streaming = mode;  // between calls buf[cur] always holds the pull layout (phase 0)
+    h->streaming_chosen = mode != LBM_STREAM_AUTO;
+    // between calls buf[cur] always holds the pull layout (phase 0)
+    h->streaming = h->streaming_chosen ? mode : default_streaming(h->precision);
     return LBM_OK;
 }
 
@@ -1341,7 +1347,7 @@ struct lbm_batch_s {
     int rows = 0;             // launch shape: rows per block (0: batch_shape's),
     int prefetch = -1;        // L2 prefetch distance (-1: batch_shape's),
     int interleave = 1;       // interleaved block order (uniform batches only; see batch_kernel)
-    int streaming = -1;       // lbm_batch_set_streaming; -1: one buffer, two for FP64
+    int streaming = LBM_STREAM_AUTO;  // lbm_batch_set_streaming
     bool dirty = true;        // table must be rebuilt and uploaded
     int precision = -1, problem = -1, flow = -1;
     int graph_chunk = 128;    // longest graph-replayed piece; even, so that every
@@ -1387,7 +1393,7 @@ void batch_drop_graph(lbm_batch_s *b) {
 template <typename real>
 size_t entry_bytes() { return sizeof(BatchEntry<real>); }
 
-bool batch_sweeps_chosen(const lbm_batch_s *b) { return b->streaming >= 0; }
+bool batch_sweeps_chosen(const lbm_batch_s *b) { return b->streaming != LBM_STREAM_AUTO; }
 
 // Default launch shape of a batch, whatever the members' own lbm_set_launch
 // settings; blocks of a one-size batch are interleaved over the members.  The fastest
@@ -1537,7 +1543,8 @@ int batch_steps(lbm_batch_s *b, long long n) {
     // in each member's buffer parity[r]; the last one or two run over the two
     // buffers, so that between calls every member's state is the two-buffer one.
     const bool multi = !batch_sweeps_chosen(b) && (b->tile.t > 0 || b->band.threads > 0);
-    const bool one = !multi && (b->streaming < 0 ? b->precision != LBM_FP64 : b->streaming == LBM_STREAM_ONE_BUFFER);
+    const int streaming = batch_sweeps_chosen(b) ? b->streaming : default_streaming(b->precision);
+    const bool one = !multi && streaming == LBM_STREAM_ONE_BUFFER;
     int launches = 0;  // of several-step pieces: the buffers they have changed
     const long long aa = (one && n >= 3) ? ((n & 1) ? n - 1 : n - 2) : 0;
     auto direct = [&](long long from, long long len, bool diag, bool ob) -> int {
@@ -1767,9 +1774,9 @@ int lbm_batch_set_launch(lbm_batch b, int rows_per_block, int prefetch_rows, int
 }
 
 int lbm_batch_set_streaming(lbm_batch b, int mode) {
-    if (!b || (mode != LBM_STREAM_TWO_BUFFERS && mode != LBM_STREAM_ONE_BUFFER))
-        return batch_err(LBM_ERR_ARG,
-                         "lbm_batch_set_streaming: mode must be LBM_STREAM_TWO_BUFFERS or LBM_STREAM_ONE_BUFFER");
+    if (!b || (mode != LBM_STREAM_AUTO && mode != LBM_STREAM_TWO_BUFFERS && mode != LBM_STREAM_ONE_BUFFER))
+        return batch_err(LBM_ERR_ARG, "lbm_batch_set_streaming: mode must be LBM_STREAM_AUTO, "
+                                      "LBM_STREAM_TWO_BUFFERS or LBM_STREAM_ONE_BUFFER");
     if (b->stream) cudaStreamSynchronize(b->stream);  // no captured piece may be in flight
     batch_drop_graph(b);
     b->streaming = mode;

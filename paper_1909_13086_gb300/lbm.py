@@ -23,7 +23,7 @@ LBM_OK, LBM_ERR_ARG, LBM_ERR_OOM, LBM_ERR_CUDA, LBM_ERR_DIVERGED, LBM_ERR_STATE,
     0, -1, -2, -3, -4, -5, -6
 LBM_FP64, LBM_FP32, LBM_FP16, LBM_BF16, LBM_FP16_SR, LBM_BF16_SR = 0, 1, 2, 3, 4, 5
 LBM_CAVITY, LBM_STEFAN = 0, 1
-LBM_STREAM_TWO_BUFFERS, LBM_STREAM_ONE_BUFFER = 0, 1
+LBM_STREAM_AUTO, LBM_STREAM_TWO_BUFFERS, LBM_STREAM_ONE_BUFFER = -1, 0, 1
 FIELD_BITS = {"H": 1, "T": 2, "fl": 4, "ux": 8, "uy": 16, "rho": 32}
 FIELD_NAMES = ("H", "T", "fl", "ux", "uy", "rho")
 PRECISIONS = {"fp64": LBM_FP64, "fp32": LBM_FP32, "fp16": LBM_FP16, "bf16": LBM_BF16,
@@ -199,7 +199,7 @@ def lbm_set_staging(h, bands: int = -1) -> None:
     _check(lib().lbm_set_staging(h, int(bands)), h)
 
 
-def lbm_set_streaming(h, mode: int = LBM_STREAM_ONE_BUFFER) -> None:
+def lbm_set_streaming(h, mode: int = LBM_STREAM_AUTO) -> None:
     _check(lib().lbm_set_streaming(h, int(mode)), h)
 
 
@@ -298,7 +298,7 @@ def lbm_batch_set_launch(b, rows: int = 0, prefetch: int = -1, interleave: int =
     _check(lib().lbm_batch_set_launch(b, int(rows), int(prefetch), int(interleave)))
 
 
-def lbm_batch_set_streaming(b, mode: int = LBM_STREAM_ONE_BUFFER) -> None:
+def lbm_batch_set_streaming(b, mode: int = LBM_STREAM_AUTO) -> None:
     _check(lib().lbm_batch_set_streaming(b, int(mode)))
 
 

@@ -5,7 +5,8 @@
 //     batch tile w h t  band threads rows | solo tile w h t  band threads rows
 //     | solo tiles, dynamic shared memory of one | default prefetch of the first lattice
 //     with 16-bit storage, and of the batch
-//     | rows per block of the batch's sweeps
+//     | rows per block of the batch's sweeps | whether the lattice, and the batch, take several steps
+//     per launch after lbm_(batch_)set_streaming to one buffer, and after -1
 #include "lbm_api.cu"
 
 #include <iostream>
@@ -38,12 +39,18 @@ int main() {
             batch_build<float>(&b);
             prefetch = reinterpret_cast<BatchEntry<float> *>(b.host_entries.data())->a[0].prefetch;
         }
-        const lbm_s &h = lats[0];
+        lbm_s &h = lats[0];
         TileArgs tl{};
         if (h.tile.t) tl = tile_args(&h, h.tile, h.tile.t, tile_cells(&h, h.tile.w, h.tile.h, h.tile.t, 1));
-        std::printf("%d %d %d %d %d %d %d %d %d %d %d %u %d %d %d\n", b.tile.w, b.tile.h, b.tile.t, b.band.threads, b.band.rows,
+        std::printf("%d %d %d %d %d %d %d %d %d %d %d %u %d %d %d", b.tile.w, b.tile.h, b.tile.t, b.band.threads, b.band.rows,
                     h.tile.w, h.tile.h, h.tile.t, h.band.threads, h.band.rows, tl.tiles_x * tl.tiles_y, tl.smem,
                     default_prefetch16(&h), prefetch, batch_shape(&b).rows);
+        for (int mode : {1, -1}) {
+            const int rc = lbm_set_streaming(&h, mode) | lbm_batch_set_streaming(&b, mode);
+            std::printf(" %d %d", rc == 0 && (use_tiles(&h) || use_bands(&h)),
+                        rc == 0 && !batch_sweeps_chosen(&b) && (b.tile.t > 0 || b.band.threads > 0));
+        }
+        std::printf("\n");
     }
     return 0;
 }

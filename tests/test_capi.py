@@ -84,3 +84,13 @@ def test_streaming_constants_match_header(built):
     text = open(os.path.join(ROOT, "include", "lbm.h")).read()
     m = re.search(r"enum \{ LBM_STREAM_TWO_BUFFERS = (\d+), LBM_STREAM_ONE_BUFFER = (\d+) \};", text)
     assert m and (int(m.group(1)), int(m.group(2))) == (built.LBM_STREAM_TWO_BUFFERS, built.LBM_STREAM_ONE_BUFFER)
+
+
+def test_streaming_auto_matches_header_and_is_the_default(built):
+    import inspect
+
+    text = open(os.path.join(ROOT, "include", "lbm.h")).read()
+    m = re.search(r"enum \{ LBM_STREAM_AUTO = (-?\d+) \};", text)
+    assert m and int(m.group(1)) == built.LBM_STREAM_AUTO
+    for f in (built.lbm_set_streaming, built.lbm_batch_set_streaming):
+        assert inspect.signature(f).parameters["mode"].default == built.LBM_STREAM_AUTO

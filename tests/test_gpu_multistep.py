@@ -214,3 +214,33 @@ def test_narrow_lattices_by_every_path(stream, prec, nx):
             lat.step(n)
         assert_same(lats[0], lats[2], (prec, nx, n))
         assert_same(lats[1], lats[2], (prec, nx, n))
+
+
+def test_modes_in_turn(stream):
+    """lbm_set_streaming between calls, LBM_STREAM_AUTO among the modes: a lattice and a
+    batch go on from the same state whatever moved it there."""
+    p = workloads.params(Ra=1e6, strip_center=0.4)
+    for prec in ("fp32", "fp16sr", "fp64"):
+        lat, ref = (start(130, 70, p, prec, stream) for _ in range(2))
+        members = [start(64, 32, p, prec, stream, seed=k) for k in range(2)]
+        refs = [start(64, 32, p, prec, stream, seed=k) for k in range(2)]
+        lbm.lbm_set_streaming(ref.h, lbm.LBM_STREAM_TWO_BUFFERS)
+        batch, batch_ref = lbm.Batch(2, stream), lbm.Batch(2, stream)
+        for b, ms in ((batch, members), (batch_ref, refs)):
+            for m in ms:
+                b.add(m)
+        lbm.lbm_batch_set_streaming(batch_ref.b, lbm.LBM_STREAM_TWO_BUFFERS)
+        for mode in (lbm.LBM_STREAM_ONE_BUFFER, lbm.LBM_STREAM_AUTO, lbm.LBM_STREAM_TWO_BUFFERS, lbm.LBM_STREAM_AUTO):
+            lbm.lbm_set_streaming(lat.h, mode)
+            lbm.lbm_batch_set_streaming(batch.b, mode)
+            for n in (7, 20, 20):
+                for x in (lat, ref, batch, batch_ref):
+                    x.step(n)
+        assert_same(lat, ref, prec)
+        for x, y in zip(members, refs):
+            assert_same(x, y, prec)
+        batch.close()
+        batch_ref.close()
+    for bad in (-2, 2):
+        with pytest.raises(lbm.LbmError):
+            lbm.lbm_set_streaming(lat.h, bad)

@@ -23,7 +23,8 @@ def plans(tmp_path_factory):
         out = subprocess.run([exe], input=" ".join(map(str, line)), capture_output=True, text=True, check=True).stdout
         keys = ("w", "h", "t", "threads", "rows")
         v = [int(x) for x in out.split()]
-        return dict(zip(keys, v[:5])), dict(zip(keys + ("tiles", "smem", "prefetch16", "batch_prefetch", "batch_rows"), v[5:]))
+        more = ("tiles", "smem", "prefetch16", "batch_prefetch", "batch_rows", "one", "batch_one", "auto", "batch_auto")
+        return dict(zip(keys, v[:5])), dict(zip(keys + more, v[5:]))
 
     return ask
 
@@ -115,3 +116,10 @@ def test_batch_shapes(plans, prec, problem, flow, rows, prefetch):
     """Members stepped one cell per thread keep their own shape."""
     solo = plans(prec, problem, flow, [(256, 128)] * 32)[1]
     assert (solo["batch_rows"], solo["batch_prefetch"]) == (rows, prefetch)
+
+
+@pytest.mark.parametrize("prec,size,n", [("fp32", (64, 32), 2), ("fp32", (2048, 1024), 2), ("bf16sr", (256, 128), 1)])
+def test_the_choice_can_be_given_back(plans, prec, size, n):
+    solo = plans(prec, workloads.CAVITY, 1, [size] * n)[1]
+    assert (solo["one"], solo["batch_one"]) == (0, 0)
+    assert (solo["auto"], solo["batch_auto"]) == (1, 1)
