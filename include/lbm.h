@@ -254,10 +254,12 @@ int lbm_get_launch_stats(lbm_handle h, lbm_launch_stats *out);
  * steps each (best of two, after a warm-up) on a scratch lattice with the
  * handle's size, precision and parameters -- the handle's own state is not
  * touched, but the scratch lattice is allocated and freed -- and applies the
- * fastest with lbm_set_launch (graph_chunk unchanged).  The choice is cached
- * per (nx, ny, precision, problem, flow_on) for the life of the process, so
- * later handles of the same kind are tuned without timing.  Outputs (may be
- * NULL): the chosen rows and prefetch, and its time per step in microseconds
+ * fastest with lbm_set_launch (graph_chunk unchanged).  A lattice that takes several
+ * steps per launch (lbm_set_streaming) is swept at its diagnostic steps only: it
+ * keeps its shape, which is returned with the time of the kernels it runs.  The choice
+ * is cached per (nx, ny, precision, problem, flow_on, streaming) for the life of the
+ * process, so later handles of the same kind are tuned without timing.  Outputs (may be
+ * NULL): the shape's rows and prefetch, and the time per step in microseconds
  * (0 when it came from the cache).  Synchronises.  Errors: LBM_ERR_ARG,
  * LBM_ERR_STATE, LBM_ERR_OOM, LBM_ERR_CUDA. */
 int lbm_autotune(lbm_handle h, int steps_per_trial, int *rows, int *prefetch, float *us_per_step);
@@ -377,10 +379,11 @@ int lbm_batch_set_streaming(lbm_batch b, int mode);
  * member, interleaved) for steps_per_trial steps each (best of three, after a
  * warm-up) on scratch lattices of the batch's composition -- the same sizes,
  * precision and parameters, allocated and freed here; the members' states are
- * not touched -- and applies the fastest with lbm_batch_set_launch.  The
- * choice is cached per composition (precision, problem, flow and the members'
+ * not touched -- and applies the fastest with lbm_batch_set_launch.  A batch that
+ * takes several steps per launch keeps its shape, as in lbm_autotune.  The
+ * choice is cached per composition (precision, problem, flow, streaming and the members'
  * sizes in order) for the life of the process.  Outputs (may be NULL): the
- * chosen shape and its time per step in microseconds (0 when it came from the
+ * shape and the time per step in microseconds (0 when it came from the
  * cache).  Synchronises.  Errors: LBM_ERR_ARG, LBM_ERR_STATE (empty batch),
  * LBM_ERR_OOM, LBM_ERR_CUDA. */
 int lbm_batch_autotune(lbm_batch b, int steps_per_trial, int *rows, int *prefetch, int *interleave,

@@ -1229,18 +1229,20 @@ const char *lbm_version(void) { return "btrirt 0.1 sm_103a"; }
 
 
 // ---------------------------------------------------------------------------
-// Autotuner: picks the launch shape (rows per block, L2 prefetch distance) for
-// a lattice size by timing candidates on a scratch lattice of the same size,
-// precision and parameters, so the caller's state is untouched.  Results are
-// cached per (nx, ny, precision, problem, flow_on, streaming) for the process.
+// Autotuner: picks the launch shape (rows per block, L2 prefetch distance) of the
+// sweeps for a lattice size by timing candidates on a scratch lattice of the same size,
+// precision and parameters, so the caller's state is untouched.  A lattice that takes
+// several steps per launch is swept at its diagnostic steps only: its shape stays, and
+// the time is that of the kernels it runs.  Results are cached per (nx, ny, precision,
+// problem, flow_on, streaming, several steps per launch) for the process.
 // ---------------------------------------------------------------------------
 namespace {
 
 struct TuneKey {
-    int nx, ny, precision, problem, flow, streaming;
+    int nx, ny, precision, problem, flow, streaming, multi;
     bool operator==(const TuneKey &o) const {
         return nx == o.nx && ny == o.ny && precision == o.precision && problem == o.problem && flow == o.flow &&
-               streaming == o.streaming;
+               streaming == o.streaming && multi == o.multi;
     }
 };
 struct TuneEntry {
@@ -1251,13 +1253,30 @@ struct TuneEntry {
 std::mutex g_tune_mutex;
 std::vector<TuneEntry> g_tune_cache;
 
+// The best of reps calls of `steps` steps on the stream, in us per step.
+template <typename Step>
+int time_steps(cudaEvent_t e0, cudaEvent_t e1, cudaStream_t s, int reps, int steps, Step &&step, float *us) {
+    float best_ms = 1e30f;
+    for (int rep = 0; rep < reps; ++rep) {
+        if (cudaEventRecord(e0, s) != cudaSuccess) return LBM_ERR_CUDA;
+        const int rc = step(steps);
+        if (rc != LBM_OK) return rc;
+        if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) return LBM_ERR_CUDA;
+        float ms = 0.0f;
+        if (cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best_ms) best_ms = ms;
+    }
+    *us = best_ms * 1000.0f / (float)steps;
+    return LBM_OK;
+}
+
 }  // namespace
 
 extern "C" int lbm_autotune(lbm_handle h, int steps_per_trial, int *rows_out, int *prefetch_out,
                             float *us_per_step_out) {
     if (!h || steps_per_trial < 1) return set_err(h, LBM_ERR_ARG, "lbm_autotune: bad argument");
     if (!h->params_set) return set_err(h, LBM_ERR_STATE, "lbm_autotune: parameters not set");
-    const TuneKey key{h->nx, h->ny, h->precision, h->p.problem, h->p.flow_on != 0, h->streaming};
+    const bool multi = use_tiles(h) || use_bands(h);
+    const TuneKey key{h->nx, h->ny, h->precision, h->p.problem, h->p.flow_on != 0, h->streaming, multi};
     TuneEntry best{key, h->rows, h->prefetch, 0.0f};
     bool cached = false;
     {
@@ -1274,32 +1293,28 @@ extern "C" int lbm_autotune(lbm_handle h, int steps_per_trial, int *rows_out, in
         int rc = lbm_create(h->nx, h->ny, h->precision, h->stream, &t);
         if (rc != LBM_OK) return set_err(h, rc, "lbm_autotune: scratch lattice: %s", lbm_last_error(nullptr));
         rc = lbm_set_params(t, &h->p);
-        if (rc == LBM_OK) rc = lbm_set_streaming(t, h->streaming);
+        if (rc == LBM_OK) rc = lbm_set_streaming(t, multi ? LBM_STREAM_AUTO : h->streaming);
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (rc == LBM_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
             rc = set_err(h, LBM_ERR_CUDA, "lbm_autotune: cudaEventCreate failed");
-        best.us_per_step = 1e30f;
+        auto step = [&](long long n) { return lbm_step(t, n); };
         const int rows_c[] = {1, 2, 3, 4};
         const int pf_c[] = {0, 2, 4, 8, 16, 24, 32, 48};
+        best.us_per_step = 1e30f;
+        if (multi && rc == LBM_OK) {
+            rc = lbm_set_launch(t, h->rows, h->prefetch, h->graph_chunk);
+            if (rc == LBM_OK) rc = lbm_step(t, 4);  // warm-up
+            if (rc == LBM_OK) rc = time_steps(e0, e1, t->stream, 3, steps_per_trial, step, &best.us_per_step);
+        }
         for (int rows : rows_c) {
-            if (rc != LBM_OK || rows > h->ny) break;
+            if (multi || rc != LBM_OK || rows > h->ny) break;
             for (int pf : pf_c) {
                 if (rc != LBM_OK) break;
                 if (pf >= h->ny) continue;
                 rc = lbm_set_launch(t, rows, pf, h->graph_chunk);
                 if (rc == LBM_OK) rc = lbm_step(t, 4);  // warm-up (and graph capture)
-                float best_ms = 1e30f;
-                for (int rep = 0; rep < 2 && rc == LBM_OK; ++rep) {
-                    if (cudaEventRecord(e0, t->stream) != cudaSuccess) rc = LBM_ERR_CUDA;
-                    if (rc == LBM_OK) rc = lbm_step(t, steps_per_trial);
-                    if (rc == LBM_OK && (cudaEventRecord(e1, t->stream) != cudaSuccess ||
-                                         cudaEventSynchronize(e1) != cudaSuccess))
-                        rc = LBM_ERR_CUDA;
-                    float ms = 0.0f;
-                    if (rc == LBM_OK && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best_ms)
-                        best_ms = ms;
-                }
-                const float us = best_ms * 1000.0f / (float)steps_per_trial;
+                float us = 1e30f;
+                if (rc == LBM_OK) rc = time_steps(e0, e1, t->stream, 2, steps_per_trial, step, &us);
                 if (rc == LBM_OK && us < best.us_per_step) {
                     best.rows = rows;
                     best.prefetch = pf;
@@ -1314,10 +1329,12 @@ extern "C" int lbm_autotune(lbm_handle h, int steps_per_trial, int *rows_out, in
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         g_tune_cache.push_back(best);
     }
-    const int rc = lbm_set_launch(h, best.rows, best.prefetch, h->graph_chunk);
-    if (rc != LBM_OK) return rc;
-    if (rows_out) *rows_out = best.rows;
-    if (prefetch_out) *prefetch_out = best.prefetch;
+    if (!multi) {
+        const int rc = lbm_set_launch(h, best.rows, best.prefetch, h->graph_chunk);
+        if (rc != LBM_OK) return rc;
+    }
+    if (rows_out) *rows_out = h->rows;
+    if (prefetch_out) *prefetch_out = h->prefetch;
     if (us_per_step_out) *us_per_step_out = cached ? 0.0f : best.us_per_step;
     return LBM_OK;
 }
@@ -1394,6 +1411,8 @@ template <typename real>
 size_t entry_bytes() { return sizeof(BatchEntry<real>); }
 
 bool batch_sweeps_chosen(const lbm_batch_s *b) { return b->streaming != LBM_STREAM_AUTO; }
+// several steps per launch (the table is built)
+bool batch_several(const lbm_batch_s *b) { return !batch_sweeps_chosen(b) && (b->tile.t > 0 || b->band.threads > 0); }
 
 // Default launch shape of a batch, whatever the members' own lbm_set_launch
 // settings; blocks of a one-size batch are interleaved over the members.  The fastest
@@ -1542,7 +1561,7 @@ int batch_steps(lbm_batch_s *b, long long n) {
     // call, an even number, alternate push (even j) and local (odd j) sweeps
     // in each member's buffer parity[r]; the last one or two run over the two
     // buffers, so that between calls every member's state is the two-buffer one.
-    const bool multi = !batch_sweeps_chosen(b) && (b->tile.t > 0 || b->band.threads > 0);
+    const bool multi = batch_several(b);
     const int streaming = batch_sweeps_chosen(b) ? b->streaming : default_streaming(b->precision);
     const bool one = !multi && streaming == LBM_STREAM_ONE_BUFFER;
     int launches = 0;  // of several-step pieces: the buffers they have changed
@@ -1798,10 +1817,10 @@ int lbm_batch_destroy(lbm_batch b) {
 }  // extern "C"
 
 // ---------------------------------------------------------------------------
-// Batch autotuner: times launch shapes of a batch (rows per block, L2
+// Batch autotuner: times launch shapes of a batch's sweeps (rows per block, L2
 // prefetch distance, interleaved block order) on scratch lattices of the same
-// composition and applies the fastest; cached per composition for the
-// process.
+// composition and applies the fastest; a batch that takes several steps per launch
+// keeps its shape, as in lbm_autotune.  Cached per composition for the process.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -1809,6 +1828,7 @@ struct BatchTune {
     std::string key;
     int rows, prefetch, interleave;
     float us_per_step;
+    bool multi, uniform;
 };
 std::mutex g_btune_mutex;
 std::vector<BatchTune> g_btune_cache;
@@ -1829,7 +1849,7 @@ extern "C" int lbm_batch_autotune(lbm_batch b, int steps_per_trial, int *rows_ou
     if (!b || steps_per_trial < 1) return batch_err(LBM_ERR_ARG, "lbm_batch_autotune: bad argument");
     if (b->members.empty()) return batch_err(LBM_ERR_STATE, "lbm_batch_autotune: the batch is empty");
     const std::string key = batch_key(b);
-    BatchTune best{key, b->rows, b->prefetch, b->interleave, 0.0f};
+    BatchTune best{key, b->rows, b->prefetch, b->interleave, 0.0f, false, false};
     bool cached = false;
     {
         std::lock_guard<std::mutex> lock(g_btune_mutex);
@@ -1846,11 +1866,7 @@ extern "C" int lbm_batch_autotune(lbm_batch b, int steps_per_trial, int *rows_ou
         std::vector<lbm_handle> scratch;
         lbm_batch t = nullptr;
         int rc = lbm_batch_create((int)b->members.size(), b->stream, &t);
-        // shapes of the sweeps are timed, whether or not they take the plain steps
-        if (rc == LBM_OK)
-            t->streaming = b->streaming >= 0            ? b->streaming
-                           : b->precision == LBM_FP64 ? LBM_STREAM_TWO_BUFFERS
-                                                      : LBM_STREAM_ONE_BUFFER;
+        if (rc == LBM_OK) t->streaming = b->streaming;
         for (size_t r = 0; r < b->members.size() && rc == LBM_OK; ++r) {
             const lbm_s *h = b->members[r];
             lbm_handle s = nullptr;
@@ -1864,28 +1880,28 @@ extern "C" int lbm_batch_autotune(lbm_batch b, int steps_per_trial, int *rows_ou
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (rc == LBM_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
             rc = LBM_ERR_CUDA;
+        auto step = [&](long long n) { return lbm_batch_step(t, n); };
         const int rows_c[] = {1, 2, 3, 4};
         const int pf_c[] = {0, 4, 8, 16};
         const int ninter = b->members.size() > 1 ? 2 : 1;  // interleaving needs several members
         best.us_per_step = 1e30f;
+        if (rc == LBM_OK) rc = lbm_batch_set_launch(t, b->rows, b->prefetch, b->interleave);
+        if (rc == LBM_OK) rc = lbm_batch_step(t, 4);  // warm-up, table upload
+        if (rc == LBM_OK) {
+            best.multi = batch_several(t);
+            best.uniform = t->uniform > 0;
+            if (best.multi) rc = time_steps(e0, e1, t->stream, 3, steps_per_trial, step, &best.us_per_step);
+        }
         for (int rows : rows_c) {
+            if (best.multi) break;
             for (int k = 0; k < 4 && rc == LBM_OK; ++k) {
                 for (int il = 0; il < ninter && rc == LBM_OK; ++il) {
                     rc = lbm_batch_set_launch(t, rows, pf_c[k], il);
                     if (rc == LBM_OK) rc = lbm_batch_step(t, 4);  // warm-up, table upload
                     if (rc == LBM_OK && il == 1 && t->uniform == 0) break;  // not a one-size batch
-                    float best_ms = 1e30f;
-                    for (int rep = 0; rep < 3 && rc == LBM_OK; ++rep) {  // the second replays a graph
-                        if (cudaEventRecord(e0, t->stream) != cudaSuccess) rc = LBM_ERR_CUDA;
-                        if (rc == LBM_OK) rc = lbm_batch_step(t, steps_per_trial);
-                        if (rc == LBM_OK && (cudaEventRecord(e1, t->stream) != cudaSuccess ||
-                                             cudaEventSynchronize(e1) != cudaSuccess))
-                            rc = LBM_ERR_CUDA;
-                        float ms = 0.0f;
-                        if (rc == LBM_OK && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms < best_ms)
-                            best_ms = ms;
-                    }
-                    const float us = best_ms * 1000.0f / (float)steps_per_trial;
+                    float us = 1e30f;
+                    if (rc == LBM_OK)  // the second replays a graph
+                        rc = time_steps(e0, e1, t->stream, 3, steps_per_trial, step, &us);
                     if (rc == LBM_OK && us < best.us_per_step) {
                         best.rows = rows;
                         best.prefetch = pf_c[k];
@@ -1903,8 +1919,15 @@ extern "C" int lbm_batch_autotune(lbm_batch b, int steps_per_trial, int *rows_ou
         std::lock_guard<std::mutex> lock(g_btune_mutex);
         g_btune_cache.push_back(best);
     }
-    const int rc = lbm_batch_set_launch(b, best.rows, best.prefetch, best.interleave);
-    if (rc != LBM_OK) return rc;
+    if (best.multi) {  // the shape of its sweeps as it is
+        const BatchShape shape = batch_shape(b);
+        best.rows = b->rows > 0 ? b->rows : shape.rows;
+        best.prefetch = b->prefetch >= 0 ? b->prefetch : shape.prefetch;
+        best.interleave = best.uniform ? b->interleave : 0;
+    } else {
+        const int rc = lbm_batch_set_launch(b, best.rows, best.prefetch, best.interleave);
+        if (rc != LBM_OK) return rc;
+    }
     if (rows_out) *rows_out = best.rows;
     if (prefetch_out) *prefetch_out = best.prefetch;
     if (interleave_out) *interleave_out = best.interleave;

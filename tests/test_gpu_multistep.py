@@ -244,3 +244,32 @@ def test_modes_in_turn(stream):
     for bad in (-2, 2):
         with pytest.raises(lbm.LbmError):
             lbm.lbm_set_streaming(lat.h, bad)
+
+
+def test_autotuners_time_what_runs(stream):
+    """Where several steps share a launch the tuners leave the sweeps' shape alone and
+    return the time of the kernels that run: far less than a sweep per step takes here."""
+    p = workloads.params(Ra=1e6, strip_center=0.35)
+    lat, swept = (lbm.Lattice(260, 126, p, precision="fp32", stream=stream) for _ in range(2))
+    lbm.lbm_set_launch(lat.h, 7, 5, 64)
+    lbm.lbm_set_streaming(swept.h, lbm.LBM_STREAM_ONE_BUFFER)
+    t, ts = lbm.lbm_autotune(lat.h, 100), lbm.lbm_autotune(swept.h, 100)
+    assert (t["rows"], t["prefetch"]) == (7, 5) and ts["rows"] in (1, 2, 3, 4)
+    assert 0 < 1.5 * t["us_per_step"] < ts["us_per_step"]
+    lbm.lbm_set_streaming(swept.h, lbm.LBM_STREAM_AUTO)
+    assert lbm.lbm_autotune(swept.h, 100)["us_per_step"] == 0.0  # the same kind as the first now
+    us = []
+    for mode in (lbm.LBM_STREAM_AUTO, lbm.LBM_STREAM_TWO_BUFFERS):
+        b = lbm.Batch(2, stream)
+        members = [lbm.Lattice(260, 126, p, precision="fp32", stream=stream) for _ in range(2)]
+        for m in members:
+            b.add(m)
+        lbm.lbm_batch_set_streaming(b.b, mode)
+        if mode == lbm.LBM_STREAM_AUTO:
+            lbm.lbm_batch_set_launch(b.b, 3, 2, 1)
+        t = lbm.lbm_batch_autotune(b.b, 100)
+        if mode == lbm.LBM_STREAM_AUTO:
+            assert (t["rows"], t["prefetch"], t["interleave"]) == (3, 2, 1)
+        us.append(t["us_per_step"])
+        b.close()
+    assert 0 < 1.5 * us[0] < us[1]
