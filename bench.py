@@ -29,7 +29,7 @@ the aggregate MLUPS and the 16-bit results' largest melt-fraction and Nusselt
 differences from an FP64 run of the same requests.
 
 --batch N times the batched path instead: N cavities of 256 x 128 (the
-serving size; Ra and strip centre varied, seeded) advanced together, two steps
+serving size; Ra and strip centre varied, seeded) advanced together, several steps
 per launch over all of them (one in FP64; graph-replayed); the last step carries
 the diagnostics.  Same JSON line, device-resident timing only.
 """
@@ -71,24 +71,6 @@ def sweep_launches(warmup: int, steps: int) -> int:
     diag = {n for n in range(warmup + 1, warmup + steps + 1) if n % DIAG_EVERY == 0}
     diag.add(warmup + steps)
     return steps + len(diag)
-
-
-def kernel_launches(precision: str, warmup: int, steps: int) -> int:
-    """Kernels launched by lbm_step(steps) after `warmup` steps.  FP32 takes two
-    steps per launch: the library cuts the call into pieces that end at the
-    diagnostic steps and are at most 128 long; a piece's last step, if diagnostic,
-    is a sweep and a fold, an odd step before it a sweep."""
-    if precision != "fp32":
-        return sweep_launches(warmup, steps)
-    total, at, end = 0, warmup, warmup + steps
-    while at < end:
-        stop = min(end, (at // DIAG_EVERY + 1) * DIAG_EVERY)
-        diag = stop - at <= 128
-        n = min(stop - at, 128)
-        plain = n - 1 if diag else n
-        total += plain // 2 + plain % 2 + (2 if diag else 0)
-        at += n
-    return total
 
 
 def workload_config(precision: str) -> dict:
@@ -407,10 +389,12 @@ def run_ours(args) -> None:
         if dist:
             dist.barrier()
         torch.cuda.synchronize()
+        launched = lbm.lbm_get_kernel_launches(lat.h)
         start.record(stream)
         lat.step(args.steps)
         stop.record(stream)
         torch.cuda.synchronize()
+        launched = lbm.lbm_get_kernel_launches(lat.h) - launched
     if dist:
         dist.barrier()
     elapsed = start.elapsed_time(stop) / 1e3
@@ -424,11 +408,13 @@ def run_ours(args) -> None:
     if not args.no_e2e:
         e2e = measure_e2e(args, lat, p, prec, stream, dist, local)
 
-    # ---- roofline of the sweep (the only kernel in the timed region)
+    # ---- roofline of a step
     peak, peak_kind = measured_peak_gbs()
     kernel_s = elapsed / args.steps
     alg_bytes = BYTES_PER_LUP[prec] * cells
-    achieved = alg_bytes / kernel_s / 1e9
+    # a launch reads and writes every population once, whether it takes one step or two
+    folds = sweep_launches(args.warmup, args.steps) - args.steps
+    achieved = alg_bytes * (launched - folds) / elapsed / 1e9
     traffic = profiled_traffic(prec)
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic,
@@ -436,8 +422,7 @@ def run_ours(args) -> None:
                 "algorithmic_bytes_per_launch": alg_bytes}
     if traffic:
         # The DRAM side: the profiled bytes per step (warm L2, as in this
-        # loop) over the measured time.  FP32 moves populations once per two
-        # steps.  A step that starts on rows the
+        # loop) over the measured time.  A launch that starts on rows the
         # previous one left in L2 moves fewer bytes than it reads and writes,
         # so `frac` (algorithmic bytes) can exceed 1 while this stays below.
         roofline["dram_achieved"] = round(traffic / kernel_s / 1e9, 1)
@@ -462,7 +447,7 @@ def run_ours(args) -> None:
         "config": workload_config(prec),
         "roofline": roofline,
         "e2e": e2e,
-        "gpu_launches": kernel_launches(prec, args.warmup, args.steps),
+        "gpu_launches": launched,
         "clocks": clocks.summary(),
         "melt_fraction": d["melt_fraction"],
     }
@@ -538,6 +523,15 @@ def serving_leg() -> dict:
 BATCH_NX, BATCH_NY = 256, 128
 
 
+def batch_launches(steps: int, launched: int) -> tuple[str, str]:
+    """How a batch's call of `steps` steps ran, from the kernels it launched: the last
+    step is a sweep and a fold, the others are sweeps or share launches."""
+    if launched > steps:
+        return "one fused launch per step", "the library's default for the storage type (lbm_batch_set_streaming)"
+    return (f"{steps - 1} steps in {launched - 2} launches and a diagnostic one",
+            "one buffer read and the other written per launch, the last step a sweep")
+
+
 def run_batch(args) -> None:
     import numpy as np
     import torch
@@ -563,16 +557,18 @@ def run_batch(args) -> None:
     with ClockSampler(0) as clocks:
         b.step(args.warmup)
         torch.cuda.synchronize()
+        launched = lbm.lbm_batch_get_kernel_launches(b.b)
         start.record(stream)
         b.step(args.steps)
         stop.record(stream)
         torch.cuda.synchronize()
+        launched = lbm.lbm_batch_get_kernel_launches(b.b) - launched
     elapsed = start.elapsed_time(stop) / 1e3
     cells = n * BATCH_NX * BATCH_NY
     kernel_s = elapsed / args.steps
     alg_bytes = BYTES_PER_LUP[prec] * cells
     peak, peak_kind = measured_peak_gbs()
-    achieved = alg_bytes / kernel_s / 1e9
+    achieved = alg_bytes * (launched - 1) / elapsed / 1e9  # a launch moves every population once; one fold
     nan = sum(lat.diagnostics(raise_on_diverged=False)["nan_flag"] for lat in lats)
     assert nan == 0
     line = {
@@ -582,29 +578,24 @@ def run_batch(args) -> None:
         "vs_baseline": None, "dtype": prec, "data": "synthetic",
         "config": {"workload": f"batch of {n} cavities {BATCH_NX}x{BATCH_NY} (Ra 1e6-1e8, strip "
                                f"W/4 at 0.2-0.8 W, seeded), {prec.upper()} populations, "
-                               + ("one fused launch per step" if prec == "fp64" else "several steps per launch"
-                                  if cells <= 1 << 19 else "two steps per launch"),
+                               + batch_launches(args.steps, launched)[0],
                    "lattices": n, "precision": prec,
-                   "streaming": ("two buffers" if prec == "fp64" else
-                                 "one buffer read and the other written per launch, the last step a sweep"),
+                   "streaming": batch_launches(args.steps, launched)[1],
                    # the populations in both buffers
                    "l2": (f"inputs larger than L2 ({alg_bytes / 1e6:.0f} MB of populations in the two "
                           "buffers), no flush" if alg_bytes > L2_MB * 1e6 else
                           f"the populations ({alg_bytes / 1e6:.0f} MB in the two buffers) fit in the "
                           f"{L2_MB:.0f} MB L2: a step reads what the previous one wrote, no flush"),
+                   # the shape of the sweeps, where they take the steps
                    "launch": ({"rows": tuned["rows"], "prefetch": tuned["prefetch"],
                                "interleave": tuned["interleave"], "by": "lbm_batch_autotune"}
-                              if tuned else "default")},
+                              if tuned and launched > args.steps else "default")},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": profiled_traffic(prec, n),
                      "peak_source": f"{peak_kind} HBM copy bandwidth",
                      "algorithmic_bytes_per_launch": alg_bytes},
         "e2e": None,
-        # two steps per launch and an odd one alone (up to 2^19 cells at most 16 per
-        # launch), the diagnostic step and its fold
-        "gpu_launches": (args.steps + 1 if prec == "fp64" else
-                         -(-(args.steps - 1) // 16) + 2 if cells <= 1 << 19 else
-                         (args.steps - 1) // 2 + (args.steps - 1) % 2 + 2),
+        "gpu_launches": launched,
         "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)

@@ -249,6 +249,11 @@ typedef struct {
 } lbm_launch_stats;
 int lbm_get_launch_stats(lbm_handle h, lbm_launch_stats *out);
 
+/* Kernels that lbm_step has launched on the handle since lbm_create, replayed graphs
+ * included: one per sweep or per several steps (lbm_set_streaming), and the fold after a
+ * diagnostic sweep.  Errors: LBM_ERR_ARG. */
+int lbm_get_kernel_launches(lbm_handle h, long long *kernels);
+
 /* Autotuner: times every launch shape of a small candidate set (rows per block
  * 1, 2, 3, 4; prefetch distance 0, 2, 4, 8, 16, 24, 32, 48 rows) for steps_per_trial
  * steps each (best of two, after a warm-up) on a scratch lattice with the
@@ -349,6 +354,10 @@ int lbm_batch_count(lbm_batch b, int *count);
 
 /* Advance every member n >= 0 steps, asynchronously on the batch's stream. */
 int lbm_batch_step(lbm_batch b, long long n);
+
+/* Kernels that lbm_batch_step has launched since lbm_batch_create, counted as by
+ * lbm_get_kernel_launches.  Errors: LBM_ERR_ARG. */
+int lbm_batch_get_kernel_launches(lbm_batch b, long long *kernels);
 
 /* Launch shape of the batch's step kernel: rows of a member walked by each
  * block (0 = the default: 2; with 16-bit storage 3 for cavities with flow, else 4;

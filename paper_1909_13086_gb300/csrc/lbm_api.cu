@@ -64,6 +64,7 @@ struct ChunkGraph {
     int phase = 0;
     int flip = 0, end_phase = 0;  // the handle's state after the piece: cur ^ flip, phase,
     bool end_prev = false;        // has_prev (single lattices)
+    long long kernels = 0;        // in the piece
     cudaGraphExec_t exec = nullptr;
     unsigned long long stamp = 0;
 };
@@ -88,6 +89,7 @@ struct lbm_s {
     ChunkGraph graphs[kGraphCache];
     unsigned long long graph_clock = 0;
     lbm_launch_stats stats{};   // sweeps launched directly / replayed, graphs captured
+    long long kernels = 0;  // launched by lbm_step (lbm_get_kernel_launches)
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     void *buf[2] = {nullptr, nullptr};  // 18 planes each
@@ -557,6 +559,7 @@ int launch_one(lbm_s *h, bool diag) {
     h->cur ^= 1;
     h->has_prev = true;
     h->step = next;
+    h->kernels += diag ? 2 : 1;  // and the fold
     return LBM_OK;
 }
 
@@ -576,6 +579,7 @@ int launch_one_aa(lbm_s *h, bool diag) {
     h->phase ^= 1;
     h->has_prev = false;  // buf[cur ^ 1] is stale until the call's closing two-buffer sweeps
     h->step = next;
+    h->kernels += diag ? 2 : 1;
     return LBM_OK;
 }
 
@@ -591,6 +595,7 @@ int launch_tiles(lbm_s *h, int T) {
     h->cur ^= 1;
     h->has_prev = false;  // buf[cur ^ 1] is T steps old until the call's closing sweep
     h->step += T;
+    h->kernels += 1;
     return LBM_OK;
 }
 
@@ -607,6 +612,7 @@ int launch_bands(lbm_s *h) {
         h->cur ^= 1;
         h->has_prev = false;
         h->step += 2;
+        h->kernels += 1;
         return LBM_OK;
     }
 }
@@ -692,6 +698,7 @@ int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
             const int cur0 = h->cur, phase0 = h->phase;
             const long long step0 = h->step;
             const bool prev0 = h->has_prev;
+            const long long kernels0 = h->kernels;
             CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
             const int rc = launch_sweeps<real, S>(h, len, diag, one_buffer);
             cudaGraph_t graph = nullptr;
@@ -699,10 +706,12 @@ int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
             slot->flip = h->cur ^ cur0;
             slot->end_phase = h->phase;
             slot->end_prev = h->has_prev;
+            slot->kernels = h->kernels - kernels0;
             h->cur = cur0;
             h->phase = phase0;
             h->step = step0;
             h->has_prev = prev0;
+            h->kernels = kernels0;
             if (rc != LBM_OK) {
                 if (graph) cudaGraphDestroy(graph);
                 return rc;
@@ -726,6 +735,7 @@ int run_piece(lbm_s *h, long long len, bool diag, bool one_buffer = false) {
         h->has_prev = slot->end_prev;
         h->step += len;
         h->stats.sweeps_replayed += len;
+        h->kernels += slot->kernels;
         return LBM_OK;
     }
     const int rc = launch_sweeps<real, S>(h, len, diag, one_buffer);
@@ -991,6 +1001,12 @@ int lbm_step(lbm_handle h, long long n) {
 int lbm_get_launch_stats(lbm_handle h, lbm_launch_stats *out) {
     if (!h || !out) return set_err(h, LBM_ERR_ARG, "NULL argument");
     *out = h->stats;
+    return LBM_OK;
+}
+
+int lbm_get_kernel_launches(lbm_handle h, long long *kernels) {
+    if (!h || !kernels) return set_err(h, LBM_ERR_ARG, "NULL argument");
+    *kernels = h->kernels;
     return LBM_OK;
 }
 
@@ -1373,6 +1389,7 @@ struct lbm_batch_s {
                                      // piece's first launch within its call; the
                                      // members' own parities are a device table)
     unsigned long long graph_clock = 0;
+    long long kernels = 0;  // launched by lbm_batch_step (lbm_batch_get_kernel_launches)
     cudaEvent_t ev = nullptr;
     lbm_alloc_fn alloc = nullptr;
     lbm_free_fn release = nullptr;
@@ -1504,6 +1521,7 @@ int batch_multi(lbm_batch_s *b, long long len, bool diag, int j) {
     auto sweep = [&](bool d) {
         e = launch_batch<float, S>(b->entries, b->starts, b->parity, nm, b->uniform, b->uniform > 0 ? b->interleave : 0,
                                    b->nblocks, b->problem, b->flow != 0, d, j & 1, b->stream, true, kPull);
+        b->kernels += d ? 2 : 1;  // and the fold
         ++j;
     };
     const long long plain = diag ? len - 1 : len;
@@ -1518,10 +1536,12 @@ int batch_multi(lbm_batch_s *b, long long len, bool diag, int j) {
             for (const lbm_s *h : b->members) cells = std::max(cells, tile_cells(h, b->tile.w, b->tile.h, T, 1));
             e = launch_batch_tile<S>(b->entries, b->mstarts, b->parity, nm, b->mblocks, j & 1,
                                      tile_args(b->members[0], b->tile, T, cells), b->stream);
+            b->kernels += 1;
             ++j;
         } else {
             e = launch_batch_band<S>(b->entries, b->mstarts, b->parity, nm, b->mblocks, j & 1,
                                      band_args(b->members[0], b->band), b->stream);
+            b->kernels += 1;
             ++j;
         }
     }
@@ -1584,6 +1604,7 @@ int batch_steps(lbm_batch_s *b, long long n) {
                                                         diag && j == len - 1, (int)(jj & 1),
                                                         b->stream, true, sm);
             if (e != cudaSuccess) return batch_err(LBM_ERR_CUDA, "batch launch failed: %s", cudaGetErrorString(e));
+            b->kernels += diag && j == len - 1 ? 2 : 1;
         }
         return LBM_OK;
     };
@@ -1614,9 +1635,12 @@ int batch_steps(lbm_batch_s *b, long long n) {
             } else if (!slot->exec) {
                 BATCH_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
                 const int before = launches;
+                const long long kernels0 = b->kernels;
                 const int rc = direct(0, len, diag, ob);
                 slot->flip = (launches ^ before) & 1;
                 launches = before;
+                slot->kernels = b->kernels - kernels0;
+                b->kernels = kernels0;
                 cudaGraph_t g = nullptr;
                 const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
                 if (rc != LBM_OK || e2 != cudaSuccess) {
@@ -1637,6 +1661,7 @@ int batch_steps(lbm_batch_s *b, long long n) {
             slot->stamp = ++b->graph_clock;
             BATCH_TRY(cudaGraphLaunch(slot->exec, b->stream));
             launches += slot->flip;
+            b->kernels += slot->kernels;
             return LBM_OK;
         }
         return direct(from, len, diag, ob);
@@ -1778,6 +1803,12 @@ int lbm_batch_step(lbm_batch b, long long n) {
         BATCH_TRY(cudaStreamWaitEvent(h->stream, b->ev, 0));
         last = h->stream;
     }
+    return LBM_OK;
+}
+
+int lbm_batch_get_kernel_launches(lbm_batch b, long long *kernels) {
+    if (!b || !kernels) return batch_err(LBM_ERR_ARG, "lbm_batch_get_kernel_launches: NULL argument");
+    *kernels = b->kernels;
     return LBM_OK;
 }
 

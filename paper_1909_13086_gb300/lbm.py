@@ -74,7 +74,8 @@ EXPORTED = ("lbm_create", "lbm_set_params", "lbm_get_derived", "lbm_step", "lbm_
             "lbm_destroy", "lbm_last_error", "lbm_set_allocator", "lbm_version", "lbm_step_static",
             "lbm_batch_create", "lbm_batch_add", "lbm_batch_remove", "lbm_batch_count",
             "lbm_batch_step", "lbm_batch_destroy", "lbm_autotune", "lbm_set_history",
-            "lbm_read_history", "lbm_batch_set_launch", "lbm_batch_set_streaming", "lbm_batch_autotune")
+            "lbm_read_history", "lbm_batch_set_launch", "lbm_batch_set_streaming", "lbm_batch_autotune",
+            "lbm_get_kernel_launches", "lbm_batch_get_kernel_launches")
 
 _lib = None
 _D = ctypes.POINTER(ctypes.c_double)
@@ -99,6 +100,8 @@ def lib() -> ctypes.CDLL:
     L.lbm_set_diag_every.argtypes = [H, ctypes.c_longlong]
     L.lbm_set_launch.argtypes = [H, ctypes.c_int, ctypes.c_int, ctypes.c_int]
     L.lbm_get_launch_stats.argtypes = [H, ctypes.POINTER(lbm_launch_stats)]
+    L.lbm_get_kernel_launches.argtypes = [H, ctypes.POINTER(ctypes.c_longlong)]
+    L.lbm_batch_get_kernel_launches.argtypes = [ctypes.c_void_p, ctypes.POINTER(ctypes.c_longlong)]
     L.lbm_set_staging.argtypes = [H, ctypes.c_int]
     L.lbm_set_streaming.argtypes = [H, ctypes.c_int]
     L.lbm_batch_set_streaming.argtypes = [H, ctypes.c_int]
@@ -207,6 +210,12 @@ def lbm_set_wait_limit(h, tries: int = 1 << 20, force_timeout: bool = False) -> 
     _check(lib().lbm_set_wait_limit(h, int(tries), 1 if force_timeout else 0), h)
 
 
+def lbm_get_kernel_launches(h) -> int:
+    n = ctypes.c_longlong()
+    _check(lib().lbm_get_kernel_launches(h, ctypes.byref(n)), h)
+    return n.value
+
+
 def lbm_get_launch_stats(h) -> dict:
     st = lbm_launch_stats()
     _check(lib().lbm_get_launch_stats(h, ctypes.byref(st)), h)
@@ -296,6 +305,12 @@ def lbm_batch_step(b, n: int) -> None:
 
 def lbm_batch_set_launch(b, rows: int = 0, prefetch: int = -1, interleave: int = 0) -> None:
     _check(lib().lbm_batch_set_launch(b, int(rows), int(prefetch), int(interleave)))
+
+
+def lbm_batch_get_kernel_launches(b) -> int:
+    n = ctypes.c_longlong()
+    _check(lib().lbm_batch_get_kernel_launches(b, ctypes.byref(n)))
+    return n.value
 
 
 def lbm_batch_set_streaming(b, mode: int = LBM_STREAM_AUTO) -> None:

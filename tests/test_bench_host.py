@@ -162,3 +162,10 @@ def test_reference_arm_line(capsys, monkeypatch):
     monkeypatch.setenv("RANK", "1")
     bench.main(["--impl", "reference", "--steps", "1", "--warmup", "3"])
     assert capsys.readouterr().out.strip() == ""
+
+
+def test_batch_line_states_how_the_steps_shared_launches():
+    assert bench.batch_launches(100, 101)[0] == "one fused launch per step"
+    text, streaming = bench.batch_launches(100, 15)
+    assert text == "99 steps in 13 launches and a diagnostic one"
+    assert streaming.startswith("one buffer read and the other written")

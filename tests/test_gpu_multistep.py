@@ -273,3 +273,36 @@ def test_autotuners_time_what_runs(stream):
         us.append(t["us_per_step"])
         b.close()
     assert 0 < 1.5 * us[0] < us[1]
+
+
+@pytest.mark.parametrize("diag_every,per_call", [(0, 4 + 1 + 2), (4, 4 * 2 + 1 + 2), (1, 10 * 2)])
+def test_kernel_launches_are_counted(stream, diag_every, per_call):
+    """A call of 10 steps, launched directly, captured and replayed.  Bands: four
+    pairs, an odd step, a diagnostic sweep and its fold; diagnostics every 4th step: two
+    pieces of a pair, an odd step, a sweep and a fold, then one step and a sweep and a
+    fold; every step: ten sweeps and folds.  Two buffers: a sweep per step, a fold."""
+    p = workloads.params(Ra=1e6, strip_center=0.6)
+    lat, ref = (lbm.Lattice(1025, 513, p, precision="fp32", stream=stream) for _ in range(2))
+    lbm.lbm_set_diag_every(lat.h, diag_every)
+    lbm.lbm_set_streaming(ref.h, lbm.LBM_STREAM_TWO_BUFFERS)
+    for call in range(1, 4):
+        # each call starts at a multiple of diag_every
+        lat.set_populations(*lat.populations()[:2], 0)
+        before = lbm.lbm_get_kernel_launches(lat.h)
+        lat.step(10)
+        assert lbm.lbm_get_kernel_launches(lat.h) - before == per_call
+        ref.step(10)
+        assert lbm.lbm_get_kernel_launches(ref.h) == 11 * call
+
+
+def test_kernel_launches_of_a_batch_are_counted(stream):
+    p = workloads.params(Ra=1e5)
+    for prec, members, want in (("fp32", 60, 4 + 1 + 2), ("fp64", 2, 11)):
+        lats = [lbm.Lattice(128, 128, p, precision=prec, stream=stream) for _ in range(members)]
+        b = lbm.Batch(members, stream)
+        for lat in lats:
+            b.add(lat)
+        for call in range(1, 4):
+            b.step(10)
+            assert lbm.lbm_batch_get_kernel_launches(b.b) == want * call
+        b.close()
