@@ -169,3 +169,13 @@ def test_batch_line_states_how_the_steps_shared_launches():
     text, streaming = bench.batch_launches(100, 15)
     assert text == "99 steps in 13 launches and a diagnostic one"
     assert streaming.startswith("one buffer read and the other written")
+
+
+def test_workload_config_of_the_default_workload():
+    """FP32 at 2048 x 1024 takes two steps per launch from one buffer into the other;
+    16-bit storage runs in one buffer; FP64 over two."""
+    streaming = {p: bench.workload_config(p)["streaming"] for p in ("fp32", "bf16sr", "fp64")}
+    assert streaming["fp32"] == ("one buffer read and the other written per two steps (bands); diagnostic steps are "
+                                 "sweeps")
+    assert streaming["bf16sr"].startswith("one buffer (push / local sweeps)")
+    assert streaming["fp64"] == "two buffers"

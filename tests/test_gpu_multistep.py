@@ -306,3 +306,55 @@ def test_kernel_launches_of_a_batch_are_counted(stream):
             b.step(10)
             assert lbm.lbm_batch_get_kernel_launches(b.b) == want * call
         b.close()
+
+
+@pytest.mark.parametrize("rates", [{}, RATES])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (31, 3), (33, 17), (64, 32), (65, 33), (181, 181), (256, 128)])
+def test_fp64_tiles(stream, rates, nx, ny):
+    """With k0 = k0f = 1 the collision drops the terms in the old populations: both
+    forms, in tiles and in sweeps."""
+    compare(nx, ny, workloads.params(Ra=1e5, strip_center=0.4, **rates), "fp64", stream, (2, 3, 18, 33, 33), 9)
+
+
+@pytest.mark.parametrize("prec,nx,ny", [("fp32", 64, 32), ("fp64", 64, 32), ("bf16", 65, 33), ("fp32", 1025, 513)])
+def test_history_shorter_than_a_launch(stream, prec, nx, ny):
+    """A ring of one or three entries wraps inside a launch of several steps."""
+    for cap in (1, 3):
+        lat, ref = (start(nx, ny, workloads.params(Ra=1e5, strip_center=0.4), prec, stream) for _ in range(2))
+        lbm.lbm_set_streaming(ref.h, lbm.LBM_STREAM_TWO_BUFFERS)
+        for L in (lat, ref):
+            lbm.lbm_set_history(L.h, cap)
+        for n in (2, 19, 19, 20):
+            for L in (lat, ref):
+                L.step(n)
+            assert_same(lat, ref, (prec, cap, n))
+            assert len(lbm.lbm_read_history(lat.h, 256)["step"]) == min(cap, lat.populations()[2])
+
+
+@pytest.mark.parametrize("prec,nx,ny", [("fp32", 64, 32), ("fp64", 64, 32), ("bf16sr", 65, 33), ("fp32", 1025, 513)])
+def test_no_heated_strip(stream, prec, nx, ny):
+    compare(nx, ny, workloads.params(Ra=1e5, strip_width=0.0, **RATES), prec, stream, (2, 3, 18, 18), 9)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("prec,nx,ny", [("fp32", 64, 32), ("fp64", 64, 32), ("fp16", 65, 33), ("bf16sr", 64, 32),
+                                        ("fp32", 1025, 513)])
+def test_non_finite_populations(stream, prec, nx, ny, bad):
+    """A non-finite value spreads through tiles and bands as through sweeps."""
+    lat, ref = (start(nx, ny, workloads.params(Ra=1e5), prec, stream) for _ in range(2))
+    lbm.lbm_set_streaming(ref.h, lbm.LBM_STREAM_TWO_BUFFERS)
+    f, g, _ = lat.populations()
+    f[3, ny // 2, nx // 2] = bad
+    g[5, 1, 2] = bad
+    for L in (lat, ref):
+        L.set_populations(f, g, 0)
+        L.step(7)
+    for x, y in zip(lat.populations(), ref.populations()):
+        assert np.array_equal(x, y, equal_nan=True)
+    assert lat.diagnostics(raise_on_diverged=False)["nan_flag"] == ref.diagnostics(raise_on_diverged=False)["nan_flag"] == 1
+
+
+@pytest.mark.parametrize("prec", ["fp16", "fp16sr", "bf16"])
+@pytest.mark.parametrize("copies", [1, 14])
+def test_batches_of_other_16_bit_types(stream, prec, copies):
+    test_batches(stream, prec, copies)

@@ -212,3 +212,59 @@ def test_pair_offsets(nx, ny, paired):
                     assert want not in stored
                     stored[want] = 1
             assert loads[0] == stores[0] and loads[1] == stores[1]
+
+
+@pytest.mark.parametrize("paired", [False, True])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (3, 3), (5, 4), (64, 3), (65, 3), (126, 3), (127, 4), (128, 3), (129, 4),
+                                   (130, 3), (191, 3), (255, 3), (256, 4), (257, 3), (300, 3)])
+def test_pair_offsets_by_path(nx, ny, paired):
+    """The pull and the push of a pair as the kernels take them: one path with the wall
+    rules for every lane of a warp that touches a side wall and for the bottom and top
+    rows, fixed offsets for the others.  A missing second cell loads its own row's padding
+    and stores nothing."""
+    cs = 2 if paired else 1
+    tile = ny * RS
+    slot = [(2 * i if paired else i) * TW for i in range(9)]
+    pairs = range(0, -(-nx // TW) * TW, 2)  # all lanes of the tiles' warps
+    touches = {x: x == 0 or x + 1 >= nx - 1 for x in pairs}
+    for x in range(0, nx, 2):
+        warp = range(x // 64 * 64, x // 64 * 64 + 64, 2)
+        side = any(touches[w] for w in warp)
+        lx = x % TW
+        dL = cs * (TW - 1) - tile if lx == 0 and x > 0 else -cs
+        dR = tile - cs * (TW - 2) if lx == TW - 2 and x + 2 < nx else 2 * cs
+        left, right0, right1, has1 = x == 0, x == nx - 1, x + 1 >= nx - 1, x + 1 < nx
+        for y in range(ny):
+            bottom, top = y == 0, y == ny - 1
+            p = place(x, y, 0, ny, paired)
+
+            def wall0(i):
+                cx, cy = C[i]
+                return (cx > 0 and left) or (cx < 0 and right0) or (cy > 0 and bottom) or (cy < 0 and top)
+
+            def wall1(i):
+                cx, cy = C[i]
+                return not has1 or (cx < 0 and right1) or (cy > 0 and bottom) or (cy < 0 and top)
+
+            for i, (cx, cy) in enumerate(C):
+                o = OPP[i]
+                into, own = slot[i] - cy * RS, slot[o]
+                out, mine = slot[o] + cy * RS, slot[i]
+                if side or bottom or top:
+                    pull = (own if wall0(i) else into + (dL if cx > 0 else cs if cx < 0 else 0),
+                            own + cs if wall1(i) else into + (0 if cx > 0 else dR if cx < 0 else cs))
+                    push = (mine if wall0(o) else out + (cs if cx > 0 else dL if cx < 0 else 0),
+                            mine + cs if wall1(o) else out + (dR if cx > 0 else 0 if cx < 0 else cs))
+                elif cx == 0:
+                    pull, push = (into, into + cs), (out, out + cs)
+                else:
+                    pull = (into + (dL if cx > 0 else cs), into + (0 if cx > 0 else dR))
+                    push = (out + (cs if cx > 0 else dL), out + (dR if cx > 0 else 0))
+                for c in (0, 1):
+                    if c and not has1:
+                        assert p + pull[1] == place(x + 1, y, o, ny, paired)
+                        continue
+                    for at, sx, sy, there, here in ((pull[c], x + c - cx, y - cy, i, o), (push[c], x + c + cx, y + cy, o, i)):
+                        inside = 0 <= sx < nx and 0 <= sy < ny
+                        want = place(sx, sy, there, ny, paired) if inside else place(x + c, y, here, ny, paired)
+                        assert p + at == want, (nx, ny, x + c, y, i)
