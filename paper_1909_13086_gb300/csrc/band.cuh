@@ -17,8 +17,8 @@
 // thread keeps its columns' directions 0, 2 and 4 in registers.  Step 1 is
 // computed on a pair of columns and a row more than the core on every side that is
 // not a wall, by the same operations as in the neighbouring block, so the bits are
-// those of two sweeps.  The bands of one launch run at the same time, one wave of
-// blocks; successive launches march them in opposite directions, so that each
+// those of two sweeps.  The bands of one lattice run at the same time, one wave of
+// blocks (of a large batch in several); successive launches march them in opposite directions, so that each
 // starts on the rows the previous one wrote last.
 //
 // 2048 x 1024 FP32 on GB300: 36.7 us per step with one-buffer sweeps, 26.3 here: 137

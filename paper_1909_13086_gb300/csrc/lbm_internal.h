@@ -39,7 +39,8 @@ enum Streaming { kPull = 0, kAAPush = 1, kAALocal = 2, kPullNarrow = 3, kAAPushN
 //     index(x, y, p) = ((x / kTW) * ny + y) * 18 * kTW + p * kTW + x % kTW.
 // A warp's 18 loads of one cell row are then one base register plus
 // compile-time offsets (plane p: p*kTW; row above / below: -/+ 18*kTW).
-constexpr int kTW = 128;  // tile width = threads per block (fastest of 128/256/512 on GB300)
+constexpr int kTW = 128;  // tile width (fastest of 128/256/512 on GB300); a sweep's block has kTW
+                          // threads, or kTW / 2 with two cells each
 constexpr int kPlanes = 18;
 constexpr int kRS = kPlanes * kTW;  // elements per tile row
 

@@ -2,7 +2,8 @@
 //
 // Layout: tile-major structure of arrays (lbm_internal.h).  One thread per
 // lattice column of a kTW-wide tile (two neighbouring columns in the cavity
-// sweeps with flow in FP32 arithmetic, sweep_block_two), walking `rows` rows; a
+// sweeps with flow in FP32 arithmetic, sweep_block_two, but for narrow lattices,
+// launch_sweep), walking `rows` rows; a
 // warp covers 32 (64) consecutive cells of one row, so every load and store is a coalesced 128 B
 // line (FP32).  In the interior the 18 pull loads of a cell are one base
 // register plus compile-time offsets; boundary rows and the two warps of a

@@ -22,7 +22,8 @@
 // and 1.6, BF16-SR 7.8 and 1.8, 512 x 512 FP32 7.1 and 4.6, 1024 x 4 Stefan FP64 8.6 and
 // 2.9.  Bound by latency: 4.2 us a launch, then per step one cell's chain and the
 // barrier (256 x 128: 43 % issue active).  Two cells per thread, as in the sweeps, has
-// half the warps and is slower (512 x 512 5.4).
+// half the warps and is slower (512 x 512 5.4).  FP64 is bound by its pipe: an SM holds
+// its share of the tiles and no more (tile_args).
 #pragma once
 
 #include "sweep.cuh"

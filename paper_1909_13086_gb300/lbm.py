@@ -394,7 +394,7 @@ class Lattice:
         return lbm_diagnostics(self.h, raise_on_diverged)
 
     def fields(self, names=FIELD_NAMES) -> dict:
-        # side by side in the library's order: read back in one copy
+        # side by side in the library's order: read back in one copy (views of one block)
         order = [k for k in FIELD_NAMES if k in names]
         out = dict(zip(order, np.empty((len(order), self.ny, self.nx))))
         mask = 0
