@@ -1730,11 +1730,13 @@ __host__ __device__ constexpr int sweep_threads() {
 // FP16-SR 21.7 / 21.6 / 21.1, 1001 x 701 BF16-SR 9.1 / 9.1 / 8.8; 32 x 256 x 128
 // batches FP32 18.2 / 17.7 / -, BF16-SR 15.0 / 14.7 / 15.7.  The FP32 batch's diagnostic
 // sweep spills at 10 (calls of one step, 10 / 8: 32 x 256 x 128 32.5 / 30.9, 8 x 1024 x 512
-// 99.2 / 98.5).
+// 99.2 / 98.5).  16-bit storage rounded to nearest spills at 12 (one buffer, 12 / 11 / 10:
+// 2048 x 1024 FP16 21.2 / 19.9 / 20.5, BF16 19.7 / 19.3 / 20.3, 161 x 6500 FP16 19.0 / 18.3 /
+// 18.7).
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM, bool BATCH>
 __host__ __device__ constexpr int sweep_blocks() {
     if (takes_two<real, PROB, FLOW, MODE, SM>())
-        return Store<S>::kDev ? (BATCH ? 10 : 12) : (BATCH && MODE == kSweepDiag ? 8 : 10);
+        return Store<S>::kDev ? (BATCH ? 10 : (Store<S>::kSR ? 12 : 11)) : (BATCH && MODE == kSweepDiag ? 8 : 10);
     return sizeof(real) == 4 ? 1024 / kTW : 1;
 }
 
