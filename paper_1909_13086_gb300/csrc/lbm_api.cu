@@ -385,14 +385,12 @@ BandPlan band_plan(lbm_s *const *lats, size_t n) {
     if (n == 1 && 2 * strips > room && tallest > 4 && tallest <= 16 && (long long)lats[0]->nx * tallest <= 1 << 20)
         return BandPlan();
     const int highest = strips > room ? std::min(tallest, 64) : tallest;  // one wave may not be had
-    std::vector<int> each(n);
-    for (size_t r = 0; r < n; ++r) each[r] = band_strips(lats[r], plan.threads);
     long long least = 1ll << 62;
     for (int rows = std::min(4, highest); rows <= highest; ++rows) {
         long long blocks = 0, longest = 0;
         for (size_t r = 0; r < n; ++r) {
             const int bands = (lats[r]->ny + rows - 1) / rows;
-            blocks += (long long)each[r] * bands;
+            blocks += (long long)band_strips(lats[r], plan.threads) * bands;
             longest = std::max(longest, (long long)(lats[r]->ny + bands - 1) / bands);
         }
         const long long cost = (blocks + room - 1) / room * (longest + 2);
