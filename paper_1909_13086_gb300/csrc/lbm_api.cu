@@ -259,8 +259,8 @@ size_t tile_smem(const lbm_s *h, int w, int hh, int T) {
 // tiles: 256 x 128 FP32 5.4 and 1.7 us, 512 x 512 7.1 and 4.5, 1024 x 512 9.0 and
 // 8.3; 256 x 128 BF16-SR 7.8 and 1.9), above which the sweep's larger launches
 // have paid for themselves.  FP64: its pipe binds all but the launches, so up to 2^15
-// cells with flow (sweep and tiles: 64 x 32 9.4 and 7.1, 256 x 128 20.2 and 14.0) and
-// 2^14 without (1024 x 4 Stefan: 8.6 and 2.9).
+// cells with flow (sweep and tiles: 64 x 32 9.5 and 7.1, 128 x 128 10.5 and 8.8, 256 x 128
+// 14.2 and 14.0) and 2^14 without (1024 x 4 Stefan: 7.8 and 2.9).
 // A batch, of one member too, has the kernel for cavities with flow in FP32
 // arithmetic only (launch_batch_tile).
 TilePlan tile_plan(lbm_s *const *lats, size_t n, bool batch) {
@@ -327,16 +327,11 @@ TileArgs tile_args(const lbm_s *h, const TilePlan &plan, int T, int cells) {
     tl.threads = std::min(most, ((cells + rounds - 1) / rounds + 31) / 32 * 32);
     tl.q_offset = (unsigned)tile_q_offset(h, tl.W, tl.H, T);
     tl.smem = (unsigned)tile_smem(h, tl.W, tl.H, T);
-    // FP64: two blocks on one SM take twice as long, and with programmatic launches
-    // a launch's blocks find the previous ones still resident and gather on what is
-    // free.  Each block asks for so much shared memory that an SM holds its even
-    // share of the tiles and no more (us per step, 100-step calls, without and with:
-    // 64 x 32 8.5 and 7.1, 128 x 64 13.1 and 7.3, 181 x 181 23.4 and 14.7, 256 x 128
-    // 27.8 and 14.0; sweeps 9.4, 13.3, 19.8, 20.2).  FP32 is bound by latency and
-    // shares SMs well.
-    const int share = (tl.tiles_x * tl.tiles_y + h->num_sms - 1) / h->num_sms;
-    if (h->precision == LBM_FP64 && share < 8)
-        tl.smem = std::max(tl.smem, (unsigned)(kTileSmemMax / (share + 1) + 1024) / 16 * 16);
+    // FP64 (us per step, 100-step calls, without share_smem and with: 64 x 32 8.5 and 7.1,
+    // 128 x 64 13.1 and 7.3, 181 x 181 23.4 and 14.7, 256 x 128 27.8 and 14.0; sweeps
+    // with it 9.5, 10.5, 16.0, 14.2).  FP32 is bound by latency and shares SMs well.
+    if (h->precision == LBM_FP64)
+        tl.smem = std::max(tl.smem, share_smem((long long)tl.tiles_x * tl.tiles_y, h->num_sms));
     tl.qgroup = h->qgroup;
     return tl;
 }
@@ -464,6 +459,7 @@ SweepArgs<real> make_args(const lbm_s *h, const void *src, void *dst) {
     a.a0f = real(1) - a.k0f;
     a.s1 = std::fma(real(-0.5), a.k1f, real(1));
     a.s2 = std::fma(real(-0.5), a.k2f, real(1));
+    a.sms = h->num_sms;
     a.unit = a.a0 == real(0) && (!h->p.flow_on || a.a0f == real(0));
     a.strip_on = h->strip_on;
     a.lo2 = h->lo2;

@@ -120,6 +120,7 @@ struct alignas(16) SweepArgs {
     long long wait_limit;
     // field outputs (kFields), nx*ny doubles each, row-major; NULL = skip
     double *oH, *oT, *oFL, *oUX, *oUY, *oRHO;
+    int sms;  // SMs of the device (share_smem; the host's)
 };
 
 // Several steps of a small lattice in one launch (tile.cuh): T steps by blocks
@@ -129,6 +130,14 @@ constexpr int kTileThreads64 = 256;   // FP64 (its pipe is busy with four warps;
 constexpr int kTileMaxSteps = 16;
 constexpr int kTileMaxNx = 4096;      // the inflow's fold: 32 lanes x 128 columns
 constexpr size_t kTileSmemMax = 230400;
+// Dynamic shared memory with which an SM holds its even share of a launch's blocks and
+// no more; 0 from eight blocks an SM on.  For FP64: two blocks on one SM take twice as long,
+// and with programmatic launches a launch's blocks find the previous ones still resident
+// and gather on what is free.
+inline unsigned share_smem(long long blocks, int sms) {
+    const long long share = (blocks + sms - 1) / sms;
+    return share < 8 ? (unsigned)(kTileSmemMax / (share + 1) + 1024) / 16 * 16 : 0u;
+}
 struct TileArgs {
     int T;                 // steps of this launch, 1 .. kTileMaxSteps
     int W, H;              // core of a block; W a multiple of 32 in the cavity

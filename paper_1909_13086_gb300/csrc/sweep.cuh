@@ -2256,12 +2256,12 @@ __global__ void repack_kernel(void *bufv, void *buf2v, double *stage, int nx, in
 // ---- launch dispatch (instantiated per storage type in sweep_*.cu) ----
 // A launch, with the programmatic-serialization attribute when pdl is set.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
-                            bool pdl, Args &&...args) {
+static cudaError_t launch_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned smem, cudaStream_t s,
+                               bool pdl, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2269,6 +2269,12 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
+                            bool pdl, Args &&...args) {
+    return launch_smem(kernel, grid, block, 0u, s, pdl, std::forward<Args>(args)...);
 }
 
 // A sweep, by one cell per thread although two would do:
@@ -2289,8 +2295,21 @@ static cudaError_t launch_sweep(const SweepArgs<real> &a, dim3 grid, cudaStream_
                 return launch_k(lattice_kernel<real, S, PROB, FLOW, MODE, SM + kPullNarrow>, grid, dim3(kTW), s, pdl, a);
         }
     }
-    return launch_k(lattice_kernel<real, S, PROB, FLOW, MODE, SM>, grid, dim3(sweep_threads<real, PROB, FLOW, MODE, SM>()),
-                    s, pdl, a);
+    auto *kernel = lattice_kernel<real, S, PROB, FLOW, MODE, SM>;
+    unsigned smem = 0;
+    if constexpr (sizeof(real) == 8) {
+        // us per step without share_smem and with: 128 x 128 with flow 18.8 and 10.5, without
+        // 11.7 and 7.9, 256 x 128 20.2 and 14.2, 333 x 111 20.1 and 17.3, 512 x 128 without flow
+        // 14.5 and 12.4; 64 x 32, whose 32 blocks rarely meet, 9.35 and 9.67
+        const long long blocks = (long long)grid.x * grid.y;
+        smem = blocks > a.sms / 4 ? share_smem(blocks, a.sms) : 0u;
+        if (smem) {
+            // per device and idempotent; no state is kept here
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemMax);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    return launch_smem(kernel, grid, dim3(sweep_threads<real, PROB, FLOW, MODE, SM>()), smem, s, pdl, a);
 }
 
 template <typename real, typename S, int PROB, bool FLOW>
