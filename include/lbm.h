@@ -328,7 +328,9 @@ int lbm_write_populations(lbm_handle h, const double *f, const double *g, long l
  *
  * Members keep their own memory and state; lbm_diagnostics, lbm_read_fields
  * and friends keep working on them between batch steps.  Every member must
- * share the device, precision, problem kind and flow_on of the first one; the
+ * share the device, precision, problem kind and flow_on of the first one (a member given
+ * others by lbm_set_params is an LBM_ERR_STATE of lbm_batch_step; other parameters and
+ * lbm_set_history take effect at the next one); the
  * last step of each lbm_batch_step is a diagnostic step for every member (their
  * diag_every setting does not apply inside a batch).  The batch orders its
  * work after what is queued on the members' streams and their streams after

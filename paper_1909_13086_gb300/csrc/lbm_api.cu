@@ -90,6 +90,8 @@ struct lbm_s {
     unsigned long long graph_clock = 0;
     lbm_launch_stats stats{};   // sweeps launched directly / replayed, graphs captured
     long long kernels = 0;  // launched by lbm_step (lbm_get_kernel_launches)
+    unsigned long long generation = 0;  // of what a batch's table holds of the handle: its
+                                        // parameters and the history's address
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     void *buf[2] = {nullptr, nullptr};  // 18 planes each
@@ -949,6 +951,7 @@ int lbm_set_params(lbm_handle h, const lbm_params *p) {
     int rc = derive(h, p, &d);
     if (rc != LBM_OK) return rc;
     drop_graphs(h);
+    h->generation += 1;
     h->p = *p;
     h->d = d;
     if (p->problem == LBM_CAVITY && p->strip_width > 0.0) {
@@ -1168,6 +1171,7 @@ int lbm_set_history(lbm_handle h, long long capacity) {
     DeviceGuard g(h->device);
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     drop_graphs(h);
+    h->generation += 1;
     dev_free(h, h->hist);
     h->hist = nullptr;
     h->hist_cap = 0;
@@ -1364,6 +1368,7 @@ struct lbm_batch_s {
     std::vector<unsigned char> host_entries;
     std::vector<int> host_starts;
     std::vector<int> host_parity;
+    std::vector<unsigned long long> host_generation;  // the members' when the table was built
     int nblocks = 0;
     TilePlan tile;            // several steps per launch, unless lbm_batch_set_streaming
     BandPlan band;            // asked for sweeps
@@ -1453,6 +1458,8 @@ void batch_build(lbm_batch_s *b) {
     const size_t eb = entry_bytes<real>();
     b->host_entries.assign(eb * b->members.size(), 0);
     b->host_starts.assign(b->members.size(), 0);
+    b->host_generation.resize(b->members.size());
+    for (size_t r = 0; r < b->members.size(); ++r) b->host_generation[r] = b->members[r]->generation;
     b->uniform = 0;
     int start = 0, mstart = 0;
     // several steps per launch: tiles while the members are few and small, else bands;
@@ -1546,7 +1553,12 @@ int batch_multi(lbm_batch_s *b, long long len, bool diag, int j) {
 template <typename real, typename S>
 int batch_steps(lbm_batch_s *b, long long n) {
     const int nm = (int)b->members.size();
+    // a member whose parameters or history were set since the table was built
+    for (int r = 0; r < nm && !b->dirty; ++r) b->dirty = b->members[r]->generation != b->host_generation[r];
     if (b->dirty) {
+        for (const lbm_s *h : b->members)
+            if (h->p.problem != b->problem || (h->p.flow_on != 0) != (b->flow != 0))
+                return batch_err(LBM_ERR_STATE, "lbm_batch_step: a member's problem or flow_on is no longer the batch's");
         batch_build<real>(b);
         BATCH_TRY(cudaMemcpyAsync(b->entries, b->host_entries.data(), b->host_entries.size(),
                                   cudaMemcpyHostToDevice, b->stream));

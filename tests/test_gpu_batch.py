@@ -289,3 +289,45 @@ def test_batch_row_bands_in_both_directions_match_oracle(orc, stream, rows):
             assert err <= 1e-12, (ny, rows, name, err)
         assert lat.diagnostics()["Q_cum"] == pytest.approx(ref.diagnostics()["Q_cum"], rel=1e-12, abs=1e-15)
     b.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16sr", "fp64"])
+@pytest.mark.parametrize("n", [1, 3])
+def test_members_set_anew_between_steps(stream, prec, n):
+    """A member's history taken, resized and freed, and its parameters set, between batch
+    steps: the table follows, and the member ends where it ends alone."""
+    cases = CASES[:n]
+    members, solo = ([make(stream, prec, nx, ny, kw) for nx, ny, kw in cases] for _ in range(2))
+    b = lbm.Batch(4, stream)
+    for lat in members:
+        b.add(lat)
+
+    def step(k):
+        b.step(k)
+        for lat in solo:
+            lat.step(k)
+
+    def same():
+        for s, m in zip(solo, members):
+            for x, y in zip(s.populations(), m.populations()):
+                assert np.array_equal(x, y)
+
+    step(30)
+    for cap in (64, 8, 0, 16):
+        for lat in (members[0], solo[0]):
+            lbm.lbm_set_history(lat.h, cap)
+        step(30)
+        h, hs = (lbm.lbm_read_history(lat.h, 100) for lat in (members[0], solo[0]))
+        assert len(h["step"]) == min(cap, 30)
+        assert np.array_equal(h["step"], hs["step"]) and h["Q"] == pytest.approx(hs["Q"], rel=1e-12)
+    same()
+    nx, ny, kw = cases[0]
+    for lat in (members[0], solo[0]):
+        lbm.lbm_set_params(lat.h, workloads.params(**{**kw, "Ra": 1e5, "strip_center": 0.7, "Ste": 0.5}))
+    step(31)
+    same()
+    lbm.lbm_set_params(members[0].h, workloads.params(**{**kw, "flow_on": 0}))
+    with pytest.raises(lbm.LbmError) as e:
+        b.step(1)
+    assert e.value.status == lbm.LBM_ERR_STATE
+    b.close()
