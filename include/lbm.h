@@ -362,10 +362,8 @@ int lbm_batch_step(lbm_batch b, long long n);
 int lbm_batch_get_kernel_launches(lbm_batch b, long long *kernels);
 
 /* Launch shape of the batch's step kernel: rows of a member walked by each
- * block (0 = the default: 2; with 16-bit storage 3 for cavities with flow, else 4;
- * up to 1024), the L2 prefetch distance in rows (-1 = the default: 4, but for
- * cavities with flow other than LBM_FP64 0 unless the storage is 16-bit and the
- * members' populations exceed 64 MB),
+ * block (0 = the default: 2 to 4, by storage, problem and the members' size together;
+ * up to 1024), the L2 prefetch distance in rows (-1 = the default: 0 or 4, likewise),
  * and interleave = 1 (the default) to number the blocks of a one-size batch
  * member after member (block b belongs to member b mod n) instead of member
  * by member (0; a batch whose members' block counts differ is always member

@@ -333,7 +333,7 @@ TileArgs tile_args(const lbm_s *h, const TilePlan &plan, int T, int cells) {
     // 128 x 64 13.1 and 7.3, 181 x 181 23.4 and 14.7, 256 x 128 27.8 and 14.0; sweeps
     // with it 9.5, 10.5, 16.0, 14.2).  FP32 is bound by latency and shares SMs well.
     if (h->precision == LBM_FP64)
-        tl.smem = std::max(tl.smem, share_smem((long long)tl.tiles_x * tl.tiles_y, h->num_sms));
+        tl.smem = std::max(tl.smem, share_smem((long long)tl.tiles_x * tl.tiles_y, h->num_sms, 7));
     tl.qgroup = h->qgroup;
     return tl;
 }
@@ -1439,18 +1439,30 @@ bool batch_several(const lbm_batch_s *b) { return !batch_sweeps_chosen(b) && (b-
 //   and 14.9), but 4 rows ahead for 16-bit members of more than 64 MB together (one buffer
 //   each; BF16-SR, prefetch 0 / 4: 48 x 256 x 128, 57 MB, 20.8 / 20.9; 96 40.9 / 39.7; 32
 //   x 512 x 256 53.1 / 49.9; a call of one step, 64 x 256 x 128, 75 MB, 42.1 / 40.6).
-// - One cell per thread: 2 rows, 4 with 16-bit storage, 4 rows ahead (32 x 512 x 256
-//   periodic with flow, at prefetch 0 and 4: FP32 102.1 and 95.3; FP16, 3 rows and none
-//   ahead against 4 and 4: 70.6 and 67.2).
+// - One cell per thread, us per step (of a one-step call): FP32 2 rows and none ahead (16 x
+//   256 x 128 without flow, prefetch 0 / 4 7.8 / 8.0), but beyond 64 MB 3 rows (8 x 1024 x
+//   512 without flow, rows and prefetch 2, 0 / 2, 4 / 3, 0: 46.6 / 55.4 / 44.1; 64 x 256 x 128
+//   periodic 41.0 (59.4) / 41.9 (56.4) / 38.1 (55.3)), or with flow 2 rows, 4 ahead (8 x 1024
+//   x 512 2, 0 / 2, 4: 99.4 / 91.7).  16-bit storage: 3 rows and none ahead, 4 rows from 16
+//   MB (without flow in a cavity 32), 4 ahead beyond 64 MB (3, 0 / 4, 0 / 4, 4: BF16-SR 4 x 256
+//   x 128 periodic with flow 12.2 / 14.7 / 14.7, 16 x 18.9 / 16.9 / 17.0, 8 x 1024 x 512 71.2 /
+//   68.9 / 65.2).  FP64: 2 rows, 4 ahead.
 struct BatchShape {
     int rows, prefetch;
 };
 BatchShape batch_shape(const lbm_batch_s *b) {
     const bool half = b->precision != LBM_FP32 && b->precision != LBM_FP64;
-    if (b->problem != LBM_CAVITY || !b->flow || b->precision == LBM_FP64) return {half ? 4 : 2, 4};
+    const bool cavity = b->problem == LBM_CAVITY, flow = b->flow != 0;
+    if (b->precision == LBM_FP64) return {2, 4};
     size_t total = 0;
     for (const lbm_s *h : b->members) total += buffer_bytes(h);
-    return {half ? 3 : 2, half && total > (64u << 20) ? 4 : 0};
+    const size_t mb = total >> 20;
+    if (!cavity || !flow) {
+        if (half) return {mb >= (cavity ? 32u : 16u) ? 4 : 3, mb >= 64 ? 4 : 0};
+        if (mb < 64) return {2, 0};
+        return flow ? BatchShape{2, 4} : BatchShape{3, 0};
+    }
+    return {half ? 3 : 2, half && mb >= 64 ? 4 : 0};
 }
 
 template <typename real>

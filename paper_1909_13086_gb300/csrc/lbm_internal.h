@@ -131,12 +131,12 @@ constexpr int kTileMaxSteps = 16;
 constexpr int kTileMaxNx = 4096;      // the inflow's fold: 32 lanes x 128 columns
 constexpr size_t kTileSmemMax = 230400;
 // Dynamic shared memory with which an SM holds its even share of a launch's blocks and
-// no more; 0 from eight blocks an SM on.  For FP64: two blocks on one SM take twice as long,
-// and with programmatic launches a launch's blocks find the previous ones still resident
-// and gather on what is free.
-inline unsigned share_smem(long long blocks, int sms) {
+// no more; 0 where that is more than `most` (7 at most).  For FP64: two blocks on one SM
+// take twice as long, and with programmatic launches a launch's blocks find the previous
+// ones still resident and gather on what is free.
+inline unsigned share_smem(long long blocks, int sms, int most) {
     const long long share = (blocks + sms - 1) / sms;
-    return share < 8 ? (unsigned)(kTileSmemMax / (share + 1) + 1024) / 16 * 16 : 0u;
+    return share <= most ? (unsigned)(kTileSmemMax / (share + 1) + 1024) / 16 * 16 : 0u;
 }
 struct TileArgs {
     int T;                 // steps of this launch, 1 .. kTileMaxSteps

@@ -2280,14 +2280,18 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
 // A sweep, by one cell per thread although two would do:
 // - where pairs leave half of the threads of all blocks idle, or three in four of every
 //   second block's (us per step, two cells and one: 16 x 65535 BF16-SR 84.8 and 51.2, 64 x
-//   16384 FP16 22.8 and 16.3, 160 x 6500 18.8 and 14.2, FP32 in one buffer 21.4 and 18.9).
-//   FP32 over two buffers and the diagnostic sweeps gain nothing by it;
+//   16384 FP16 22.8 and 16.3, 160 x 6500 18.8 and 14.2, FP32 in one buffer 21.4 and 18.9),
+//   in lattices of enough rows of tiles to keep the SMs busy (two cells and one: 129 x
+//   2000 BF16-SR 7.6 and 7.8, 129 x 4000 11.9 and 10.6; 64 x 2000 FP32 6.1 and 6.3, 64 x 4000
+//   7.3 and 6.8).  FP32 over two buffers and the diagnostic sweeps gain nothing by it;
 // - on a caller's FP32 buffers off 8-byte boundaries (lbm_step_static).
 template <typename real, typename S, int PROB, bool FLOW, int MODE, int SM>
 static cudaError_t launch_sweep(const SweepArgs<real> &a, dim3 grid, cudaStream_t s, bool pdl) {
     if constexpr (takes_two<real, PROB, FLOW, MODE, SM>()) {
         bool one = false;
-        if constexpr (MODE == kSweep) one = a.nx <= kTW / 2 || (a.nx > kTW && a.nx <= kTW + kTW / 4);
+        if constexpr (MODE == kSweep)
+            one = (a.nx <= kTW / 2 || (a.nx > kTW && a.nx <= kTW + kTW / 4)) &&
+                  (a.nx > kTW ? 2 : 1) * a.ny > (Store<S>::kDev ? 6000 : 3500);
         else one = (reinterpret_cast<uintptr_t>(a.src) | reinterpret_cast<uintptr_t>(a.dst)) % 8 != 0;
         // FP32: kPull of kSweepDiag, the others of kSweep; 16-bit: all of kSweep
         if constexpr (Store<S>::kDev ? MODE == kSweep : (MODE == kSweep) == (SM != kPull)) {
@@ -2300,9 +2304,11 @@ static cudaError_t launch_sweep(const SweepArgs<real> &a, dim3 grid, cudaStream_
     if constexpr (sizeof(real) == 8) {
         // us per step without share_smem and with: 128 x 128 with flow 18.8 and 10.5, without
         // 11.7 and 7.9, 256 x 128 20.2 and 14.2, 333 x 111 20.1 and 17.3, 512 x 128 without flow
-        // 14.5 and 12.4; 64 x 32, whose 32 blocks rarely meet, 9.35 and 9.67
+        // 14.5 and 12.4; 64 x 32, whose 32 blocks rarely meet, 9.35 and 9.67.  With flow
+        // registers leave room for three blocks, and shared memory for more only takes L1:
+        // 33 x 1000, seven blocks an SM, 18.1 and 20.6
         const long long blocks = (long long)grid.x * grid.y;
-        smem = blocks > a.sms / 4 ? share_smem(blocks, a.sms) : 0u;
+        smem = blocks > a.sms / 4 ? share_smem(blocks, a.sms, FLOW ? 3 : 7) : 0u;
         if (smem) {
             // per device and idempotent; no state is kept here
             const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemMax);

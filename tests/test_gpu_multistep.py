@@ -358,3 +358,19 @@ def test_non_finite_populations(stream, prec, nx, ny, bad):
 @pytest.mark.parametrize("copies", [1, 14])
 def test_batches_of_other_16_bit_types(stream, prec, copies):
     test_batches(stream, prec, copies)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16", "bf16", "fp16sr", "bf16sr"])
+@pytest.mark.parametrize("nx,ny", [(33, 6101), (129, 3101)])
+def test_tall_narrow_lattices_by_every_path(stream, prec, nx, ny):
+    """Enough rows for the plain sweeps to take one cell per thread."""
+    p = workloads.params(Ra=1e5, strip_center=0.4, strip_width=0.5, **RATES)
+    lats = [start(nx, ny, p, prec, stream) for _ in range(3)]
+    lbm.lbm_set_streaming(lats[1].h, lbm.LBM_STREAM_ONE_BUFFER)
+    lbm.lbm_set_streaming(lats[2].h, lbm.LBM_STREAM_TWO_BUFFERS)
+    for lat in lats:
+        lbm.lbm_set_diag_every(lat.h, 5)
+        for n in (2, 7, 12):
+            lat.step(n)
+    assert_same(lats[0], lats[2], (prec, nx))
+    assert_same(lats[1], lats[2], (prec, nx))

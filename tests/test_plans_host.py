@@ -109,12 +109,15 @@ def test_16_bit_storage_beyond_l2_prefetches(plans, prec, size, n, solo_pf, batc
         assert solo["prefetch16"] == solo_pf
 
 
-@pytest.mark.parametrize("prec,problem,flow,rows,prefetch", [
-    ("fp32", workloads.CAVITY, 1, 2, 0), ("bf16sr", workloads.CAVITY, 1, 3, 0), ("fp32", workloads.STEFAN, 1, 2, 4),
-    ("fp16", workloads.STEFAN, 0, 4, 4), ("bf16", workloads.CAVITY, 0, 4, 4), ("fp32", workloads.CAVITY, 0, 2, 4)])
-def test_batch_shapes(plans, prec, problem, flow, rows, prefetch):
-    """Members stepped one cell per thread keep their own shape."""
-    solo = plans(prec, problem, flow, [(256, 128)] * 32)[1]
+@pytest.mark.parametrize("prec,problem,flow,n,rows,prefetch", [
+    ("fp32", workloads.CAVITY, 1, 32, 2, 0), ("bf16sr", workloads.CAVITY, 1, 32, 3, 0), ("bf16sr", workloads.CAVITY, 1, 64, 3, 4),
+    ("fp32", workloads.STEFAN, 0, 16, 2, 0), ("fp32", workloads.STEFAN, 0, 32, 3, 0), ("fp32", workloads.CAVITY, 0, 64, 3, 0),
+    ("fp32", workloads.STEFAN, 1, 16, 2, 0), ("fp32", workloads.STEFAN, 1, 32, 2, 4),
+    ("fp16", workloads.STEFAN, 0, 4, 3, 0), ("fp16", workloads.STEFAN, 1, 16, 4, 0), ("bf16", workloads.CAVITY, 0, 16, 3, 0),
+    ("bf16", workloads.CAVITY, 0, 32, 4, 0), ("bf16", workloads.CAVITY, 0, 64, 4, 4)])
+def test_batch_shapes(plans, prec, problem, flow, n, rows, prefetch):
+    """Rows per block and prefetch distance by storage, problem and total size."""
+    solo = plans(prec, problem, flow, [(256, 128)] * n)[1]
     assert (solo["batch_rows"], solo["batch_prefetch"]) == (rows, prefetch)
 
 
